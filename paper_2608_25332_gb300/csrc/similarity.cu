@@ -587,10 +587,12 @@ __global__ void __launch_bounds__(256) merge_argmax_kernel(const SimArgs a, cons
 }
 
 // assign[b][j]: own position for kept rows, best over splits for the others
+// (and clears *n_long, the counter of the sort that follows, when given)
 __global__ void merge_assign_kernel(const SimArgs a, const int* kpos, int n_split,
-                                    const float* ws_best, const int* ws_bidx, int* assign) {
+                                    const float* ws_best, const int* ws_bidx, int* assign, int* n_long) {
   pdl_wait_prior();  // the partials come from the Gram before
   pdl_allow_next();
+  if (n_long != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *n_long = 0;
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (size_t)a.B * a.N_v) return;
   const int kp = kpos[i];
@@ -614,36 +616,54 @@ __global__ void merge_assign_kernel(const SimArgs a, const int* kpos, int n_spli
 
 // merged[b][a] = (sum of rows j with assign[b][j] == a, ascending j) / count.
 // The member lists come from a counting sort per sample: counts (atomics),
-// exclusive offsets, unordered fill. One CTA per kept row orders its members
-// by rank (ascending row index, so the sum order is fixed), fetches the member
-// rows with bulk copies (cp.async.bulk, one thread issuing) into a ring of
-// shared-memory row slots, SLOTS rows per batch, and sums them slot by slot in
-// rank order, each thread over its 16-byte pieces of the row. A centroid with
-// more members than the sort buffer takes them from a scan of assign in
-// windows (ascending by construction). Each CTA is a short chain of dependent
-// steps, so the configuration is chosen for CTAs resident per SM: rows of at
-// most 8 KiB take 128 threads with 4 pieces each (8 CTAs per SM), longer rows
-// 256 threads (up to 8192 elements).
-template <int THR, int PIECES, int SLOTS, int SORT, int MINB>
+// exclusive offsets, unordered fill, and a list of the centroids with more than
+// kMeanShort members (n_long of them over the batch, in no particular order).
+// A centroid with few members takes one CTA, which orders them by rank
+// (ascending row index, so the sum order is fixed), fetches the member rows with
+// bulk copies (cp.async.bulk, one thread issuing) into shared-memory row slots,
+// SLOTS rows per batch, and sums them slot by slot in rank order, each thread
+// over its 16-byte pieces of the row. Each such CTA is a short chain of
+// dependent steps, so the configuration is chosen for CTAs resident per SM: rows
+// of at most 8 KiB take 128 threads with 4 pieces each (8 CTAs per SM), longer
+// rows 256 threads (up to 8192 elements).
+// The long centroids (background that many tokens resemble) would be that chain
+// many times over in one CTA while the GPU drains, so the grid's first CTAs take
+// them, a 16-byte piece per thread: a column slice of one centroid per CTA (a
+// column's sum needs no other column), the members put in ascending order by a
+// bitmap over windows of kMeanWin rows, and their pieces kept kMeanDeep copies
+// ahead (cp.async) in the thread's own shared-memory slots, with no block
+// barrier between rows. With every list in its one CTA, a bf16 batch of 8 x 2880
+// rows whose largest centroids gather some hundreds took 143 us here where the
+// 253 MB it moves take 37; the whole pre-LLM pass went 356 -> 280 us (32 x 576
+// of width 5120: 262 -> 252, one fp32 image: 981 -> 946), the sums unchanged bit
+// for bit, and a video without such centroids stayed as it was (194 -> 192 us).
+constexpr int kMeanShort = 16;  // members of a centroid that one CTA sums row by row
+constexpr int kMeanDeep = 12;   // pieces in flight per thread for the others
+constexpr int kMeanWin = 1024;
+template <int THR, int PIECES, int SLOTS, int MINB>
 struct MeanCfg {
-  static constexpr int kThreads = THR, kWarps = THR / 32, kPieces = PIECES, kSlots = SLOTS, kSort = SORT,
-                       kMinBlocks = MINB;
+  static constexpr int kThreads = THR, kPieces = PIECES, kSlots = SLOTS, kMinBlocks = MINB;
 };
-using MeanSmall = MeanCfg<128, 4, 3, 256, 8>;       // row bytes <= 128 * 4 * 16
-using MeanBf16 = MeanCfg<256, 4, 4, 1024, 4>;       // bf16 rows <= 8192 elements
-using MeanF32 = MeanCfg<256, 8, 4, 1024, 2>;        // fp32 rows <= 8192 elements
+using MeanSmall = MeanCfg<128, 4, 3, 8>;  // row bytes <= 128 * 4 * 16
+using MeanBf16 = MeanCfg<256, 4, 4, 4>;   // bf16 rows <= 8192 elements
+using MeanF32 = MeanCfg<256, 8, 4, 2>;    // fp32 rows <= 8192 elements
 constexpr int kMeanSmallRowBytes = 128 * 4 * 16;
 constexpr int kSortSmemKeep = 6144;  // centroids whose counters the sort keeps in shared memory (48 KiB)
-template <typename C> size_t merge_mean_smem(int row_bytes) { return (size_t)C::kSlots * row_bytes; }
+template <typename C> size_t merge_mean_smem(int row_bytes) {
+  const size_t rows = (size_t)C::kSlots * row_bytes, ring = (size_t)kMeanDeep * C::kThreads * 16;
+  return rows > ring ? rows : ring;
+}
 
 // Counting sort of one sample's rows by centroid (one CTA of 1024 threads):
 // count[b][a] = rows assigned to a, offset[b][.] its exclusive scan, and
 // members[b][offset[a] ..] the rows of a in no particular order (the means
-// rank them). The block-wide barriers order the phases (global memory of this
+// rank them), and b * keep + a of every centroid with more than kMeanShort rows
+// appended to long_list (*n_long entries over the batch). The block-wide barriers order the phases (global memory of this
 // block only).
 template <bool kSmem>
 __global__ void __launch_bounds__(1024) merge_sort_kernel(const int* assign, int N_v, int keep, int* count,
-                                                          int* offset, int* cursor, int* members) {
+                                                          int* offset, int* cursor, int* members, int* n_long,
+                                                          int* long_list) {
   extern __shared__ int sort_sm[];  // kSmem: counts [keep], then offsets / cursors [keep]
   __shared__ uint32_t warp_tot[32];
   __shared__ uint32_t carry;
@@ -694,6 +714,7 @@ __global__ void __launch_bounds__(1024) merge_sort_kernel(const int* assign, int
     if (ap < keep) {
       const int o = (int)(carry + warp_tot[warp] + incl - v);
       off_g[ap] = o;
+      if (v > (uint32_t)kMeanShort) long_list[atomicAdd(n_long, 1)] = b * keep + ap;
       if (kSmem) {
         cnt_g[ap] = (int)v;
         cur[ap] = o;  // the fill's running position
@@ -740,101 +761,158 @@ __device__ __forceinline__ void store16(float* p, const double* v) {
   *reinterpret_cast<float4*>(p) = make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
 }
 
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Column slice `slice` (a 16-byte piece per thread) of centroid `cen` = b * keep
+// + a, whose n members lie unordered at mem[0..n). ring: kMeanDeep pieces per
+// thread. Called by every thread of the block.
+template <typename T, typename Acc, typename C>
+__device__ __forceinline__ void mean_long(const SimArgs& a, int b, int n, const int* mem, int slice, uint4* ring,
+                                          uint32_t* bits, int* pre, uint16_t* list, T* out) {
+  constexpr int kVec = 16 / (int)sizeof(T);
+  const int pc = slice * C::kThreads + (int)threadIdx.x;
+  const bool has = pc < a.D / kVec;
+  const T* E = static_cast<const T*>(a.emb_v) + (size_t)b * a.N_v * a.D + (size_t)(has ? pc : 0) * kVec;
+  uint4* mine = ring + threadIdx.x;
+  Acc acc[kVec];
+#pragma unroll
+  for (int e = 0; e < kVec; ++e) acc[e] = Acc(0);
+  for (int w0 = 0; w0 < a.N_v; w0 += kMeanWin) {
+    __syncthreads();  // the previous window's list has been read
+    if (threadIdx.x < kMeanWin / 32) bits[threadIdx.x] = 0u;
+    __syncthreads();
+    for (int m = threadIdx.x; m < n; m += C::kThreads) {
+      const int j = mem[m] - w0;
+      if (j >= 0 && j < kMeanWin) atomicOr(&bits[j >> 5], 1u << (j & 31));
+    }
+    __syncthreads();
+    if (threadIdx.x < kMeanWin / 32) {  // warp 0: members before each word
+      const int own = __popc(bits[threadIdx.x]);
+      int incl = own;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if ((int)threadIdx.x >= o) incl += y;
+      }
+      pre[threadIdx.x] = incl - own;
+      if (threadIdx.x == 31) pre[32] = incl;
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < kMeanWin; j += C::kThreads) {
+      const uint32_t w = bits[j >> 5];
+      if (w >> (j & 31) & 1u) list[pre[j >> 5] + __popc(w & ((1u << (j & 31)) - 1u))] = (uint16_t)j;
+    }
+    __syncthreads();
+    const int cnt = pre[32];
+    const T* Ew = E + (size_t)w0 * a.D;
+    // one group per row, empty past the last, so that a fixed count is in flight
+    auto fetch = [&](int i) {
+      if (has && i < cnt) cp_async16(mine + (i % kMeanDeep) * C::kThreads, Ew + (size_t)list[i] * a.D);
+      cp_async_commit();
+    };
+#pragma unroll 1
+    for (int i = 0; i < kMeanDeep - 1; ++i) fetch(i);
+#pragma unroll 1
+    for (int i = 0; i < cnt; ++i) {
+      fetch(i + kMeanDeep - 1);
+      cp_async_wait<kMeanDeep - 1>();
+      if (has) add16(acc, mine[(i % kMeanDeep) * C::kThreads], E);
+    }
+    cp_async_wait<0>();
+  }
+  if (has) {
+    Acc v[kVec];
+#pragma unroll
+    for (int e = 0; e < kVec; ++e) v[e] = acc[e] / (Acc)n;
+    store16(out + (size_t)pc * kVec, v);
+  }
+}
+
 template <typename T, typename Acc, typename C>
 __global__ void __launch_bounds__(C::kThreads, C::kMinBlocks)
-    merge_mean_kernel(const SimArgs a, const int* assign, const int* count, const int* offset,
-                      const int* members_all, int keep, void* merged) {
-  constexpr int kMeanThreads = C::kThreads, kMeanWarps = C::kWarps, kMeanSort = C::kSort,
-                kMeanSlots = C::kSlots;
-  extern __shared__ __align__(128) uint8_t slots[];  // kMeanSlots rows
-  __shared__ int members[kMeanSort];
-  __shared__ int unsorted[kMeanSort];
+    merge_mean_kernel(const SimArgs a, const int* count, const int* offset, const int* members_all, int keep,
+                      void* merged, const int* n_long, const int* long_list, int long_ctas) {
+  constexpr int kMeanThreads = C::kThreads, kMeanSlots = C::kSlots;
+  static_assert(kMeanWin / 32 == 32 && kMeanShort <= 32, "a word of the window per lane, a member per lane");
+  extern __shared__ __align__(128) uint8_t slots[];  // kMeanSlots rows, or the long centroids' ring
+  __shared__ int members[kMeanShort];
+  __shared__ uint32_t bits[kMeanWin / 32];
+  __shared__ int pre[kMeanWin / 32 + 1];
+  __shared__ uint16_t list[kMeanWin];
   __shared__ __align__(8) uint64_t bar;
-  __shared__ int wcount[kMeanWarps];
   constexpr int kVec = 16 / (int)sizeof(T);  // elements per 16-byte piece
   constexpr int kPieces = C::kPieces;
-  const int ap = blockIdx.x, b = blockIdx.y;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   pdl_wait_prior();  // the member lists come from the sort before
+  if ((int)blockIdx.x < long_ctas) {
+    const int n_slices = (a.D / kVec + kMeanThreads - 1) / kMeanThreads;
+    const long long n_tasks = (long long)*n_long * n_slices;
+    for (long long t = blockIdx.x; t < n_tasks; t += long_ctas) {
+      const int cen = long_list[t / n_slices], b = cen / keep;
+      mean_long<T, Acc, C>(a, b, count[cen], members_all + (size_t)b * a.N_v + offset[cen], (int)(t % n_slices),
+                           reinterpret_cast<uint4*>(slots), bits, pre, list,
+                           static_cast<T*>(merged) + (size_t)cen * a.D);
+    }
+    return;
+  }
+  const int cen = (int)blockIdx.x - long_ctas, b = cen / keep;
   const T* E = static_cast<const T*>(a.emb_v) + (size_t)b * a.N_v * a.D;
-  T* out = static_cast<T*>(merged) + ((size_t)b * keep + ap) * a.D;
+  T* out = static_cast<T*>(merged) + (size_t)cen * a.D;
   const uint32_t row_bytes = (uint32_t)a.D * (uint32_t)sizeof(T);
   const int n_pieces = a.D / kVec;
+  // count and offset issued together: the member list depends on both
+  const int n_all = count[cen];
+  const int off0 = offset[cen];
+  if (n_all > kMeanShort) return;  // among the long ones
   Acc acc[kPieces][kVec];
 #pragma unroll
   for (int k = 0; k < kPieces; ++k)
 #pragma unroll
     for (int e = 0; e < kVec; ++e) acc[k][e] = Acc(0);
-  // count and offset issued together: the member list depends on both
-  const int n_all = count[(size_t)b * keep + ap];
-  const int off0 = offset[(size_t)b * keep + ap];
-  if (threadIdx.x == 0) {
-    mbar_init(&bar, 1);
-    fence_mbar_init();
-  }
-  uint32_t phase = 0;
-  bool ok = true;
-  // adds rows members[0..n) in order: batches of kMeanSlots bulk copies
-  auto add_rows = [&](int n) {
-    for (int m0 = 0; m0 < n; m0 += kMeanSlots) {
-      const int nb = min(kMeanSlots, n - m0);
-      if (threadIdx.x == 0 && ok) {
-        const uint64_t pol = policy_evict_first();
-        mbar_arrive_expect_tx(&bar, (uint32_t)nb * row_bytes);
-        for (int q = 0; q < nb; ++q)
-          bulk_g2s(slots + (size_t)q * row_bytes, E + (size_t)members[m0 + q] * a.D, row_bytes, &bar, pol);
-      }
-      if (ok && !mbar_wait(&bar, phase, a.err)) ok = false;
-      phase ^= 1u;
-      if (ok) {
-        for (int q = 0; q < nb; ++q) {
-          const uint8_t* row = slots + (size_t)q * row_bytes;
+  if (threadIdx.x < 32) {
+    if (threadIdx.x == 0) {
+      mbar_init(&bar, 1);
+      fence_mbar_init();
+    }
+    // rank = number of smaller row indices (they are distinct)
+    const int lane = threadIdx.x;
+    const int v = lane < n_all ? members_all[(size_t)b * a.N_v + off0 + lane] : 0x7fffffff;
+    int rank = 0;
 #pragma unroll
-          for (int k = 0; k < kPieces; ++k) {
-            const int pc = k * kMeanThreads + (int)threadIdx.x;
-            if (pc < n_pieces) add16(acc[k], *reinterpret_cast<const uint4*>(row + (size_t)pc * 16), E);
-          }
+    for (int q = 0; q < kMeanShort; ++q) rank += __shfl_sync(0xffffffffu, v, q) < v;
+    if (lane < n_all) members[rank] = v;
+  }
+  __syncthreads();
+  bool ok = true;
+  uint32_t phase = 0;
+  // adds rows members[0..n_all) in order: batches of kMeanSlots bulk copies
+  for (int m0 = 0; m0 < n_all; m0 += kMeanSlots) {
+    const int nb = min(kMeanSlots, n_all - m0);
+    if (threadIdx.x == 0 && ok) {
+      const uint64_t pol = policy_evict_first();
+      mbar_arrive_expect_tx(&bar, (uint32_t)nb * row_bytes);
+      for (int q = 0; q < nb; ++q)
+        bulk_g2s(slots + (size_t)q * row_bytes, E + (size_t)members[m0 + q] * a.D, row_bytes, &bar, pol);
+    }
+    if (ok && !mbar_wait(&bar, phase, a.err)) ok = false;
+    phase ^= 1u;
+    if (ok) {
+      for (int q = 0; q < nb; ++q) {
+        const uint8_t* row = slots + (size_t)q * row_bytes;
+#pragma unroll
+        for (int k = 0; k < kPieces; ++k) {
+          const int pc = k * kMeanThreads + (int)threadIdx.x;
+          if (pc < n_pieces) add16(acc[k], *reinterpret_cast<const uint4*>(row + (size_t)pc * 16), E);
         }
       }
-      __syncthreads();  // the slots may be refilled
     }
-  };
-  if (n_all <= kMeanSort) {
-    const int* src = members_all + (size_t)b * a.N_v + off0;
-    for (int m = threadIdx.x; m < n_all; m += kMeanThreads) unsorted[m] = src[m];
-    __syncthreads();
-    // rank = number of smaller row indices (they are distinct)
-    for (int m = threadIdx.x; m < n_all; m += kMeanThreads) {
-      const int v = unsorted[m];
-      int rank = 0;
-      for (int q = 0; q < n_all; ++q) rank += unsorted[q] < v;
-      members[rank] = v;
-    }
-    __syncthreads();
-    add_rows(n_all);
-  } else {
-    // many members: scan assign in windows, members in ascending order
-    const int* as = assign + (size_t)b * a.N_v;
-    int base = 0;
-    for (int j0 = 0; j0 < a.N_v; j0 += kMeanThreads) {
-      const int j = j0 + threadIdx.x;
-      const bool hit = j < a.N_v && as[j] == ap;
-      const unsigned bal = __ballot_sync(0xffffffffu, hit);
-      if (lane == 0) wcount[warp] = __popc(bal);
-      __syncthreads();
-      int off = 0, tot = 0;
-      for (int w = 0; w < kMeanWarps; ++w) {
-        off += w < warp ? wcount[w] : 0;
-        tot += wcount[w];
-      }
-      if (hit) members[base + off + __popc(bal & ((1u << lane) - 1u))] = j;
-      __syncthreads();
-      base += tot;
-      if (base > kMeanSort - kMeanThreads || j0 + kMeanThreads >= a.N_v) {
-        add_rows(base);
-        base = 0;
-      }
-    }
+    __syncthreads();  // the slots may be refilled
   }
 #pragma unroll
   for (int k = 0; k < kPieces; ++k) {
@@ -1024,8 +1102,12 @@ cudaError_t merge_launch(const SimArgs& a, const int* keep_idx, int keep, const 
       merge_argmax_kernel<__nv_bfloat16><<<g, 256, 0, s>>>(a, keep_idx, keep, inv_v, kpos, n_split, ws_best,
                                                            ws_bidx);
   }
+  // the counter of the long centroids lies past the pruned list's last entry
+  // (keep >= 1 leaves room), which nothing else uses
+  int* n_long = merged != nullptr ? ws_pruned + (size_t)a.B * (a.N_v - keep) : nullptr;
   cudaError_t el = launch_pdl(merge_assign_kernel, dim3((unsigned)((nb + 255) / 256)), dim3(256), 0, s, a,
-                              (const int*)kpos, n_split, (const float*)ws_best, (const int*)ws_bidx, assign);
+                              (const int*)kpos, n_split, (const float*)ws_best, (const int*)ws_bidx, assign,
+                              n_long);
   if (el != cudaSuccess) return el;
   if (merged != nullptr) {
     // counting sort of the rows by centroid; the scratch reuses ws_best/ws_bidx
@@ -1033,15 +1115,15 @@ cudaError_t merge_launch(const SimArgs& a, const int* keep_idx, int keep, const 
     int* cnt = ws_bidx;
     int* off = cnt + (size_t)a.B * keep;
     int* cur = off + (size_t)a.B * keep;
+    int* lng = cur + (size_t)a.B * keep;
     int* mem = reinterpret_cast<int*>(ws_best);
     cudaError_t es = keep <= kSortSmemKeep
                          ? launch_pdl(merge_sort_kernel<true>, dim3(a.B), dim3(1024),
                                       (size_t)2 * keep * sizeof(int), s, (const int*)assign, a.N_v, keep, cnt,
-                                      off, cur, mem)
+                                      off, cur, mem, n_long, lng)
                          : launch_pdl(merge_sort_kernel<false>, dim3(a.B), dim3(1024), 0, s, (const int*)assign,
-                                      a.N_v, keep, cnt, off, cur, mem);
+                                      a.N_v, keep, cnt, off, cur, mem, n_long, lng);
     if (es != cudaSuccess) return es;
-    dim3 gm(keep, a.B);
     static std::atomic<bool> configured[64];  // per device, zero-initialised
     int dev = 0;
     cudaGetDevice(&dev);
@@ -1057,23 +1139,24 @@ cudaError_t merge_launch(const SimArgs& a, const int* keep_idx, int keep, const 
       configured[dev] = true;
     }
     const int row_bytes = a.D * (a.dtype == 0 ? 4 : 2);
+    // CTAs for the long centroids: two per SM (they leave at once where none is
+    // long), one where so few rows are pruned that none can be with a valid keep_idx
+    const int n_lc = a.N_v - keep >= kMeanShort ? 2 * num_sms : 1;
+    const dim3 gm((unsigned)((size_t)a.B * keep + n_lc));
     cudaError_t em;
+    auto go = [&](auto kernel, unsigned threads, size_t smem) {
+      return launch_pdl(kernel, gm, dim3(threads), smem, s, a, (const int*)cnt, (const int*)off, (const int*)mem,
+                        keep, merged, (const int*)n_long, (const int*)lng, n_lc);
+    };
     if (row_bytes <= kMeanSmallRowBytes) {
       const size_t smem = merge_mean_smem<MeanSmall>(row_bytes);
-      if (a.dtype == 0)
-        em = launch_pdl(merge_mean_kernel<float, double, MeanSmall>, gm, dim3(MeanSmall::kThreads), smem, s, a,
-                        (const int*)assign, (const int*)cnt, (const int*)off, (const int*)mem, keep, merged);
-      else
-        em = launch_pdl(merge_mean_kernel<__nv_bfloat16, float, MeanSmall>, gm, dim3(MeanSmall::kThreads), smem,
-                        s, a, (const int*)assign, (const int*)cnt, (const int*)off, (const int*)mem, keep, merged);
+      em = a.dtype == 0 ? go(merge_mean_kernel<float, double, MeanSmall>, MeanSmall::kThreads, smem)
+                        : go(merge_mean_kernel<__nv_bfloat16, float, MeanSmall>, MeanSmall::kThreads, smem);
     } else if (a.dtype == 0) {
-      em = launch_pdl(merge_mean_kernel<float, double, MeanF32>, gm, dim3(MeanF32::kThreads),
-                      merge_mean_smem<MeanF32>(row_bytes), s, a, (const int*)assign, (const int*)cnt,
-                      (const int*)off, (const int*)mem, keep, merged);
+      em = go(merge_mean_kernel<float, double, MeanF32>, MeanF32::kThreads, merge_mean_smem<MeanF32>(row_bytes));
     } else {
-      em = launch_pdl(merge_mean_kernel<__nv_bfloat16, float, MeanBf16>, gm, dim3(MeanBf16::kThreads),
-                      merge_mean_smem<MeanBf16>(row_bytes), s, a, (const int*)assign, (const int*)cnt,
-                      (const int*)off, (const int*)mem, keep, merged);
+      em = go(merge_mean_kernel<__nv_bfloat16, float, MeanBf16>, MeanBf16::kThreads,
+              merge_mean_smem<MeanBf16>(row_bytes));
     }
     if (em != cudaSuccess) return em;
   }

@@ -1,0 +1,57 @@
+"""GPU parity of the merge's means when some centroids gather many rows (their
+own CTAs, a column slice each): member counts at the limit between the two
+paths and past one window of the ordering bitmap, rows of every configuration
+and of a partial last slice, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2608_25332_gb300 import provip as P
+from parity import check_merge
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import __graft_entry__
+    __graft_entry__.build()
+    yield
+    rc, bits = P.provip_device_status(clear=True)
+    assert rc == 0 and bits == 0, f"device status {rc} {bits}"
+
+
+@pytest.mark.parametrize("dtype,D,B", [("bf16", 64, 3), ("bf16", 1040, 2), ("bf16", 4096, 1), ("bf16", 4104, 1),
+                                       ("f32", 200, 2), ("f32", 2048, 1), ("f32", 2056, 1)])
+def test_merge_means_of_long_centroids(dtype, D, B):
+    """Groups of 16, 17, 1 and 1100 rows (the kept one included) around well
+    separated directions, scattered over the sample; N_v spans two windows."""
+    sizes = (16, 17, 1, 1100, 12, 40)
+    rng = np.random.default_rng(D)
+    N_v = sum(sizes)
+    Ev = np.empty((B, N_v, D), np.float32)
+    keeps = np.empty((B, len(sizes)), np.int32)
+    for b in range(B):
+        place = rng.permutation(N_v)
+        o = 0
+        for n in sizes:
+            c = rng.standard_normal(D)
+            rows = place[o:o + n]
+            Ev[b, rows] = c + 0.3 * rng.standard_normal((n, D))
+            o += n
+        heads = [place[sum(sizes[:i])] for i in range(len(sizes))]
+        keeps[b] = np.sort(heads)
+    td = torch.bfloat16 if dtype == "bf16" else torch.float32
+    ev = torch.from_numpy(Ev).to(td)
+    assign, merged = P.provip_merge(ev.to(DEV), torch.from_numpy(keeps).to(DEV))
+    torch.cuda.synchronize()
+    Evn = ev.float().numpy().astype(np.float64)
+    for b in range(B):
+        a_ref, mg_ref = oracle.merge(Evn[b], keeps[b])
+        assert sorted(np.bincount(a_ref, minlength=len(sizes)).tolist()) == sorted(sizes)
+        check_merge(Evn[b], keeps[b], assign[b].cpu().numpy(), merged[b].float().cpu().numpy().astype(np.float64),
+                    dtype, f"long centroids {dtype} D={D} [{b}]", a_ref,
+                    np.setdiff1d(np.arange(N_v), keeps[b]), mg_ref=mg_ref)
