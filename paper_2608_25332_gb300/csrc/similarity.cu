@@ -1014,7 +1014,7 @@ cudaError_t vis_inv_norm_launch(const SimArgs& a, float* inv_v, cudaStream_t s) 
 cudaError_t relevance_launch(const SimArgs& a, const uint8_t* mask, float* inv_v, float* p,
                              float* ws_sum, float* ws_mu, float* ws_invt, int n_split,
                              int num_sms, cudaStream_t s, cudaEvent_t mask_ready) {
-  // bf16 with at most 128 text rows: the text rows' inverse norms, one
+  // bf16 (up to 4096 text rows): the text rows' inverse norms, one
   // tensor-core read of the visual rows (norms, cosines and de-meaning sums)
   // and a small max kernel
   if (relevance_tc_supported(a)) {

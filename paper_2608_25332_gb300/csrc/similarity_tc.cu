@@ -315,16 +315,28 @@ __global__ void __launch_bounds__(kMergeThreads, 1)
 //     butterfly, then the four lane quadrants in order).
 // relevance_finish_kernel then forms mu_i = (sum of the tile sums in tile
 // order) / N_v and p_j = max_{i in T} (Y[b][j][i] - mu_i) (Sec. 4.3).
+// More than 128 text rows are split into blocks of at most 128 (grid z); each
+// block's CTAs read the visual tiles again (from L2, where the first block's
+// loads left them) and form their norms themselves. These CTAs are bound by the
+// latency of their K loop and are few, so they run one per SM with two
+// accumulators (kAcc = 2), each over half of the K slices: the tensor core
+// truncates at every accumulation, and the shorter chains keep p as close to its
+// value as the FFMA kernel that took such texts before (relative error of p
+// against 64 bits over widths 2048 to 5120: 2-7e-7, FFMA 6-12e-7). That kernel
+// took 990 us on 4 x 1443 visual rows under 300 text rows (23 x 4 CTAs, each a
+// chain of 128 K steps of 2.4 us per 128 text rows); the whole pre-LLM pass of
+// that batch went from 1322 to 605 us.
 struct RelFusedArgs {
   int B, N_v, D, N_t_max;
-  int NT;        // text rows in the MMA (N_t_max rounded up to 16)
+  int NT;        // text rows in the MMA (a block's rows, a multiple of 16)
+  int NTs;       // text columns of Y and part (N_t_max rounded up to 16)
   int R;         // visual rows per tile (128, 96 or 64)
   int n_vt;      // visual tiles per sample
   int n_stages;  // shared-memory ring depth
   const float* inv_t;  // [B][N_t_max]
   float* inv_v;  // [B][N_v]
-  float* Y;      // [B][N_v][NT]
-  float* part;   // [B][n_vt][NT]
+  float* Y;      // [B][N_v][NTs]
+  float* part;   // [B][n_vt][NTs]
   unsigned* err;
 };
 
@@ -340,7 +352,8 @@ struct RelPipe {
   volatile int fail;
 };
 
-__global__ void __launch_bounds__(kThreads, 2)
+template <int kAcc>
+__global__ void __launch_bounds__(kThreads, 2 / kAcc)
     relevance_fused_tc(const RelFusedArgs a, const __grid_constant__ CUtensorMap mapV,
                        const __grid_constant__ CUtensorMap mapT) {
   extern __shared__ uint8_t smem_raw[];
@@ -348,6 +361,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   __shared__ float s_invt[kBM];
   __shared__ float red[4][kBM];
   const int b = blockIdx.y, tile = blockIdx.x;
+  const int tb0 = blockIdx.z * a.NT;  // first text row of the block
   const int R = a.R;
   const int n0 = tile * R;
   const int n_k = (a.D + kBK - 1) / kBK;
@@ -367,7 +381,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     fence_mbar_init();
   }
   if (threadIdx.x < 32) {
-    tmem_alloc(&pipe.tmem, kRelTmemCols);
+    tmem_alloc(&pipe.tmem, kAcc * kRelTmemCols);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -388,12 +402,13 @@ __global__ void __launch_bounds__(kThreads, 2)
         // rows past the sample's last visual row belong to the next sample (or
         // lie past the tensor and read as zeros): computed, never stored
         tma_load_2d(sa, &mapV, kb * kBK, b * a.N_v + n0, &pipe.full[s]);
-        tma_load_2d(sa + R * 128, &mapT, kb * kBK, b * a.N_t_max, &pipe.full[s]);
+        tma_load_2d(sa + R * 128, &mapT, kb * kBK, b * a.N_t_max + tb0, &pipe.full[s]);
       }
     }
   } else if (warp == 1) {
     if (lane == 0) {
       const uint32_t idesc = idesc_bf16_f32(kBM, R + a.NT);
+      const int kb1 = kAcc == 1 ? n_k : (n_k + 1) / 2;  // first slice of the second accumulator
       for (int kb = 0; kb < n_k; ++kb) {
         const int s = kb % NS;
         const uint32_t ph = (uint32_t)(kb / NS) & 1u;
@@ -405,8 +420,8 @@ __global__ void __launch_bounds__(kThreads, 2)
         const uint32_t sa = smem_u32(stages + (size_t)s * st_bytes);
 #pragma unroll
         for (int k = 0; k < kBK / 16; ++k)
-          tc_mma_bf16(pipe.tmem, smem_desc_sw128(sa + k * 32), smem_desc_sw128(sa + k * 32), idesc,
-                      (kb > 0 || k > 0) ? 1u : 0u);
+          tc_mma_bf16(pipe.tmem + (kb >= kb1 ? kRelTmemCols : 0u), smem_desc_sw128(sa + k * 32),
+                      smem_desc_sw128(sa + k * 32), idesc, ((kb != 0 && kb != kb1) || k > 0) ? 1u : 0u);
         tc_commit(&pipe.empty[s]);
       }
       tc_commit(&pipe.acc_full);  // arrives once every MMA above has completed
@@ -419,31 +434,45 @@ __global__ void __launch_bounds__(kThreads, 2)
     // launched as a programmatic dependent of the text-row norms: the loads and
     // MMAs ran under that kernel; its output (and every write below) waits here
     pdl_wait_prior();
-    s_invt[r] = r < a.N_t_max ? a.inv_t[(size_t)b * a.N_t_max + r] : 0.f;
+    s_invt[r] = tb0 + r < a.N_t_max ? a.inv_t[(size_t)b * a.N_t_max + tb0 + r] : 0.f;
     asm volatile("bar.sync 1, 128;" ::: "memory");  // s_invt complete (epilogue warps)
     const bool ok = warp_mbar_wait(&pipe.acc_full, 0, a.err) && !pipe.fail;
     tc_fence_after();
     const uint32_t taddr = pipe.tmem + ((uint32_t)(quad * 32) << 16);
     float v[32];
+    // 32 columns from column c of the accumulator (of both: one K slice has no second)
+    const bool two = kAcc == 2 && n_k > 1;
+    auto load_cols = [&](int c) {
+      tmem_ld32(taddr + (uint32_t)c, v);
+      if (two) {
+        float w[32];
+        tmem_ld32(taddr + kRelTmemCols + (uint32_t)c, w);
+        tc_wait_ld_into(w);
+        tc_wait_ld_into(v);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] += w[i];
+      } else {
+        tc_wait_ld();
+      }
+    };
     // |v_j|^2: column j of the visual block, i.e. element `lane` of the warp's 32 columns
-    tmem_ld32(taddr + (uint32_t)(quad * 32), v);
-    tc_wait_ld();
+    load_cols(quad * 32);
     float sqv = 0.f;
 #pragma unroll
     for (int i = 0; i < 32; ++i) sqv = i == lane ? v[i] : sqv;
     const float iv = sqv > 0.f ? 1.f / sqrtf(sqv) : 0.f;
-    if (rv && ok) a.inv_v[(size_t)b * a.N_v + j] = iv;
-    float* yrow = a.Y + ((size_t)b * a.N_v + (rv ? j : 0)) * a.NT;
+    if (rv && ok && blockIdx.z == 0) a.inv_v[(size_t)b * a.N_v + j] = iv;
+    const int nt = min(a.NT, a.NTs - tb0);  // the last block may be narrower
+    float* yrow = a.Y + ((size_t)b * a.N_v + (rv ? j : 0)) * a.NTs + tb0;
 #pragma unroll 1
-    for (int cb = 0; cb * 32 < a.NT; ++cb) {
-      tmem_ld32(taddr + (uint32_t)(R + cb * 32), v);
-      tc_wait_ld();
+    for (int cb = 0; cb * 32 < nt; ++cb) {
+      load_cols(R + cb * 32);
 #pragma unroll
       for (int i = 0; i < 32; ++i) v[i] = v[i] * s_invt[cb * 32 + i] * iv;
       if (rv && ok) {
 #pragma unroll
         for (int q = 0; q < 8; ++q)
-          if (cb * 32 + q * 4 < a.NT)
+          if (cb * 32 + q * 4 < nt)
             *reinterpret_cast<float4*>(yrow + cb * 32 + q * 4) =
                 make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
       }
@@ -465,12 +494,12 @@ __global__ void __launch_bounds__(kThreads, 2)
     tc_fence_before();
     asm volatile("bar.sync 1, 128;" ::: "memory");
     const int c = threadIdx.x - 64;
-    if (c < a.NT && ok)
-      a.part[((size_t)b * a.n_vt + tile) * a.NT + c] = (red[0][c] + red[1][c]) + (red[2][c] + red[3][c]);
+    if (c < nt && ok)
+      a.part[((size_t)b * a.n_vt + tile) * a.NTs + tb0 + c] = (red[0][c] + red[1][c]) + (red[2][c] + red[3][c]);
   }
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x < 32) tmem_dealloc(pipe.tmem, kRelTmemCols);
+  if (threadIdx.x < 32) tmem_dealloc(pipe.tmem, kAcc * kRelTmemCols);
 }
 
 // mu_i from the tile sums (tile order; every CTA forms all of mu), then p_j =
@@ -478,19 +507,19 @@ __global__ void __launch_bounds__(kThreads, 2)
 __global__ void __launch_bounds__(256) relevance_finish_kernel(const RelFusedArgs a, const int* text_len,
                                                                const uint8_t* mask, float* p) {
   pdl_allow_next();  // the top-k reads p only after this grid completes
-  __shared__ float mu[kBM];
-  __shared__ int valid[kBM];
+  extern __shared__ float mu[];  // mu [NTs], valid [NTs]
+  int* valid = reinterpret_cast<int*>(mu + a.NTs);
   const int b = blockIdx.y;
   const int tl = min(max(text_len[b], 0), a.N_t_max);
-  for (int c = threadIdx.x; c < a.NT; c += blockDim.x) {
+  for (int c = threadIdx.x; c < a.NTs; c += blockDim.x) {
     const bool v = c < tl && mask[(size_t)b * a.N_t_max + c] != 0;
     float s = 0.f;
     if (v) {
-      const float* col = a.part + (size_t)b * a.n_vt * a.NT + c;
+      const float* col = a.part + (size_t)b * a.n_vt * a.NTs + c;
       for (int t0 = 0; t0 < a.n_vt; t0 += 32) {
         float x[32];
 #pragma unroll
-        for (int u = 0; u < 32; ++u) x[u] = t0 + u < a.n_vt ? col[(size_t)(t0 + u) * a.NT] : 0.f;
+        for (int u = 0; u < 32; ++u) x[u] = t0 + u < a.n_vt ? col[(size_t)(t0 + u) * a.NTs] : 0.f;
 #pragma unroll
         for (int u = 0; u < 32; ++u)
           if (t0 + u < a.n_vt) s += x[u];
@@ -500,31 +529,36 @@ __global__ void __launch_bounds__(256) relevance_finish_kernel(const RelFusedArg
     valid[c] = v;
   }
   __syncthreads();
-  // a warp per kRelFinishRows rows: lane q reads the 16-byte piece q of each row
-  // (NT <= 128: at most 32 pieces), every row's load in flight, then a warp max
+  // a warp per kRelFinishRows rows: lane q reads the 16-byte pieces q, q + 32, ..
+  // of each row (one piece up to 128 text rows), every row's load in flight, then
+  // a warp max
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nq = a.NT / 4;
+  const int nq = a.NTs / 4;
   const int j0 = (blockIdx.x * (blockDim.x >> 5) + warp) * kRelFinishRows;
-  const bool has = lane < nq;
-  const int c = lane * 4;
-  const float m0 = has ? mu[c] : 0.f, m1 = has ? mu[c + 1] : 0.f, m2 = has ? mu[c + 2] : 0.f,
-              m3 = has ? mu[c + 3] : 0.f;
-  const bool v0 = has && valid[c], v1 = has && valid[c + 1], v2 = has && valid[c + 2], v3 = has && valid[c + 3];
-  const float4* y = reinterpret_cast<const float4*>(a.Y + (size_t)b * a.N_v * a.NT);
-  float4 f[kRelFinishRows];
+  const float4* y = reinterpret_cast<const float4*>(a.Y + (size_t)b * a.N_v * a.NTs);
+  float best[kRelFinishRows];
 #pragma unroll
-  for (int r = 0; r < kRelFinishRows; ++r)
-    f[r] = (has && j0 + r < a.N_v) ? y[(size_t)(j0 + r) * nq + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int r = 0; r < kRelFinishRows; ++r) best[r] = -INFINITY;
+  for (int q = lane; q < nq; q += 32) {
+    const int c = q * 4;
+    const float m0 = mu[c], m1 = mu[c + 1], m2 = mu[c + 2], m3 = mu[c + 3];
+    const bool v0 = valid[c], v1 = valid[c + 1], v2 = valid[c + 2], v3 = valid[c + 3];
+    float4 f[kRelFinishRows];
+#pragma unroll
+    for (int r = 0; r < kRelFinishRows; ++r)
+      f[r] = j0 + r < a.N_v ? y[(size_t)(j0 + r) * nq + q] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int r = 0; r < kRelFinishRows; ++r) {
+      if (v0) best[r] = fmaxf(best[r], f[r].x - m0);
+      if (v1) best[r] = fmaxf(best[r], f[r].y - m1);
+      if (v2) best[r] = fmaxf(best[r], f[r].z - m2);
+      if (v3) best[r] = fmaxf(best[r], f[r].w - m3);
+    }
+  }
 #pragma unroll
   for (int r = 0; r < kRelFinishRows; ++r) {
-    float best = -INFINITY;
-    if (v0) best = fmaxf(best, f[r].x - m0);
-    if (v1) best = fmaxf(best, f[r].y - m1);
-    if (v2) best = fmaxf(best, f[r].z - m2);
-    if (v3) best = fmaxf(best, f[r].w - m3);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
-    if (lane == 0 && j0 + r < a.N_v) p[(size_t)b * a.N_v + j0 + r] = best;
+    const float m = warp_max(best[r]);
+    if (lane == 0 && j0 + r < a.N_v) p[(size_t)b * a.N_v + j0 + r] = m;
   }
 }
 
@@ -675,7 +709,9 @@ cudaError_t merge_argmax_tc_launch(const SimArgs& a, const int* keep_idx, int ke
   return cudaGetLastError();
 }
 
-bool relevance_tc_supported(const SimArgs& a) { return a.dtype == 1 && a.N_t_max <= kBM && a.D % 8 == 0; }
+// up to the text rows that the finish kernel's shared memory holds (32 KiB)
+constexpr int kRelMaxNt = 4096;
+bool relevance_tc_supported(const SimArgs& a) { return a.dtype == 1 && a.N_t_max <= kRelMaxNt && a.D % 8 == 0; }
 
 static int rel_nt(int N_t_max) { return (N_t_max + 15) / 16 * 16; }
 
@@ -687,11 +723,11 @@ size_t relevance_fused_floats(int B, int N_v, int N_t_max) {
 // Visual rows per relevance tile: the R of 128, 96 and 64 whose tiles give the
 // busiest SM the fewest rows to take in (its tiles' visual and text rows,
 // ceil(tiles / SMs) tiles), the larger R on a tie.
-static int rel_tile_rows(int B, int N_v, int NT, int num_sms) {
+static int rel_tile_rows(int B, int N_v, int NT, int n_tb, int num_sms) {
   int best = kBM;
   long long best_cost = -1;
   for (int R = kBM; R >= 64; R -= 32) {
-    const long long tiles = (long long)B * ((N_v + R - 1) / R);
+    const long long tiles = (long long)B * ((N_v + R - 1) / R) * n_tb;
     const long long cost = ((tiles + num_sms - 1) / num_sms) * (R + NT);
     if (best_cost < 0 || cost < best_cost) {
       best_cost = cost;
@@ -703,31 +739,36 @@ static int rel_tile_rows(int B, int N_v, int NT, int num_sms) {
 
 cudaError_t relevance_tc_launch(const SimArgs& a, const uint8_t* mask, const float* inv_t, float* inv_v,
                                 float* p, float* ws, int num_sms, cudaStream_t s, cudaEvent_t mask_ready) {
-  static std::atomic<bool> smem_set[64];  // per device, zero-initialised
+  static std::atomic<bool> smem_set[64], smem_set2[64];  // per device, zero-initialised
   int dev = 0;
   cudaGetDevice(&dev);
   constexpr size_t kSmemMax = 200 * 1024;
-  cudaError_t e = set_smem(relevance_fused_tc, kSmemMax, &smem_set[dev < 64 ? dev : 0]);
+  cudaError_t e = set_smem(relevance_fused_tc<1>, kSmemMax, &smem_set[dev < 64 ? dev : 0]);
+  if (e == cudaSuccess) e = set_smem(relevance_fused_tc<2>, kSmemMax, &smem_set2[dev < 64 ? dev : 0]);
   if (e != cudaSuccess) return e;
   RelFusedArgs r;
   r.B = a.B;
   r.N_v = a.N_v;
   r.D = a.D;
   r.N_t_max = a.N_t_max;
-  r.NT = rel_nt(a.N_t_max);
-  r.R = rel_tile_rows(a.B, a.N_v, r.NT, num_sms);
+  r.NTs = rel_nt(a.N_t_max);
+  const int n_tb = (r.NTs + kBM - 1) / kBM;  // text blocks, of equal rows but for the last
+  r.NT = rel_nt((r.NTs + n_tb - 1) / n_tb);
+  r.R = rel_tile_rows(a.B, a.N_v, r.NT, n_tb, num_sms);
   r.n_vt = (a.N_v + r.R - 1) / r.R;
   r.inv_t = inv_t;
   r.inv_v = inv_v;
   r.Y = ws;
-  r.part = ws + (size_t)a.B * a.N_v * r.NT;
+  r.part = ws + (size_t)a.B * a.N_v * r.NTs;
   r.err = a.err;
-  // one CTA per SM when the tiles do not fill the GPU (deeper ring), else two
+  // one CTA per SM when the tiles do not fill the GPU or there are several text
+  // blocks (deeper ring), else two
   // the MMA reads 128 A rows (16 KiB) from the start of a stage: the last
   // stage keeps that much room even when R + NT rows are fewer
   const size_t st_bytes = (size_t)(r.R + r.NT) * 128;
   const size_t tail = st_bytes > (size_t)kABytes ? 0 : (size_t)kABytes - st_bytes;
-  const size_t budget = ((long long)a.B * r.n_vt <= num_sms ? kSmemMax - 1024 : 110 * 1024 - 1024) - tail;
+  const bool deep = n_tb > 1 || (long long)a.B * r.n_vt <= num_sms;
+  const size_t budget = (deep ? kSmemMax - 1024 : 110 * 1024 - 1024) - tail;
   int ns = (int)(budget / st_bytes);
   r.n_stages = ns > kRelMaxStages ? kRelMaxStages : (ns < 2 ? 2 : ns);
   const size_t smem = (size_t)r.n_stages * st_bytes + tail + 1024;
@@ -736,14 +777,15 @@ cudaError_t relevance_tc_launch(const SimArgs& a, const uint8_t* mask, const flo
       make_tmap_bf16_2d(&mapT, a.emb_t, (uint64_t)a.B * a.N_t_max, (uint64_t)a.D, (uint64_t)a.D * 2,
                         (uint32_t)r.NT))
     return cudaErrorInvalidValue;
-  e = launch_pdl(relevance_fused_tc, dim3(r.n_vt, a.B), dim3(kThreads), smem, s, r, mapV, mapT);
+  e = n_tb == 1 ? launch_pdl(relevance_fused_tc<1>, dim3(r.n_vt, a.B), dim3(kThreads), smem, s, r, mapV, mapT)
+                : launch_pdl(relevance_fused_tc<2>, dim3(r.n_vt, a.B, n_tb), dim3(kThreads), smem, s, r, mapV, mapT);
   if (e != cudaSuccess) return e;
   if (mask_ready != nullptr) {
     e = cudaStreamWaitEvent(s, mask_ready, 0);  // the first kernel that reads the mask
     if (e != cudaSuccess) return e;
   }
-  relevance_finish_kernel<<<dim3((a.N_v + 8 * kRelFinishRows - 1) / (8 * kRelFinishRows), a.B), 256, 0, s>>>(
-      r, a.text_len, mask, p);
+  relevance_finish_kernel<<<dim3((a.N_v + 8 * kRelFinishRows - 1) / (8 * kRelFinishRows), a.B), 256,
+                            (size_t)r.NTs * (sizeof(float) + sizeof(int)), s>>>(r, a.text_len, mask, p);
   return cudaGetLastError();
 }
 
