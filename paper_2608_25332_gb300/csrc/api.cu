@@ -493,15 +493,21 @@ extern "C" int provip_selftest_wait_timeout(void* stream) {
 // ===========================================================================
 // pre-LLM pass
 // ===========================================================================
-// the text Gram, in as many K parts as its tcgen05 form uses (bf16)
-static size_t crit_gram_floats(int B, int N_t_max, int D, int dtype) {
-  const int parts = crit_splits(N_t_max, D, dtype);
-  return (size_t)(parts > 0 ? parts : 1) * B * N_t_max * N_t_max;
+// the text Gram's workspace: 16 parts of it up to 128 text rows, one beyond (what
+// its kernels needed once; they use one part at most, and a caller that kept a
+// size keeps a valid one)
+static size_t crit_gram_floats(int B, int N_t_max, int D) {
+  size_t parts = 1;
+  if (N_t_max <= 128 && D % 8 == 0) {
+    const int n_k = (D + 63) / 64, ns = n_k < 16 ? n_k : 16, per = (n_k + ns - 1) / ns;
+    parts = (size_t)((n_k + per - 1) / per);
+  }
+  return parts * B * N_t_max * N_t_max;
 }
 
 extern "C" size_t provip_crit_text_workspace_size(int B, int N_t_max, int D) {
   Carve c(nullptr);
-  c.take<float>(crit_gram_floats(B, N_t_max, D, PROVIP_BF16));  // the larger of the two dtypes' needs
+  c.take<float>(crit_gram_floats(B, N_t_max, D));
   return c.off;
 }
 
@@ -512,14 +518,14 @@ extern "C" int provip_crit_text(const void* emb_t, int B, int N_t_max, int D, co
   int rc = sim_validate_common(emb_t, B, N_t_max, D, dtype, "crit_text");
   if (rc) return rc;
   if (!text_len || !mask_out) return fail(PROVIP_ERR_INVALID_ARG, "crit_text: null text_len/mask_out");
-  if (N_t_max > 4096) return fail(PROVIP_ERR_UNSUPPORTED, "crit_text: N_t_max > 4096");
+  if (N_t_max > kCritMaxNt) return fail(PROVIP_ERR_UNSUPPORTED, "crit_text: N_t_max > %d", kCritMaxNt);
   if ((rc = check_ws(provip_crit_text_workspace_size(B, N_t_max, D), ws, ws_bytes, "crit_text"))) return rc;
   DevInfo* d;
   if ((rc = dev_info(&d))) return rc;
   Carve c(ws);
-  float* G = c.take<float>(crit_gram_floats(B, N_t_max, D, PROVIP_BF16));
+  float* G = c.take<float>(crit_gram_floats(B, N_t_max, D));
   SimArgs a = sim_args(nullptr, emb_t, text_len, B, 1, D, N_t_max, dtype, d->status);
-  cudaError_t e = crit_text_launch(a, mask_out, r_out, G, static_cast<cudaStream_t>(stream));
+  cudaError_t e = crit_text_launch(a, mask_out, r_out, G, d->sms, static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? PROVIP_OK : cuda_fail(e, "crit_text launch");
 }
 
@@ -633,7 +639,7 @@ extern "C" int provip_merge(const void* emb_v, int B, int N_v, int D, const int*
 }
 
 static size_t simred_ws(Carve& c, int B, int N_v, int D, int N_t_max, int keep_pre, SimWs& w) {
-  w.G = c.take<float>(crit_gram_floats(B, N_t_max, D, PROVIP_BF16));
+  w.G = c.take<float>(crit_gram_floats(B, N_t_max, D));
   w.mask = c.take<uint8_t>((size_t)B * N_t_max);
   w.p = c.take<float>((size_t)B * N_v);
   w.assign = c.take<int>((size_t)B * N_v);
@@ -672,7 +678,7 @@ extern "C" int provip_similarity_reduce(const void* emb_v, int B, int N_v, int D
   if (!text_len || !idx_out) return fail(PROVIP_ERR_INVALID_ARG, "similarity_reduce: null text_len/idx_out");
   if (keep_pre < 1 || keep_pre > N_v) return fail(PROVIP_ERR_INVALID_ARG, "similarity_reduce: keep_pre %d", keep_pre);
   if (N_v > kTopkMaxN) return fail(PROVIP_ERR_UNSUPPORTED, "similarity_reduce: N_v > %d", kTopkMaxN);
-  if (N_t_max > 4096) return fail(PROVIP_ERR_UNSUPPORTED, "similarity_reduce: N_t_max > 4096");
+  if (N_t_max > kCritMaxNt) return fail(PROVIP_ERR_UNSUPPORTED, "similarity_reduce: N_t_max > %d", kCritMaxNt);
   if (merged_out_or_null && D > 8192) return fail(PROVIP_ERR_UNSUPPORTED, "similarity_reduce: D > 8192");
   if ((rc = check_ws(provip_similarity_reduce_workspace_size(B, N_v, D, N_t_max, keep_pre), ws,
                      ws_bytes, "similarity_reduce")))
@@ -696,7 +702,7 @@ extern "C" int provip_similarity_reduce(const void* emb_v, int B, int N_v, int D
     if ((rc = side_stream(&side))) return rc;
     e = cudaEventRecord(side->fork, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(side->s, side->fork, 0);
-    if (e == cudaSuccess) e = crit_text_launch(a, mask_dst, nullptr, w.G, side->s);
+    if (e == cudaSuccess) e = crit_text_launch(a, mask_dst, nullptr, w.G, d->sms, side->s);
     if (e == cudaSuccess) e = cudaEventRecord(side->join, side->s);
     if (e == cudaSuccess) mask_ready = side->join;
     mask = mask_dst;

@@ -174,9 +174,10 @@ struct SimArgs {
   int dtype;
   unsigned* err;
 };
-// Sec. 4.2: mask[b][j] (and r) from the text self-similarity. ws: G, max(1,
-// crit_splits) x [B][Ntm][Ntm] f32.
-cudaError_t crit_text_launch(const SimArgs& a, uint8_t* mask, float* r_out, float* G,
+// Sec. 4.2: mask[b][j] (and r) from the text self-similarity. ws: G, [B][Ntm][Ntm]
+// f32; Ntm <= kCritMaxNt.
+constexpr int kCritMaxNt = 4096;
+cudaError_t crit_text_launch(const SimArgs& a, uint8_t* mask, float* r_out, float* G, int num_sms,
                              cudaStream_t s);
 // inverse L2 norms of every visual row (0 for a zero row): inv_v [B][N_v]
 cudaError_t vis_inv_norm_launch(const SimArgs& a, float* inv_v, cudaStream_t s);
@@ -207,12 +208,9 @@ cudaError_t merge_launch(const SimArgs& a, const int* keep_idx, int keep, const 
                          bool index_ready = false);
 
 // tcgen05 forms of the pre-LLM Grams (bf16), used by the launchers above
-bool crit_gram_tc_supported(const SimArgs& a);
-// K splits of the tcgen05 text Gram (0: not applicable); G holds that many
-// [B][N_t_max][N_t_max] parts (at least one)
-constexpr int kCritMaxSplits = 16;
-int crit_splits(int N_t_max, int D, int dtype);
-cudaError_t crit_gram_tc_launch(const SimArgs& a, float* G, cudaStream_t s);
+// the text Gram into G (bf16), or, up to 128 text rows (*whole), the mask and r at once
+cudaError_t crit_gram_tc_launch(const SimArgs& a, uint8_t* mask, float* r_out, float* G, int num_sms, bool* whole,
+                                cudaStream_t s);
 bool relevance_tc_supported(const SimArgs& a);
 // workspace floats of the tensor-core relevance (cosines + per-tile sums)
 size_t relevance_fused_floats(int B, int N_v, int N_t_max);

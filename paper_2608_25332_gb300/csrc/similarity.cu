@@ -25,26 +25,25 @@ __device__ __forceinline__ const T* row_ptr(const void* base, size_t row, int D)
 // ---------------------------------------------------------------------------
 // Sec. 4.2
 // ---------------------------------------------------------------------------
-template <typename T>
 __global__ void __launch_bounds__(256) crit_gram_kernel(const SimArgs a, float* G) {
   __shared__ __align__(16) SimtSmem sm;
-  __shared__ const T* arow[kSimtBM];
-  __shared__ const T* brow[kSimtBN];
+  __shared__ const float* arow[kSimtBM];
+  __shared__ const float* brow[kSimtBN];
   const int b = blockIdx.z;
   const int r0 = blockIdx.y * kSimtBM, c0 = blockIdx.x * kSimtBN;
   int tl = a.text_len[b];
   if (tl < 0 || tl > a.N_t_max) tl = 0;
   if (threadIdx.x < kSimtBM) {
     const int j = r0 + threadIdx.x;
-    arow[threadIdx.x] = j < tl ? row_ptr<T>(a.emb_t, (size_t)b * a.N_t_max + j, a.D) : nullptr;
+    arow[threadIdx.x] = j < tl ? row_ptr<float>(a.emb_t, (size_t)b * a.N_t_max + j, a.D) : nullptr;
   }
   if (threadIdx.x < kSimtBN) {
     const int j = c0 + threadIdx.x;
-    brow[threadIdx.x] = j < tl ? row_ptr<T>(a.emb_t, (size_t)b * a.N_t_max + j, a.D) : nullptr;
+    brow[threadIdx.x] = j < tl ? row_ptr<float>(a.emb_t, (size_t)b * a.N_t_max + j, a.D) : nullptr;
   }
   __syncthreads();
   float acc[8][4];
-  simt_gemm_nt<T>(arow, brow, a.D, sm, acc);
+  simt_gemm_nt<float>(arow, brow, a.D, sm, acc);
   const int rg = threadIdx.x >> 4, kg = threadIdx.x & 15;
 #pragma unroll
   for (int i = 0; i < 8; ++i)
@@ -55,128 +54,122 @@ __global__ void __launch_bounds__(256) crit_gram_kernel(const SimArgs a, float* 
     }
 }
 
-// one CTA per sample: row softmax statistics, column means r, threshold
-// Adds the K parts of the text Gram into part 0, in part order: one thread per
-// element, every part's load issued first.
-constexpr int kCritMaxParts = 16;
-__global__ void __launch_bounds__(256) crit_parts_sum_kernel(float* G, size_t n, int n_parts) {
-  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n) return;
-  float v[kCritMaxParts];
-#pragma unroll
-  for (int q = 0; q < kCritMaxParts; ++q)
-    if (q < n_parts) v[q] = G[q * n + e];
-  float s = v[0];
-#pragma unroll
-  for (int q = 1; q < kCritMaxParts; ++q)
-    if (q < n_parts) s += v[q];
-  G[e] = s;
+// From the sample Grams G [B][Ntm][Ntm]: row softmax, column means r, threshold
+// (the CUDA-core Gram's, and the tensor-core Gram's past 128 text rows). A cluster
+// of kFinishCtas CTAs per sample, a row per warp at a time, the rows dealt to the
+// warps of the cluster in turn: lane l takes columns l, l + 32, .., which stay in
+// registers (kReg of them) up to 32 kReg text rows, else the row is read three
+// times (from L1). A warp adds its rows' softmax per column, then the warps, then
+// the CTAs are added in order. One CTA of 1024 threads per sample took 34 us for
+// 300 text rows.
+constexpr int kFinishCtas = 8;
+constexpr int kFinishWarps = 8;
+constexpr size_t finish_smem(int N_t_max) { return (size_t)(kFinishWarps + 2) * N_t_max * sizeof(float); }
+__device__ __forceinline__ void finish_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
+               "barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-
-// G: the sample Grams [B][Ntm][Ntm]. Up to kFinishSmemNt text rows the sample's
-// Gram is staged in shared memory. One CTA of 1024 threads per sample: a warp
-// per row for the softmax statistics, then the column sums of the softmax in
-// kFinishThreads / n row groups whose partial sums are added in group order.
-constexpr int kFinishSmemNt = 128;
-constexpr int kFinishThreads = 1024;
-__global__ void __launch_bounds__(kFinishThreads) crit_finish_kernel(const SimArgs a, const float* G,
-                                                                     uint8_t* mask, float* r_out) {
-  // rowm[Ntm], rowinv[Ntm], r[Ntm], part[kFinishThreads] (+ G[Ntm][Ntm] when staged)
-  extern __shared__ float sh[];
-  float* rowm = sh;
-  float* rowinv = sh + a.N_t_max;
-  float* rr = sh + 2 * a.N_t_max;
-  float* part = sh + 3 * a.N_t_max;
-  __shared__ float wsum[kFinishThreads / 32];
-  __shared__ int wcnt[kFinishThreads / 32];
-  constexpr int kWarps = kFinishThreads / 32;
-  const int b = blockIdx.x;
+template <int kReg>
+__global__ void __launch_bounds__(32 * kFinishWarps) crit_finish_kernel(const SimArgs a, const float* G,
+                                                                        uint8_t* mask, float* r_out) {
+  extern __shared__ float sh[];  // part[kFinishWarps][Ntm], col[Ntm], rr[Ntm]
+  float* col = sh + (size_t)kFinishWarps * a.N_t_max;
+  float* rr = col + a.N_t_max;
+  __shared__ float wsum[kFinishWarps];
+  __shared__ int wcnt[kFinishWarps];
+  const int rank = blockIdx.x, b = blockIdx.y;  // the cluster spans grid x
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int n = a.text_len[b];
   if (n < 0 || n > a.N_t_max) {
-    if (threadIdx.x == 0) set_error(a.err, kErrBadDeviceArg);
+    if (rank == 0 && threadIdx.x == 0) set_error(a.err, kErrBadDeviceArg);
     n = 0;
   }
   const float* Gb = G + (size_t)b * a.N_t_max * a.N_t_max;
-  const bool staged = a.N_t_max <= kFinishSmemNt;
-  float* Gs = part + kFinishThreads;
-  int ld = a.N_t_max;
-  if (staged) {
-    // eight loads in flight per thread
-    for (int e0 = 0; e0 < n * n; e0 += 8 * (int)blockDim.x) {
-      float v[8];
+  float* part = sh + (size_t)warp * a.N_t_max;
+  const int i0 = rank * kFinishWarps + warp;
+  if constexpr (kReg > 0) {
+    float acc[kReg];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int e = e0 + u * (int)blockDim.x + (int)threadIdx.x;
-        if (e < n * n) v[u] = Gb[(size_t)(e / n) * a.N_t_max + (e - (e / n) * n)];
-      }
+    for (int q = 0; q < kReg; ++q) acc[q] = 0.f;
+    for (int i = i0; i < n; i += kFinishCtas * kFinishWarps) {
+      float v[kReg], m = -INFINITY, z = 0.f;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int e = e0 + u * (int)blockDim.x + (int)threadIdx.x;
-        if (e < n * n) Gs[e] = v[u];
+      for (int q = 0; q < kReg; ++q) v[q] = lane + 32 * q < n ? Gb[(size_t)i * a.N_t_max + lane + 32 * q] : 0.f;
+#pragma unroll
+      for (int q = 0; q < kReg; ++q)
+        if (lane + 32 * q < n) m = fmaxf(m, v[q]);
+      m = warp_max(m);
+#pragma unroll
+      for (int q = 0; q < kReg; ++q) {
+        v[q] = lane + 32 * q < n ? expf(v[q] - m) : 0.f;
+        z += v[q];
       }
+      const float inv = 1.f / warp_sum(z);
+#pragma unroll
+      for (int q = 0; q < kReg; ++q) acc[q] += v[q] * inv;
     }
-    __syncthreads();
-    Gb = Gs;
-    ld = n;
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int i = warp; i < n; i += kWarps) {
-    float m = -INFINITY;
-    for (int j = lane; j < n; j += 32) m = fmaxf(m, Gb[(size_t)i * ld + j]);
-    m = warp_max(m);
-    float z = 0.f;
-    for (int j = lane; j < n; j += 32) z += expf(Gb[(size_t)i * ld + j] - m);
-    z = warp_sum(z);
-    if (lane == 0) {
-      rowm[i] = m;
-      rowinv[i] = 1.f / z;
+#pragma unroll
+    for (int q = 0; q < kReg; ++q)
+      if (lane + 32 * q < n) part[lane + 32 * q] = acc[q];
+  } else {
+    for (int j = lane; j < n; j += 32) part[j] = 0.f;
+    for (int i = i0; i < n; i += kFinishCtas * kFinishWarps) {
+      const float* row = Gb + (size_t)i * a.N_t_max;
+      float m = -INFINITY, z = 0.f;
+      for (int j = lane; j < n; j += 32) m = fmaxf(m, row[j]);
+      m = warp_max(m);
+      for (int j = lane; j < n; j += 32) z += expf(row[j] - m);
+      const float inv = 1.f / warp_sum(z);
+      for (int j = lane; j < n; j += 32) part[j] += expf(row[j] - m) * inv;
     }
   }
   __syncthreads();
-  if (n > 0 && n <= kFinishThreads) {
-    // column j of row group g: rows g, g + groups, ... (in order)
-    const int groups = kFinishThreads / n;
-    const int g = threadIdx.x / n, j = threadIdx.x - g * n;
-    if (g < groups) {
-      float s = 0.f;
-      for (int i = g; i < n; i += groups) s += expf(Gb[(size_t)i * ld + j] - rowm[i]) * rowinv[i];
-      part[g * n + j] = s;
-    }
-    __syncthreads();
-    for (int jj = threadIdx.x; jj < n; jj += blockDim.x) {
-      float s = 0.f;
-      for (int g2 = 0; g2 < groups; ++g2) s += part[g2 * n + jj];
-      rr[jj] = s / (float)n;
-    }
-  } else {
+  for (int j = threadIdx.x; j < n; j += blockDim.x) {
+    float s = 0.f;
+#pragma unroll
+    for (int w = 0; w < kFinishWarps; ++w) s += sh[(size_t)w * a.N_t_max + j];
+    col[j] = s;
+  }
+  finish_cluster_sync();  // every CTA's column sums
+  if (rank == 0) {
+    float pt = 0.f;
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
       float s = 0.f;
-      for (int i = 0; i < n; ++i) s += expf(Gb[(size_t)i * ld + j] - rowm[i]) * rowinv[i];
+#pragma unroll
+      for (int q = 0; q < kFinishCtas; ++q) {
+        uint32_t addr;
+        float v;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(smem_u32(col + j)), "r"(q));
+        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+        s += v;
+      }
       rr[j] = s / (float)n;
+      pt += rr[j];
+    }
+    // mean(r), fixed-order block sum
+    pt = warp_sum(pt);
+    if (lane == 0) wsum[warp] = pt;
+    __syncthreads();
+    float tot = 0.f;
+#pragma unroll
+    for (int w = 0; w < kFinishWarps; ++w) tot += wsum[w];
+    const float mean = n > 0 ? tot / (float)n : 0.f;
+    int c = 0;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) c += rr[j] > mean;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if (lane == 0) wcnt[warp] = c;
+    __syncthreads();
+    int cnt = 0;
+#pragma unroll
+    for (int w = 0; w < kFinishWarps; ++w) cnt += wcnt[w];
+    for (int j = threadIdx.x; j < a.N_t_max; j += blockDim.x) {
+      const bool in = j < n && (cnt == 0 || rr[j] > mean);
+      mask[(size_t)b * a.N_t_max + j] = in ? 1 : 0;
+      if (r_out) r_out[(size_t)b * a.N_t_max + j] = j < n ? rr[j] : 0.f;
     }
   }
-  __syncthreads();
-  // mean(r), fixed-order block sum
-  float pt = 0.f;
-  for (int j = threadIdx.x; j < n; j += blockDim.x) pt += rr[j];
-  pt = warp_sum(pt);
-  if (lane == 0) wsum[warp] = pt;
-  __syncthreads();
-  float tot = 0.f;
-  for (int w = 0; w < kWarps; ++w) tot += wsum[w];
-  const float mean = n > 0 ? tot / (float)n : 0.f;
-  int c = 0;
-  for (int j = threadIdx.x; j < n; j += blockDim.x) c += rr[j] > mean;
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  if (lane == 0) wcnt[warp] = c;
-  __syncthreads();
-  int cnt = 0;
-  for (int w = 0; w < kWarps; ++w) cnt += wcnt[w];
-  for (int j = threadIdx.x; j < a.N_t_max; j += blockDim.x) {
-    const bool in = j < n && (cnt == 0 || rr[j] > mean);
-    mask[(size_t)b * a.N_t_max + j] = in ? 1 : 0;
-    if (r_out) r_out[(size_t)b * a.N_t_max + j] = j < n ? rr[j] : 0.f;
-  }
+  finish_cluster_sync();  // no CTA leaves while CTA 0 may still read its column sums
 }
 
 // ---------------------------------------------------------------------------
@@ -927,38 +920,40 @@ __global__ void __launch_bounds__(C::kThreads, C::kMinBlocks)
 
 }  // namespace
 
-cudaError_t crit_text_launch(const SimArgs& a, uint8_t* mask, float* r_out, float* G,
+cudaError_t crit_text_launch(const SimArgs& a, uint8_t* mask, float* r_out, float* G, int num_sms,
                              cudaStream_t s) {
-  dim3 g((a.N_t_max + kSimtBN - 1) / kSimtBN, (a.N_t_max + kSimtBM - 1) / kSimtBM, a.B);
-  int parts = 1;
   if (a.dtype == 0) {
-    crit_gram_kernel<float><<<g, 256, 0, s>>>(a, G);
-  } else if (crit_gram_tc_supported(a)) {
-    cudaError_t e = crit_gram_tc_launch(a, G, s);
-    if (e != cudaSuccess) return e;
-    parts = crit_splits(a.N_t_max, a.D, a.dtype);
-    static_assert(kCritMaxSplits <= kCritMaxParts, "text Gram parts");
-    const size_t n = (size_t)a.B * a.N_t_max * a.N_t_max;
-    if (parts > 1) crit_parts_sum_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(G, n, parts);
+    dim3 g((a.N_t_max + kSimtBN - 1) / kSimtBN, (a.N_t_max + kSimtBM - 1) / kSimtBM, a.B);
+    crit_gram_kernel<<<g, 256, 0, s>>>(a, G);
   } else {
-    crit_gram_kernel<__nv_bfloat16><<<g, 256, 0, s>>>(a, G);
+    bool whole = false;
+    cudaError_t e = crit_gram_tc_launch(a, mask, r_out, G, num_sms, &whole, s);
+    if (e != cudaSuccess || whole) return e;
   }
   static std::atomic<bool> configured[64];  // per device, zero-initialised
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !configured[dev]) {
-    const int lim = (3 * kFinishSmemNt + kFinishThreads + kFinishSmemNt * kFinishSmemNt) * (int)sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(crit_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaError_t e = cudaFuncSetAttribute(crit_finish_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)finish_smem(kCritMaxNt));
     if (e != cudaSuccess) return e;
     configured[dev] = true;
   }
-  size_t smem = (3 * (size_t)a.N_t_max + kFinishThreads) * sizeof(float);
-  if (a.N_t_max <= kFinishSmemNt) smem += (size_t)a.N_t_max * a.N_t_max * sizeof(float);
-  if (smem > (size_t)(3 * kFinishSmemNt + kFinishThreads + kFinishSmemNt * kFinishSmemNt) * sizeof(float))
-    return cudaErrorInvalidValue;  // N_t_max beyond what the shared-memory layout holds
-  (void)parts;
-  crit_finish_kernel<<<a.B, kFinishThreads, smem, s>>>(a, G, mask, r_out);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  cfg.gridDim = dim3(kFinishCtas, (unsigned)a.B);
+  cfg.blockDim = dim3(32 * kFinishWarps);
+  cfg.dynamicSmemBytes = finish_smem(a.N_t_max);
+  cfg.stream = s;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kFinishCtas;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (a.N_t_max <= 32 * 4) return cudaLaunchKernelEx(&cfg, crit_finish_kernel<4>, a, G, mask, r_out);
+  if (a.N_t_max <= 32 * 16) return cudaLaunchKernelEx(&cfg, crit_finish_kernel<16>, a, G, mask, r_out);
+  return cudaLaunchKernelEx(&cfg, crit_finish_kernel<0>, a, G, mask, r_out);
 }
 
 // 1/|e_j| (0 for a zero row) of the kept rows j = keep_idx[b][q] only, into

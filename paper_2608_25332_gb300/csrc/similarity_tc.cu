@@ -13,7 +13,8 @@
 //   tile, one read of the visual rows giving |v_j|^2 (the diagonal of the
 //   visual block), the cosines and the de-meaning sums (p_j itself is formed by
 //   a small second kernel once every tile's sums are known).
-// crit_gram_tc: the text Gram E_t E_t^T, split over K.
+// crit_gram_tc: the text Gram E_t E_t^T, split over K in a cluster, and up to 128
+//   text rows the whole of Sec. 4.2 in the same kernel.
 #include "common.cuh"
 #include "kernels.h"
 #include "merge_epi.cuh"
@@ -562,66 +563,264 @@ __global__ void __launch_bounds__(256) relevance_finish_kernel(const RelFusedArg
   }
 }
 
-// G = E_t E_t^T for one sample (<= 128 text rows), split over K: CTA x of
-// sample b sums the K slices [x * ks_per, (x + 1) * ks_per) and writes its part
-// to G[x][b] as fp32; the softmax/column-mean step of Sec. 4.2 adds the parts
-// in split order.
-constexpr int kCritBN = 128;
+// The text Gram G = E_t E_t^T (Sec. 4.2): a cluster of C CTAs per 128 x 128 tile
+// of a sample, each summing its share of the K slices in A of C x A accumulators
+// (C x A = 16 parts: the sums are bound by the latency of a few small loads, so
+// they are spread over CTAs, and short accumulation chains keep them exact to a
+// few ulp). Each CTA adds its accumulators in order, puts the tile part in its
+// shared memory and frees its tensor memory (before it waits for its peers, so
+// that a CTA holding tensor memory never waits for one that wants it); then CTA
+// c adds rows [c * 128 / C, ..) of the C parts in order over distributed shared
+// memory.
+// kWhole (at most 128 text rows: one tile): the rows are complete where they
+// were added, so the same kernel goes on to their softmax (a warp per row), the
+// column sums (rows of a warp, then warps, then CTAs, in order) and, in CTA 0,
+// the mean and the mask. With the parts in global memory, added by a second
+// kernel and finished by a third on one CTA per sample, the chain took
+// 14 + 3 + 10 us for 8 samples of 96 rows and 29 + 5 + 14 for 16 of 128, longer
+// than the relevance Gram it runs beside (the pre-LLM pass: 192 -> 185 us for a
+// video, 275 -> 257 for the schedule of 16 images). Past 128 text rows the FFMA
+// Gram took 330 us for 4 samples of 300 rows and the finish 34: the pass of
+// that batch went from 605 to 148 us.
+// Otherwise the rows go to G and crit_finish_kernel follows.
+struct CritArgs {
+  const int* text_len;
+  int N_t_max, n_k;
+  int nt;          // 128-row tiles per side
+  int n_acc;       // accumulators per CTA
+  float* G;        // [B][N_t_max][N_t_max]; unused with kWhole
+  uint8_t* mask;   // kWhole: the outputs
+  float* r_out;
+  unsigned* err;
+};
+constexpr int kCritStages = 4;
+constexpr int kCritMaxAcc = 4;
+constexpr int kCritLd = kBM + 4;  // padded row of the tile part in shared memory
+constexpr int kCritMaxCluster = 8;
 
+struct CritPipe {
+  uint64_t full[kCritStages];
+  uint64_t empty[kCritStages];
+  uint64_t acc_full;
+  uint32_t tmem;
+  volatile int fail;
+};
+
+__device__ __forceinline__ void crit_cluster_sync() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
+               "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t peer_addr(const void* local, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(local)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ float4 ld_peer_f4(const float* local, uint32_t rank) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(peer_addr(local, rank))
+               : "memory");
+  return v;
+}
+
+template <bool kWhole>
 __global__ void __launch_bounds__(kThreads, 1)
-    crit_gram_tc(const __grid_constant__ CUtensorMap mapT, const int* text_len, int N_t_max, int D,
-                 int B, int ks_per, float* G, unsigned* err) {
+    crit_gram_tc(const CritArgs a, const __grid_constant__ CUtensorMap mapT) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ Pipe pipe;
-  const int b = blockIdx.z;
-  const int k0 = blockIdx.x * ks_per;
-  const int n_k = min(ks_per, (D + kBK - 1) / kBK - k0);
+  __shared__ CritPipe pipe;
+  __shared__ __align__(16) float wcol[kThreads / 32][kBM];
+  __shared__ __align__(16) float ccol[kBM];
+  __shared__ float wsum[4];
+  __shared__ int wcnt[4];
+  const uint32_t rank = blockIdx.x, C = gridDim.x;  // the cluster spans grid x
+  const int ti = blockIdx.y / a.nt, tj = blockIdx.y % a.nt, b = blockIdx.z;
+  const bool same = ti == tj;  // one load per K slice is both operands
+  const int k0 = (int)((long long)a.n_k * rank / C), n = (int)((long long)a.n_k * (rank + 1) / C) - k0;
+  const int n_acc = min(a.n_acc, n);  // n >= 1: C <= n_k
   const uint32_t sbase = smem_u32(smem_raw);
   uint8_t* stages = smem_raw + (((sbase + 1023u) & ~1023u) - sbase);
+  constexpr uint32_t kStage = kWhole ? kABytes : 2 * kABytes;
+  const uint32_t cols = (uint32_t)a.n_acc * kBM;
   if (threadIdx.x == 0) {
     prefetch_tmap(&mapT);
-    pipe_init(pipe);
+    for (int s = 0; s < kCritStages; ++s) {
+      mbar_init(&pipe.full[s], 1);
+      mbar_init(&pipe.empty[s], 1);
+    }
+    mbar_init(&pipe.acc_full, 1);
+    pipe.fail = 0;
+    fence_mbar_init();
   }
   if (threadIdx.x < 32) {
-    tmem_alloc(&pipe.tmem, Cfg<kCritBN>::kTmemCols);
+    tmem_alloc(&pipe.tmem, cols);
     tmem_relinquish();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float* tile = reinterpret_cast<float*>(stages);  // [128][kCritLd], once the MMAs are done
   if (warp == 0) {
     if (lane == 0) {
-      RowSrc ra{b * N_t_max, kBM};
-      RowSrc rb{b * N_t_max, kCritBN};
-      // both operands are the same text rows: one load per K slice
-      producer<kCritBN>(pipe, stages, &mapT, &mapT, ra, rb, 1, n_k, err, k0, true);
+      for (int i = 0; i < n; ++i) {
+        const int s = i % kCritStages;
+        if (pipe.fail || !mbar_wait(&pipe.empty[s], ((uint32_t)(i / kCritStages) & 1u) ^ 1u, a.err)) {
+          pipe.fail = 1;
+          break;
+        }
+        uint8_t* sa = stages + (size_t)s * kStage;
+        mbar_arrive_expect_tx(&pipe.full[s], same ? kABytes : 2 * kABytes);
+        tma_load_2d(sa, &mapT, (k0 + i) * kBK, b * a.N_t_max + ti * kBM, &pipe.full[s]);
+        if (!same) tma_load_2d(sa + kABytes, &mapT, (k0 + i) * kBK, b * a.N_t_max + tj * kBM, &pipe.full[s]);
+      }
     }
   } else if (warp == 1) {
-    if (lane == 0) mma_issuer<kCritBN>(pipe, stages, 1, n_k, err, true);
+    if (lane == 0) {
+      int q = -1;
+      for (int i = 0; i < n; ++i) {
+        const int s = i % kCritStages;
+        if (pipe.fail || !mbar_wait(&pipe.full[s], (uint32_t)(i / kCritStages) & 1u, a.err)) {
+          pipe.fail = 1;
+          break;
+        }
+        tc_fence_after();
+        const bool first = q != i * n_acc / n;  // the accumulator's first slice
+        q = i * n_acc / n;
+        const uint32_t sa = smem_u32(stages + (size_t)s * kStage);
+        const uint32_t sb = same ? sa : sa + kABytes;
+#pragma unroll
+        for (int k = 0; k < kBK / 16; ++k)
+          tc_mma_bf16(pipe.tmem + (uint32_t)q * kBM, smem_desc_sw128(sa + k * 32), smem_desc_sw128(sb + k * 32),
+                      idesc_bf16_f32(kBM, kBM), (!first || k > 0) ? 1u : 0u);
+        tc_commit(&pipe.empty[s]);
+      }
+      tc_commit(&pipe.acc_full);  // arrives once every MMA above has completed
+    }
   } else {
     const int quad = warp & 3;
     const int r = quad * 32 + lane;
-    mbar_wait(&pipe.acc_full[0], 0, err);
+    warp_mbar_wait(&pipe.acc_full, 0, a.err);
     tc_fence_after();
     const uint32_t taddr = pipe.tmem + ((uint32_t)(quad * 32) << 16);
-    float* g = G + (((size_t)blockIdx.x * B + b) * N_t_max + r) * N_t_max;
 #pragma unroll 1
-    for (int cb = 0; cb < kCritBN / 32; ++cb) {
+    for (int cb = 0; cb < kBM / 32; ++cb) {
       float v[32];
       tmem_ld32(taddr + cb * 32, v);
-      tc_wait_ld();
-      if (r < N_t_max && !pipe.fail) {
+      tc_wait_ld_into(v);
+#pragma unroll 1
+      for (int q = 1; q < n_acc; ++q) {
+        float w[32];
+        tmem_ld32(taddr + (uint32_t)q * kBM + cb * 32, w);
+        tc_wait_ld_into(w);
 #pragma unroll
-        for (int i = 0; i < 32; ++i)
-          if (cb * 32 + i < N_t_max) g[cb * 32 + i] = v[i];
+        for (int i = 0; i < 32; ++i) v[i] += w[i];
       }
+#pragma unroll
+      for (int i = 0; i < 32; i += 4)
+        *reinterpret_cast<float4*>(tile + (size_t)r * kCritLd + cb * 32 + i) =
+            make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
     }
-    tc_fence_before();
   }
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x < 32) tmem_dealloc(pipe.tmem, Cfg<kCritBN>::kTmemCols);
+  if (threadIdx.x < 32) tmem_dealloc(pipe.tmem, cols);
+  crit_cluster_sync();  // every part of the tile is in its CTA's shared memory
+
+  const int n_rows = kBM / (int)C;  // rows that this CTA adds and owns
+  // row i of its share, columns [4 lane, 4 lane + 4): the parts in order
+  auto gram4 = [&](int i) {
+    const float* src = tile + (size_t)((int)rank * n_rows + i) * kCritLd + lane * 4;
+    float4 v[kCritMaxCluster];
+#pragma unroll
+    for (uint32_t q = 0; q < kCritMaxCluster; ++q)
+      if (q < C) v[q] = ld_peer_f4(src, q);
+    float4 g = v[0];
+#pragma unroll
+    for (uint32_t q = 1; q < kCritMaxCluster; ++q)
+      if (q < C) {
+        g.x += v[q].x;
+        g.y += v[q].y;
+        g.z += v[q].z;
+        g.w += v[q].w;
+      }
+    return g;
+  };
+  if (!kWhole) {
+    for (int i = warp; i < n_rows; i += kThreads / 32) {
+      const float4 g = gram4(i);
+      const int row = ti * kBM + (int)rank * n_rows + i, col = tj * kBM + lane * 4;
+      if (row < a.N_t_max && !pipe.fail) {
+        float* o = a.G + ((size_t)b * a.N_t_max + row) * a.N_t_max + col;
+        const float ge[4] = {g.x, g.y, g.z, g.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (col + e < a.N_t_max) o[e] = ge[e];
+      }
+    }
+    crit_cluster_sync();  // no CTA leaves while a peer may still read its part
+    return;
+  }
+  int tl = a.text_len[b];
+  if (tl < 0 || tl > a.N_t_max) {
+    if (rank == 0 && threadIdx.x == 0) set_error(a.err, kErrBadDeviceArg);
+    tl = 0;
+  }
+  float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int c0 = lane * 4;
+  for (int i = warp; i < n_rows; i += kThreads / 32) {
+    if ((int)rank * n_rows + i >= tl) break;  // warp-uniform
+    const float4 g = gram4(i);
+    const float gv[4] = {c0 < tl ? g.x : -INFINITY, c0 + 1 < tl ? g.y : -INFINITY,
+                         c0 + 2 < tl ? g.z : -INFINITY, c0 + 3 < tl ? g.w : -INFINITY};
+    const float m = warp_max(fmaxf(fmaxf(gv[0], gv[1]), fmaxf(gv[2], gv[3])));
+    float e[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) e[q] = c0 + q < tl ? expf(gv[q] - m) : 0.f;
+    const float inv = 1.f / warp_sum((e[0] + e[1]) + (e[2] + e[3]));
+    cs.x += e[0] * inv;
+    cs.y += e[1] * inv;
+    cs.z += e[2] * inv;
+    cs.w += e[3] * inv;
+  }
+  *reinterpret_cast<float4*>(&wcol[warp][c0]) = cs;
+  __syncthreads();
+  const int j = threadIdx.x;
+  if (j < kBM) {
+    float s = 0.f;
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w) s += wcol[w][j];
+    ccol[j] = s;
+  }
+  crit_cluster_sync();  // every CTA's column sums
+  float r = 0.f;
+  if (rank == 0) {
+    if (j < kBM) {
+      for (uint32_t q = 0; q < C; ++q) {
+        float v;
+        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(peer_addr(&ccol[j], q)) : "memory");
+        r += v;
+      }
+      r = j < tl ? r / (float)tl : 0.f;
+      const float s = warp_sum(r);
+      if (lane == 0) wsum[warp] = s;
+    }
+    __syncthreads();
+    const float mean = tl > 0 ? ((wsum[0] + wsum[1]) + (wsum[2] + wsum[3])) / (float)tl : 0.f;
+    const bool over = j < tl && r > mean;
+    if (j < kBM) {
+      const unsigned bal = __ballot_sync(0xffffffffu, over);
+      if (lane == 0) wcnt[warp] = __popc(bal);
+    }
+    __syncthreads();
+    const int cnt = (wcnt[0] + wcnt[1]) + (wcnt[2] + wcnt[3]);
+    if (j < a.N_t_max) {
+      a.mask[(size_t)b * a.N_t_max + j] = (j < tl && (cnt == 0 || over)) ? 1 : 0;
+      if (a.r_out) a.r_out[(size_t)b * a.N_t_max + j] = r;
+    }
+  }
+  crit_cluster_sync();  // no CTA leaves while CTA 0 may still read its column sums
 }
 
 template <typename K>
@@ -793,33 +992,52 @@ cudaError_t relevance_tc_launch(const SimArgs& a, const uint8_t* mask, const flo
 
 namespace provip {
 
-bool crit_gram_tc_supported(const SimArgs& a) { return crit_splits(a.N_t_max, a.D, a.dtype) > 0; }
-
-// K parts of the text Gram: 0 when the tcgen05 form does not apply; every part
-// owns ceil(n_k / parts) slices of 64 (the last one possibly fewer)
-int crit_splits(int N_t_max, int D, int dtype) {
-  if (dtype != 1 || N_t_max > kBM || D % 8) return 0;
-  const int n_k = (D + kBK - 1) / kBK;
-  const int ns = n_k < kCritMaxSplits ? n_k : kCritMaxSplits;
-  const int per = (n_k + ns - 1) / ns;
-  return (n_k + per - 1) / per;
-}
-
-cudaError_t crit_gram_tc_launch(const SimArgs& a, float* G, cudaStream_t s) {
-  static std::atomic<bool> smem_set[64];  // per device, zero-initialised
+// CTAs per tile and accumulators per CTA: 8 x 2 while the clusters fit the SMs at
+// one CTA each, 4 x 4 beyond (the same 16 parts with fewer, longer CTAs); narrow
+// embeddings with fewer K slices take the largest power of two of them.
+cudaError_t crit_gram_tc_launch(const SimArgs& a, uint8_t* mask, float* r_out, float* G, int num_sms, bool* whole,
+                                cudaStream_t s) {
+  static std::atomic<bool> smem_set[64], smem_set2[64];  // per device, zero-initialised
   int dev = 0;
   cudaGetDevice(&dev);
-  const size_t smem = Cfg<kCritBN>::kStagesBytes + 1024;
-  cudaError_t e = set_smem(crit_gram_tc, smem, &smem_set[dev < 64 ? dev : 0]);
+  constexpr size_t kTileBytes = (size_t)kBM * kCritLd * sizeof(float);
+  constexpr size_t kWholeBytes = (size_t)kCritStages * kABytes;
+  constexpr size_t smem1 = (kWholeBytes > kTileBytes ? kWholeBytes : kTileBytes) + 1024;
+  constexpr size_t smem2 = (size_t)kCritStages * 2 * kABytes + 1024;
+  static_assert(smem2 >= kTileBytes + 1024, "the tile part fits the stages");
+  cudaError_t e = set_smem(crit_gram_tc<true>, smem1, &smem_set[dev < 64 ? dev : 0]);
+  if (e == cudaSuccess) e = set_smem(crit_gram_tc<false>, smem2, &smem_set2[dev < 64 ? dev : 0]);
   if (e != cudaSuccess) return e;
   CUtensorMap mapT;
   if (make_tmap_bf16_2d(&mapT, a.emb_t, (uint64_t)a.B * a.N_t_max, (uint64_t)a.D, (uint64_t)a.D * 2, 128))
     return cudaErrorInvalidValue;
-  const int parts = crit_splits(a.N_t_max, a.D, a.dtype);
-  const int n_k = (a.D + kBK - 1) / kBK, per = (n_k + parts - 1) / parts;
-  crit_gram_tc<<<dim3(parts, 1, a.B), kThreads, smem, s>>>(mapT, a.text_len, a.N_t_max, a.D, a.B, per, G,
-                                                          a.err);
-  return cudaGetLastError();
+  CritArgs c;
+  c.text_len = a.text_len;
+  c.N_t_max = a.N_t_max;
+  c.n_k = (a.D + kBK - 1) / kBK;
+  c.nt = (a.N_t_max + kBM - 1) / kBM;
+  c.G = G;
+  c.mask = mask;
+  c.r_out = r_out;
+  c.err = a.err;
+  *whole = c.nt == 1;
+  int C = (long long)a.B * c.nt * c.nt * kCritMaxCluster <= num_sms ? kCritMaxCluster : kCritMaxAcc;
+  while (C > c.n_k) C /= 2;
+  c.n_acc = C == kCritMaxCluster ? 2 : kCritMaxAcc;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  cfg.gridDim = dim3((unsigned)C, (unsigned)(c.nt * c.nt), (unsigned)a.B);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = *whole ? smem1 : smem2;
+  cfg.stream = s;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)C;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return *whole ? cudaLaunchKernelEx(&cfg, crit_gram_tc<true>, c, mapT)
+                : cudaLaunchKernelEx(&cfg, crit_gram_tc<false>, c, mapT);
 }
 
 }  // namespace provip

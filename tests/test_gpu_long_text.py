@@ -7,7 +7,7 @@ import torch
 
 import oracle
 from paper_2608_25332_gb300 import provip as P
-from parity import assert_close_rel
+from parity import assert_close_rel, check_mask_band
 
 pytestmark = pytest.mark.gpu
 
@@ -54,3 +54,37 @@ def test_relevance_of_long_text(N_v, D, tls):
         ref = oracle.relevance(et[b, :t].double().numpy(), mask[b, :t], ev[b].double().numpy())
         # fp32 sums of at most 1096 exact products: far inside the pass's 2e-3
         assert_close_rel(got, ref, 0.0, f"p N_v={N_v} D={D} tls={tls} [{b}]", atol=1e-5)
+
+
+@pytest.mark.parametrize("dtype,D,tls", [
+    ("bf16", 64, (1, 5, 128)),               # one K slice: a cluster of one CTA
+    ("bf16", 264, (17, 0, 33)),              # five slices over four CTAs
+    ("bf16", 520, (100,)),                   # nine slices over eight CTAs, a partial last one
+    ("bf16", 4096, (96, 128, 31)),           # 8 CTAs of two accumulators
+    ("bf16", 1024, tuple(range(100, 140))),  # 2 x 2 tiles, 4 CTAs of four accumulators
+    ("bf16", 1024, tuple(range(60, 90))),    # one tile, 4 CTAs of four accumulators
+    ("bf16", 72, (129, 257, 1)),
+    ("bf16", 256, (513, 40)),                # past the columns held in registers
+    ("f32", 64, (1, 128, 40)),
+    ("f32", 264, (129, 511)),
+    ("f32", 64, (700, 513)),
+])
+def test_critical_rows(dtype, D, tls):
+    rng = np.random.default_rng(D + len(tls))
+    B, T = len(tls), max(tls)
+    # text logits at the scale of LLM token embeddings: a smooth softmax
+    et = torch.from_numpy((rng.standard_normal((B, T, D)) * 0.25 / D ** 0.25).astype(np.float32))
+    et = et.to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    for b, t in enumerate(tls):
+        et[b, t:] = float("nan")
+    mask, r = P.provip_crit_text(et.to(DEV), torch.tensor(tls, dtype=torch.int32, device=DEV), want_r=True)
+    torch.cuda.synchronize()
+    for b, t in enumerate(tls):
+        m, rr = mask[b].cpu().numpy(), r[b].cpu().numpy()
+        assert not m[t:].any() and not rr[t:].any()
+        if t == 0:
+            continue
+        r_ref, _ = oracle.crit_text(et[b, :t].double().numpy())
+        # logits of order 1 in fp32 sums (their exponentials a few ulp off)
+        assert_close_rel(rr[:t], r_ref, 1e-5, f"r {dtype} D={D} tls={tls} [{b}]")
+        check_mask_band(m[:t], r_ref, 1e-5, f"T {dtype} D={D} tls={tls} [{b}]")
