@@ -357,19 +357,6 @@ int rel_splits(int B, int N_v) {
   if (n > by_rows) n = by_rows;
   return n < 1 ? 1 : n;
 }
-int merge_splits(int B, int N_v, int keep) {
-  const int rows = ((N_v + 127) / 128) * B;
-  const int cols = (keep + 63) / 64;
-  int n = (512 + rows - 1) / rows;
-  if (n > cols) n = cols;
-  if (n > 16) n = 16;
-  return n < 1 ? 1 : n;
-}
-// rows of the per-split argmax workspace: enough for either merge path
-int merge_ws_splits(int B, int N_v, int keep) {
-  const int a = merge_splits(B, N_v, keep);
-  return a > kMergeMaxSplit ? a : kMergeMaxSplit;
-}
 
 struct SimWs {
   float* G = nullptr;
@@ -589,7 +576,7 @@ extern "C" int provip_topk(const float* scores, int B, int N, int k, int* idx_ou
 }
 
 static size_t merge_ws(Carve& c, int B, int N_v, int D, int keep, SimWs& w) {
-  const int ns = merge_ws_splits(B, N_v, keep);
+  const int ns = kMergeMaxSplit;  // rows of the argmax partials
   w.inv_v = c.take<float>((size_t)B * N_v);
   w.best = c.take<float>((size_t)ns * B * N_v);
   w.bidx = c.take<int>((size_t)ns * B * N_v);
@@ -633,8 +620,7 @@ extern "C" int provip_merge(const void* emb_v, int B, int N_v, int D, const int*
   cudaError_t e = kept_inv_norm_launch(a, keep_idx, keep, w.inv_v, s);
   if (e == cudaSuccess)
     e = merge_launch(a, keep_idx, keep, w.inv_v, assign_out, merged_out, w.best, w.bidx,
-                     merge_splits(B, N_v, keep), w.pruned, dtype == PROVIP_BF16 ? w.perm : nullptr,
-                     d->sms, s);
+                     w.pruned, dtype == PROVIP_BF16 ? w.perm : nullptr, d->sms, s);
   return e == cudaSuccess ? PROVIP_OK : cuda_fail(e, "merge launch");
 }
 
@@ -645,7 +631,7 @@ static size_t simred_ws(Carve& c, int B, int N_v, int D, int N_t_max, int keep_p
   w.assign = c.take<int>((size_t)B * N_v);
   SimWs r;
   relevance_ws(c, B, N_v, D, N_t_max, r);
-  const int ns = merge_ws_splits(B, N_v, keep_pre);
+  const int ns = kMergeMaxSplit;  // rows of the argmax partials
   w.inv_v = r.inv_v;
   w.sum = r.sum;
   w.mu = r.mu;
@@ -733,8 +719,7 @@ extern "C" int provip_similarity_reduce(const void* emb_v, int B, int N_v, int D
   if (e == cudaSuccess && merged_out_or_null)
     e = merge_launch(a, idx_out, keep_pre, w.inv_v, assign_out_or_null ? assign_out_or_null : w.assign,
                      merged_out_or_null, w.best, w.bidx,
-                     merge_splits(B, N_v, keep_pre), w.pruned,
-                     dtype == PROVIP_BF16 ? w.perm : nullptr, d->sms, s, topk_writes_index(N_v));
+                     w.pruned, dtype == PROVIP_BF16 ? w.perm : nullptr, d->sms, s, topk_writes_index(N_v));
   return e == cudaSuccess ? PROVIP_OK : cuda_fail(e, "similarity_reduce launch");
 }
 

@@ -197,14 +197,14 @@ cudaError_t relevance_launch(const SimArgs& a, const uint8_t* mask, float* inv_v
                              int n_split, int num_sms, cudaStream_t s,
                              cudaEvent_t mask_ready = nullptr);
 // Sec. 4.3 merge: assign[b][j] and merged[b][a][:]
-// n_split: the SIMT split (sized by the caller); ws_pruned: [B][N_v] ints and
-// ws_perm: [B][N_v][D] bf16 for the tcgen05 path (null: CUDA-core path);
-// num_sms for its split choice
+// ws_best, ws_bidx: kMergeMaxSplit x [B][N_v]; ws_pruned: [B][N_v] ints; ws_perm:
+// [B][N_v][D] bf16 for the tcgen05 path (null: CUDA-core path); num_sms for the
+// split choices
 // index_ready: the kept-position map (in assign) and the pruned list (in
 // ws_pruned) were written by the top-k that chose keep_idx (topk_writes_index)
 cudaError_t merge_launch(const SimArgs& a, const int* keep_idx, int keep, const float* inv_v,
                          int* assign, void* merged, float* ws_best, int* ws_bidx,
-                         int n_split, int* ws_pruned, void* ws_perm, int num_sms, cudaStream_t s,
+                         int* ws_pruned, void* ws_perm, int num_sms, cudaStream_t s,
                          bool index_ready = false);
 
 // tcgen05 forms of the pre-LLM Grams (bf16), used by the launchers above

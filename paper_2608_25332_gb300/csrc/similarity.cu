@@ -10,9 +10,11 @@
 //               (= largest <v_j, v_k> / |v_k|, since |v_j| is common), ties to
 //               the lower kept position; merged_a = mean of centroid a and its
 //               members, summed in ascending row order.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
-#include "simt_gemm.cuh"
+#include "simt_split.cuh"
 
 namespace provip {
 namespace {
@@ -25,33 +27,40 @@ __device__ __forceinline__ const T* row_ptr(const void* base, size_t row, int D)
 // ---------------------------------------------------------------------------
 // Sec. 4.2
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) crit_gram_kernel(const SimArgs a, float* G) {
-  __shared__ __align__(16) SimtSmem sm;
-  __shared__ const float* arow[kSimtBM];
-  __shared__ const float* brow[kSimtBN];
-  const int b = blockIdx.z;
-  const int r0 = blockIdx.y * kSimtBM, c0 = blockIdx.x * kSimtBN;
+// the fp32 text Gram: a cluster per 64 x 64 tile (simt_split.cuh), CTA c of it
+// writing rows [c * 64 / C, ..)
+__global__ void __launch_bounds__(split::kThreads, split::kCtasPerSm) crit_gram_kernel(const SimArgs a, int C, float* G) {
+  extern __shared__ __align__(128) uint8_t ring[];
+  __shared__ const float* arow[split::kTile];
+  __shared__ const float* brow[split::kTile];
+  const int rank = blockIdx.x % C, tile = blockIdx.x / C, b = blockIdx.y;
+  const int nt = (a.N_t_max + split::kTile - 1) / split::kTile;
+  const int r0 = tile / nt * split::kTile, c0 = tile % nt * split::kTile;
   int tl = a.text_len[b];
   if (tl < 0 || tl > a.N_t_max) tl = 0;
-  if (threadIdx.x < kSimtBM) {
-    const int j = r0 + threadIdx.x;
-    arow[threadIdx.x] = j < tl ? row_ptr<float>(a.emb_t, (size_t)b * a.N_t_max + j, a.D) : nullptr;
-  }
-  if (threadIdx.x < kSimtBN) {
-    const int j = c0 + threadIdx.x;
+  if (r0 >= tl || c0 >= tl) return;  // every CTA of the cluster: nothing reads the tile
+  if (threadIdx.x < split::kTile) {
+    const int i = r0 + threadIdx.x, j = c0 + threadIdx.x;
+    arow[threadIdx.x] = i < tl ? row_ptr<float>(a.emb_t, (size_t)b * a.N_t_max + i, a.D) : nullptr;
     brow[threadIdx.x] = j < tl ? row_ptr<float>(a.emb_t, (size_t)b * a.N_t_max + j, a.D) : nullptr;
   }
   __syncthreads();
-  float acc[8][4];
-  simt_gemm_nt<float>(arow, brow, a.D, sm, acc);
-  const int rg = threadIdx.x >> 4, kg = threadIdx.x & 15;
+  int k0, k1;
+  split::share(a.D, rank, C, k0, k1);
+  split::tile_part<float>(arow, brow, k0, k1, ring, a.emb_t);
+  split::cluster_sync();
+  const int n_rows = split::kTile / C, c = c0 + (threadIdx.x & 15) * 4;
+  for (int i = threadIdx.x >> 4; i < n_rows; i += split::kThreads / 16) {
+    const int r = rank * n_rows + i;
+    const float4 g = split::sum_parts(ring, r, (threadIdx.x & 15) * 4, C);
+    if (r0 + r >= tl) continue;
+    float* o = G + ((size_t)b * a.N_t_max + r0 + r) * a.N_t_max + c;
+    const float ge[4] = {g.x, g.y, g.z, g.w};
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int jj = 0; jj < 4; ++jj) {
-      const int r = r0 + rg + 16 * i, c = c0 + kg + 16 * jj;
-      if (r < a.N_t_max && c < a.N_t_max) G[((size_t)b * a.N_t_max + r) * a.N_t_max + c] = acc[i][jj];
-    }
+    for (int e = 0; e < 4; ++e)
+      if (c + e < tl) o[e] = ge[e];
+  }
+  split::cluster_sync();  // no CTA leaves while a peer may still read its part
 }
 
 // From the sample Grams G [B][Ntm][Ntm]: row softmax, column means r, threshold
@@ -351,8 +360,17 @@ __global__ void __launch_bounds__(256) vis_sum_reduce_kernel(const SimArgs a, co
   const int d = blockIdx.x * 256 + threadIdx.x;
   const int b = blockIdx.y;
   if (d >= a.D) return;
+  const float* p = part + (size_t)b * a.D + d;
+  const size_t step = (size_t)a.B * a.D;
   float s = 0.f;
-  for (int z = 0; z < nz; ++z) s += part[((size_t)z * a.B + b) * a.D + d];
+  for (int z0 = 0; z0 < nz; z0 += 32) {  // 32 loads in flight, the adds in chunk order
+    float x[32];
+#pragma unroll
+    for (int u = 0; u < 32; ++u) x[u] = z0 + u < nz ? p[(size_t)(z0 + u) * step] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 32; ++u)
+      if (z0 + u < nz) s += x[u];
+  }
   sum[(size_t)b * a.D + d] = s;
 }
 
@@ -375,6 +393,7 @@ __global__ void __launch_bounds__(256) text_mu_kernel(const SimArgs a, const flo
   const T* t = static_cast<const T*>(a.emb_t) + ((size_t)b * a.N_t_max + i) * a.D;
   const float* sv = sum + (size_t)b * a.D;
   float ss = 0.f, dt = 0.f;
+#pragma unroll 4
   for (int d = lane * 8; d < a.D; d += 256) {
     float x[8];
     load8(t + d, x);
@@ -396,58 +415,92 @@ __global__ void __launch_bounds__(256) text_mu_kernel(const SimArgs a, const flo
   }
 }
 
-// p_j = max over critical rows of cos - mu; CTA = 64 visual rows x all text rows
+// p_j = max over critical rows of cos - mu. A cluster per 64 visual rows takes the
+// critical text rows (only those: their list is compacted first, kRelWin text
+// rows at a time) in blocks of 64 (simt_split.cuh); CTA c of it adds and keeps the
+// maxima of visual rows [c * 64 / C, ..).
+constexpr int kRelWin = 1024;
 template <typename T>
-__global__ void __launch_bounds__(256) relevance_kernel(const SimArgs a, const uint8_t* mask,
-                                                        const float* inv_v, const float* mu,
-                                                        const float* invt, float* p) {
-  __shared__ __align__(16) SimtSmem sm;
-  __shared__ const T* arow[kSimtBM];
-  __shared__ const T* brow[kSimtBN];
-  __shared__ float red[8][kSimtBN];
-  const int b = blockIdx.y, c0 = blockIdx.x * kSimtBN;
+__global__ void __launch_bounds__(split::kThreads, split::kCtasPerSm) relevance_kernel(const SimArgs a, int C, const uint8_t* mask,
+                                                                    const float* inv_v, const float* mu,
+                                                                    const float* invt, float* p) {
+  extern __shared__ __align__(128) uint8_t ring[];
+  __shared__ const T* arow[split::kTile];
+  __shared__ const T* brow[split::kTile];
+  __shared__ uint16_t crit[kRelWin];
+  __shared__ int wtot[split::kThreads / 32];
+  __shared__ __align__(16) float4 red[split::kThreads];
+  const int rank = blockIdx.x % C, b = blockIdx.y, c0 = blockIdx.x / C * split::kTile;
   const int tl = min(max(a.text_len[b], 0), a.N_t_max);
-  const int rg = threadIdx.x >> 4, kg = threadIdx.x & 15;
-  float best[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-  if (threadIdx.x < kSimtBN) {
-    const int j = c0 + threadIdx.x;
-    brow[threadIdx.x] = j < a.N_v ? row_ptr<T>(a.emb_v, (size_t)b * a.N_v + j, a.D) : nullptr;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // this thread's four visual rows, and its text rows of a block: rgrp, rgrp + n_grp, ..
+  const int nc = split::kTile / C, nq = nc / 4, n_grp = split::kThreads / nq;
+  const int quad = tid % nq, rgrp = tid / nq;
+  const int j0 = c0 + rank * nc + quad * 4;
+  float iv[4], best[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    iv[e] = j0 + e < a.N_v ? inv_v[(size_t)b * a.N_v + j0 + e] : 0.f;
+    best[e] = -INFINITY;
   }
-  for (int r0 = 0; r0 < tl; r0 += kSimtBM) {
-    __syncthreads();
-    if (threadIdx.x < kSimtBM) {
-      const int i = r0 + threadIdx.x;
+  if (tid < split::kTile) {
+    const int j = c0 + tid;
+    brow[tid] = j < a.N_v ? row_ptr<T>(a.emb_v, (size_t)b * a.N_v + j, a.D) : nullptr;
+  }
+  int k0, k1;
+  split::share(a.D, rank, C, k0, k1);
+  for (int w0 = 0; w0 < tl; w0 += kRelWin) {
+    int nT = 0;  // critical rows of the window
+    for (int i0 = 0; i0 < kRelWin && w0 + i0 < tl; i0 += split::kThreads) {
+      const int i = w0 + i0 + tid;
       const bool in = i < tl && mask[(size_t)b * a.N_t_max + i] != 0;
-      arow[threadIdx.x] = in ? row_ptr<T>(a.emb_t, (size_t)b * a.N_t_max + i, a.D) : nullptr;
-    }
-    __syncthreads();
-    float acc[8][4];
-    simt_gemm_nt<T>(arow, brow, a.D, sm, acc);
+      const unsigned bal = __ballot_sync(0xffffffffu, in);
+      if (lane == 0) wtot[warp] = __popc(bal);
+      __syncthreads();
+      int before = nT;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int r = rg + 16 * i;
-      if (arow[r] == nullptr) continue;
-      const float it = invt[(size_t)b * a.N_t_max + r0 + r], m = mu[(size_t)b * a.N_t_max + r0 + r];
-#pragma unroll
-      for (int jj = 0; jj < 4; ++jj) {
-        const int j = c0 + kg + 16 * jj;
-        if (j < a.N_v) best[jj] = fmaxf(best[jj], acc[i][jj] * it * inv_v[(size_t)b * a.N_v + j] - m);
+      for (int w = 0; w < split::kThreads / 32; ++w) {
+        before += w < warp ? wtot[w] : 0;
+        nT += wtot[w];
       }
+      if (in) crit[before + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(i - w0);
+      __syncthreads();
     }
+    for (int r0 = 0; r0 < nT; r0 += split::kTile) {
+      if (tid < split::kTile)
+        arow[tid] = r0 + tid < nT
+                        ? row_ptr<T>(a.emb_t, (size_t)b * a.N_t_max + w0 + crit[r0 + tid], a.D) : nullptr;
+      __syncthreads();
+      split::tile_part<T>(arow, brow, k0, k1, ring, a.emb_v);
+      split::cluster_sync();
+      for (int r = rgrp; r < min(split::kTile, nT - r0); r += n_grp) {
+        const float4 v = split::sum_parts(ring, r, rank * nc + quad * 4, C);
+        const size_t i = (size_t)b * a.N_t_max + w0 + crit[r0 + r];
+        const float it = invt[i], m = mu[i];
+        best[0] = fmaxf(best[0], v.x * it * iv[0] - m);
+        best[1] = fmaxf(best[1], v.y * it * iv[1] - m);
+        best[2] = fmaxf(best[2], v.z * it * iv[2] - m);
+        best[3] = fmaxf(best[3], v.w * it * iv[3] - m);
+      }
+      split::cluster_sync();  // the parts have been read
+    }
+    __syncthreads();  // crit is rewritten by the next window
   }
-  // max across the 16 row groups
-#pragma unroll
-  for (int jj = 0; jj < 4; ++jj) best[jj] = fmaxf(best[jj], __shfl_xor_sync(0xffffffffu, best[jj], 16));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane < 16)
-#pragma unroll
-    for (int jj = 0; jj < 4; ++jj) red[warp][lane + 16 * jj] = best[jj];
+  red[tid] = make_float4(best[0], best[1], best[2], best[3]);
   __syncthreads();
-  if (threadIdx.x < kSimtBN) {
-    const int j = c0 + threadIdx.x;
-    float m = -INFINITY;
-    for (int w = 0; w < 8; ++w) m = fmaxf(m, red[w][threadIdx.x]);
-    if (j < a.N_v) p[(size_t)b * a.N_v + j] = m;
+  if (rgrp == 0) {
+    float4 m = red[quad];
+    for (int g = 1; g < n_grp; ++g) {
+      const float4 o = red[g * nq + quad];
+      m.x = fmaxf(m.x, o.x);
+      m.y = fmaxf(m.y, o.y);
+      m.z = fmaxf(m.z, o.z);
+      m.w = fmaxf(m.w, o.w);
+    }
+    const float me[4] = {m.x, m.y, m.z, m.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (j0 + e < a.N_v) p[(size_t)b * a.N_v + j0 + e] = me[e];
   }
 }
 
@@ -500,81 +553,86 @@ __device__ __forceinline__ bool better(float v, int i, float bv, int bi) {
   return v > bv || (v == bv && i < bi);
 }
 
-// argmax over one split of the kept columns for a tile of 128 visual rows
+// Argmax over one split of the kept columns for 64 pruned rows: a cluster per
+// (row tile, split) walks the split's 64-column tiles (simt_split.cuh); CTA c of it
+// adds rows [c * 64 / C, ..) and keeps their running (max, lowest position).
 template <typename T>
-__global__ void __launch_bounds__(256) merge_argmax_kernel(const SimArgs a, const int* keep_idx,
-                                                           int keep, const float* inv_v,
-                                                           const int* kpos, int n_split,
-                                                           float* ws_best, int* ws_bidx) {
-  __shared__ __align__(16) SimtSmem sm;
-  __shared__ const T* arow[kSimtBM];
-  __shared__ const T* brow[kSimtBN];
-  __shared__ float kinv[kSimtBN];
-  const int b = blockIdx.y, r0 = blockIdx.x * kSimtBM, split = blockIdx.z;
-  const int ntile = (keep + kSimtBN - 1) / kSimtBN;
-  const int t0 = (int)((long long)ntile * split / n_split), t1 = (int)((long long)ntile * (split + 1) / n_split);
-  const int rg = threadIdx.x >> 4, kg = threadIdx.x & 15;
-  if (threadIdx.x < kSimtBM) {
-    const int j = r0 + threadIdx.x;
-    const bool pruned = j < a.N_v && kpos[(size_t)b * a.N_v + j] < 0;
-    arow[threadIdx.x] = pruned ? row_ptr<T>(a.emb_v, (size_t)b * a.N_v + j, a.D) : nullptr;
+__global__ void __launch_bounds__(split::kThreads, split::kCtasPerSm) merge_argmax_kernel(const SimArgs a, int C, const int* pruned,
+                                                                       int n_pruned, const int* keep_idx, int keep,
+                                                                       const float* inv_v, int n_split,
+                                                                       float* ws_best, int* ws_bidx) {
+  extern __shared__ __align__(128) uint8_t ring[];
+  __shared__ const T* arow[split::kTile];
+  __shared__ const T* brow[split::kTile];
+  __shared__ int rowj[split::kTile];
+  __shared__ float kinv[split::kTile];
+  const int rank = blockIdx.x % C, r0 = blockIdx.x / C * split::kTile, b = blockIdx.y, part = blockIdx.z;
+  const int ntile = (keep + split::kTile - 1) / split::kTile;
+  const int t0 = (int)((long long)ntile * part / n_split), t1 = (int)((long long)ntile * (part + 1) / n_split);
+  const int tid = threadIdx.x, kg = tid & 15;
+  if (tid < split::kTile) {
+    const int j = r0 + tid < n_pruned ? pruned[(size_t)b * n_pruned + r0 + tid] : -1;
+    const bool ok = j >= 0 && j < a.N_v;
+    rowj[tid] = ok ? j : -1;
+    arow[tid] = ok ? row_ptr<T>(a.emb_v, (size_t)b * a.N_v + j, a.D) : nullptr;
   }
-  float bv[8];
-  int bi[8];
+  int k0, k1;
+  split::share(a.D, rank, C, k0, k1);
+  const int n_rows = split::kTile / C;
+  constexpr int kAtOnce = split::kThreads / 16;  // rows a block takes at once
+  constexpr int kRowsPer = split::kTile / kAtOnce;
+  float bv[kRowsPer];
+  int bi[kRowsPer];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    bv[i] = -INFINITY;
-    bi[i] = 0x7fffffff;
+  for (int u = 0; u < kRowsPer; ++u) {
+    bv[u] = -INFINITY;
+    bi[u] = 0x7fffffff;
   }
   for (int t = t0; t < t1; ++t) {
-    const int a0 = t * kSimtBN;
-    __syncthreads();
-    if (threadIdx.x < kSimtBN) {
-      const int ap = a0 + threadIdx.x;
-      if (ap < keep) {
-        const int j = keep_idx[(size_t)b * keep + ap];
-        const bool ok = j >= 0 && j < a.N_v;
-        brow[threadIdx.x] = ok ? row_ptr<T>(a.emb_v, (size_t)b * a.N_v + j, a.D) : nullptr;
-        kinv[threadIdx.x] = ok ? inv_v[(size_t)b * a.N_v + j] : 0.f;
-      } else {
-        brow[threadIdx.x] = nullptr;
-        kinv[threadIdx.x] = 0.f;
-      }
+    const int a0 = t * split::kTile;
+    if (tid < split::kTile) {
+      const int j = a0 + tid < keep ? keep_idx[(size_t)b * keep + a0 + tid] : -1;
+      const bool ok = j >= 0 && j < a.N_v;
+      brow[tid] = ok ? row_ptr<T>(a.emb_v, (size_t)b * a.N_v + j, a.D) : nullptr;
+      kinv[tid] = ok ? inv_v[(size_t)b * a.N_v + j] : 0.f;
     }
     __syncthreads();
-    float acc[8][4];
-    simt_gemm_nt<T>(arow, brow, a.D, sm, acc);
+    split::tile_part<T>(arow, brow, k0, k1, ring, a.emb_v);
+    split::cluster_sync();
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int u = 0; u < kRowsPer; ++u) {
+      if ((tid >> 4) + kAtOnce * u >= n_rows) continue;  // warp-uniform
+      const float4 g = split::sum_parts(ring, rank * n_rows + (tid >> 4) + kAtOnce * u, kg * 4, C);
+      const float ge[4] = {g.x, g.y, g.z, g.w};
 #pragma unroll
-      for (int jj = 0; jj < 4; ++jj) {
-        const int ap = a0 + kg + 16 * jj;
-        if (ap < keep) {
-          const float v = acc[i][jj] * kinv[kg + 16 * jj];
-          if (better(v, ap, bv[i], bi[i])) {
-            bv[i] = v;
-            bi[i] = ap;
-          }
+      for (int e = 0; e < 4; ++e) {
+        const int ap = a0 + kg * 4 + e;
+        const float v = ge[e] * kinv[kg * 4 + e];
+        if (ap < keep && better(v, ap, bv[u], bi[u])) {
+          bv[u] = v;
+          bi[u] = ap;
         }
       }
     }
+    split::cluster_sync();  // the parts and kinv have been read
   }
-  // combine the 16 lanes of each row group
+  // combine the 16 lanes of each row
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int u = 0; u < kRowsPer; ++u) {
+    if ((tid >> 4) + kAtOnce * u >= n_rows) continue;
 #pragma unroll
     for (int o = 8; o > 0; o >>= 1) {
-      const float ov = __shfl_xor_sync(0xffffffffu, bv[i], o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi[i], o);
-      if (better(ov, oi, bv[i], bi[i])) {
-        bv[i] = ov;
-        bi[i] = oi;
+      const float ov = __shfl_xor_sync(0xffffffffu, bv[u], o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi[u], o);
+      if (better(ov, oi, bv[u], bi[u])) {
+        bv[u] = ov;
+        bi[u] = oi;
       }
     }
-    const int j = r0 + rg + 16 * i;
-    if (kg == 0 && j < a.N_v) {
-      ws_best[((size_t)split * a.B + b) * a.N_v + j] = bv[i];
-      ws_bidx[((size_t)split * a.B + b) * a.N_v + j] = bi[i];
+    const int j = rowj[rank * n_rows + (tid >> 4) + kAtOnce * u];
+    if (kg == 0 && j >= 0) {
+      ws_best[((size_t)part * a.B + b) * a.N_v + j] = bv[u];
+      ws_bidx[((size_t)part * a.B + b) * a.N_v + j] = bi[u];
     }
   }
 }
@@ -923,8 +981,11 @@ __global__ void __launch_bounds__(C::kThreads, C::kMinBlocks)
 cudaError_t crit_text_launch(const SimArgs& a, uint8_t* mask, float* r_out, float* G, int num_sms,
                              cudaStream_t s) {
   if (a.dtype == 0) {
-    dim3 g((a.N_t_max + kSimtBN - 1) / kSimtBN, (a.N_t_max + kSimtBM - 1) / kSimtBM, a.B);
-    crit_gram_kernel<<<g, 256, 0, s>>>(a, G);
+    const int nt = (a.N_t_max + split::kTile - 1) / split::kTile;
+    const int C = split::cluster_size((long long)a.B * nt * nt, a.D, num_sms);
+    static std::atomic<bool> set[64];  // per device, zero-initialised
+    const cudaError_t e = split::launch(crit_gram_kernel, split::kSmem<float>, set, dim3((unsigned)(C * nt * nt), (unsigned)a.B), C, s, a, C, G);
+    if (e != cudaSuccess) return e;
   } else {
     bool whole = false;
     cudaError_t e = crit_gram_tc_launch(a, mask, r_out, G, num_sms, &whole, s);
@@ -1020,7 +1081,9 @@ cudaError_t relevance_launch(const SimArgs& a, const uint8_t* mask, float* inv_v
   const int chunk = (a.N_v + n_split - 1) / n_split;
   dim3 g1((a.D + 255) / 256, a.B, n_split);
   dim3 g2((a.N_t_max + 7) / 8, a.B);
-  dim3 g3((a.N_v + kSimtBN - 1) / kSimtBN, a.B);
+  const int n_vt = (a.N_v + split::kTile - 1) / split::kTile;
+  const int C = split::cluster_size((long long)a.B * n_vt, a.D, num_sms);
+  const dim3 g3((unsigned)(C * n_vt), (unsigned)a.B);
   // ws_sum holds n_split partial sums followed by their total
   float* total = ws_sum + (size_t)n_split * a.B * a.D;
   dim3 g4((a.D + 255) / 256, a.B);
@@ -1059,7 +1122,9 @@ cudaError_t relevance_launch(const SimArgs& a, const uint8_t* mask, float* inv_v
       const cudaError_t e = cudaStreamWaitEvent(s, mask_ready, 0);  // the first kernel that reads the mask
       if (e != cudaSuccess) return e;
     }
-    relevance_kernel<float><<<g3, 256, 0, s>>>(a, mask, inv_v, ws_mu, ws_invt, p);
+    static std::atomic<bool> set[64];  // per device, zero-initialised
+    return split::launch(relevance_kernel<float>, split::kSmem<float>, set, g3, C, s, a, C, mask, (const float*)inv_v, (const float*)ws_mu,
+                         (const float*)ws_invt, p);
   } else {
     if (!fused) vis_sum_kernel<__nv_bfloat16><<<g1, 256, 0, s>>>(a, inv_v, ws_sum, chunk);
     vis_sum_reduce_kernel<<<g4, 256, 0, s>>>(a, ws_sum, n_split, total);
@@ -1068,38 +1133,47 @@ cudaError_t relevance_launch(const SimArgs& a, const uint8_t* mask, float* inv_v
       const cudaError_t e = cudaStreamWaitEvent(s, mask_ready, 0);
       if (e != cudaSuccess) return e;
     }
-    relevance_kernel<__nv_bfloat16><<<g3, 256, 0, s>>>(a, mask, inv_v, ws_mu, ws_invt, p);
+    static std::atomic<bool> set[64];  // per device, zero-initialised
+    return split::launch(relevance_kernel<__nv_bfloat16>, split::kSmem<__nv_bfloat16>, set, g3, C, s, a, C, mask, (const float*)inv_v,
+                         (const float*)ws_mu, (const float*)ws_invt, p);
   }
-  return cudaGetLastError();
 }
 
 cudaError_t merge_launch(const SimArgs& a, const int* keep_idx, int keep, const float* inv_v,
-                         int* assign, void* merged, float* ws_best, int* ws_bidx, int n_split,
-                         int* ws_pruned, void* ws_perm, int num_sms, cudaStream_t s, bool index_ready) {
+                         int* assign, void* merged, float* ws_best, int* ws_bidx, int* ws_pruned,
+                         void* ws_perm, int num_sms, cudaStream_t s, bool index_ready) {
   // kpos lives in `assign` until the final assignment overwrites it: it is
-  // read by merge_argmax_kernel and merge_assign_kernel (same index only).
+  // read by merge_assign_kernel (same index only).
   int* kpos = assign;
   const size_t nb = (size_t)a.B * a.N_v;
   const int tc_split = merge_tc_split(a.B, a.N_v, keep, num_sms);
-  const bool tc = ws_pruned != nullptr && ws_perm != nullptr && merge_tc_supported(a, keep, tc_split);
-  // the kept-position map, and the pruned rows for the tensor-core Gram
-  if (!index_ready)
-    merge_index_kernel<<<a.B, 1024, 0, s>>>(keep_idx, keep, a.N_v, kpos, tc ? ws_pruned : nullptr, a.err);
+  const bool tc = ws_perm != nullptr && merge_tc_supported(a, keep, tc_split);
+  const int n_pruned = a.N_v - keep;
+  int n_split = 1;
+  // the kept-position map and the pruned rows
+  if (!index_ready) merge_index_kernel<<<a.B, 1024, 0, s>>>(keep_idx, keep, a.N_v, kpos, ws_pruned, a.err);
   if (tc) {
     cudaError_t e = merge_argmax_tc_launch(a, keep_idx, keep, inv_v, ws_pruned, ws_perm, tc_split, ws_best,
                                            ws_bidx, num_sms, &n_split, s);
     if (e != cudaSuccess) return e;
-  } else {
-    dim3 g((a.N_v + kSimtBM - 1) / kSimtBM, a.B, n_split);
-    if (a.dtype == 0)
-      merge_argmax_kernel<float><<<g, 256, 0, s>>>(a, keep_idx, keep, inv_v, kpos, n_split, ws_best, ws_bidx);
-    else
-      merge_argmax_kernel<__nv_bfloat16><<<g, 256, 0, s>>>(a, keep_idx, keep, inv_v, kpos, n_split, ws_best,
-                                                           ws_bidx);
+  } else if (n_pruned > 0) {
+    // column splits until three CTAs per SM are there, then the K split
+    const int rt = (n_pruned + split::kTile - 1) / split::kTile, ct = (keep + split::kTile - 1) / split::kTile;
+    n_split = (int)std::min<long long>(std::min(ct, kMergeMaxSplit), 3ll * num_sms / ((long long)rt * a.B));
+    if (n_split < 1) n_split = 1;
+    const int C = split::cluster_size((long long)rt * a.B * n_split, a.D, num_sms);
+    const dim3 g((unsigned)(C * rt), (unsigned)a.B, (unsigned)n_split);
+    static std::atomic<bool> set_f32[64], set_bf16[64];  // per device, zero-initialised
+    const cudaError_t e =
+        a.dtype == 0 ? split::launch(merge_argmax_kernel<float>, split::kSmem<float>, set_f32, g, C, s, a, C, (const int*)ws_pruned, n_pruned,
+                                     keep_idx, keep, inv_v, n_split, ws_best, ws_bidx)
+                     : split::launch(merge_argmax_kernel<__nv_bfloat16>, split::kSmem<__nv_bfloat16>, set_bf16, g, C, s, a, C, (const int*)ws_pruned,
+                                     n_pruned, keep_idx, keep, inv_v, n_split, ws_best, ws_bidx);
+    if (e != cudaSuccess) return e;
   }
   // the counter of the long centroids lies past the pruned list's last entry
   // (keep >= 1 leaves room), which nothing else uses
-  int* n_long = merged != nullptr ? ws_pruned + (size_t)a.B * (a.N_v - keep) : nullptr;
+  int* n_long = merged != nullptr ? ws_pruned + (size_t)a.B * n_pruned : nullptr;
   cudaError_t el = launch_pdl(merge_assign_kernel, dim3((unsigned)((nb + 255) / 256)), dim3(256), 0, s, a,
                               (const int*)kpos, n_split, (const float*)ws_best, (const int*)ws_bidx, assign,
                               n_long);
@@ -1136,7 +1210,7 @@ cudaError_t merge_launch(const SimArgs& a, const int* keep_idx, int keep, const 
     const int row_bytes = a.D * (a.dtype == 0 ? 4 : 2);
     // CTAs for the long centroids: two per SM (they leave at once where none is
     // long), one where so few rows are pruned that none can be with a valid keep_idx
-    const int n_lc = a.N_v - keep >= kMeanShort ? 2 * num_sms : 1;
+    const int n_lc = n_pruned >= kMeanShort ? 2 * num_sms : 1;
     const dim3 gm((unsigned)((size_t)a.B * keep + n_lc));
     cudaError_t em;
     auto go = [&](auto kernel, unsigned threads, size_t smem) {
