@@ -55,3 +55,32 @@ def test_merge_means_of_long_centroids(dtype, D, B):
         check_merge(Evn[b], keeps[b], assign[b].cpu().numpy(), merged[b].float().cpu().numpy().astype(np.float64),
                     dtype, f"long centroids {dtype} D={D} [{b}]", a_ref,
                     np.setdiff1d(np.arange(N_v), keeps[b]), mg_ref=mg_ref)
+
+
+@pytest.mark.parametrize("keep", [2, 40])
+@pytest.mark.parametrize("D", [264, 2056])
+def test_fp32_means_of_huge_and_non_finite_values(keep, D):
+    """fp32 sums that leave fp32's range, cancel, or meet infinities and NaN give
+    the means that double sums give (the GPU's own member sets, both paths)."""
+    rng = np.random.default_rng(D + keep)
+    N_v = 80
+    Ev = rng.standard_normal((1, N_v, D)).astype(np.float32)
+    Ev[0, :, 0] = 3.0e38                      # the sum overflows fp32, the mean does not
+    Ev[0, :, 1] = np.where(np.arange(N_v) % 2, 3.0e38, -3.0e38)
+    Ev[0, 9, 2] = np.inf
+    Ev[0, 9, 3], Ev[0, 10, 3] = np.inf, -np.inf
+    Ev[0, 11, 4] = np.nan
+    Ev[0, :, 5] = 1e-40                       # subnormal
+    Ev[0, :, 6] = 1e30 * rng.standard_normal(N_v)
+    keeps = np.sort(rng.choice(N_v, keep, replace=False)).astype(np.int32)[None]
+    assign, merged = P.provip_merge(torch.from_numpy(Ev).to(DEV), torch.from_numpy(keeps).to(DEV))
+    torch.cuda.synchronize()
+    a = assign[0].cpu().numpy()
+    with np.errstate(invalid="ignore", over="ignore"):
+        ref = np.stack([Ev[0, a == q].astype(np.float64).mean(axis=0) for q in range(keep)])
+    got = merged[0].cpu().numpy().astype(np.float64)
+    assert np.array_equal(np.isnan(ref), np.isnan(got))
+    fin = np.isfinite(ref)
+    assert np.array_equal(ref[~fin & ~np.isnan(ref)], got[~fin & ~np.isnan(ref)])
+    # one unit in the last place (the sums' own rounding is 2^-24 below it)
+    assert np.all(np.abs(got[fin] - ref[fin]) <= np.spacing(np.abs(ref[fin]).astype(np.float32)))
