@@ -129,7 +129,7 @@ __device__ __forceinline__ void phase_row(const CompactArgs& a, int phase, long 
 template <int kSlots>
 __global__ void __launch_bounds__(kCompactThreadsSmall) compact_kernel(const CompactArgs a, int np0,
                                                                    int np1, int np2, int small,
-                                                                   int alone) {
+                                                                   int alone, int early) {
   extern __shared__ __align__(128) uint8_t slots[];
   __shared__ __align__(8) uint64_t bars[kSlots];
   __shared__ char* ring_dst[kSlots];
@@ -159,8 +159,10 @@ __global__ void __launch_bounds__(kCompactThreadsSmall) compact_kernel(const Com
   }
 
   // a kernel launched as this grid's programmatic dependent may start now (it
-  // waits for this grid's completion before touching anything written here)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // waits for this grid's completion before touching anything written here);
+  // not when this grid started before the selection had read its scores, which
+  // such a kernel may rewrite
+  if (!early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (blockIdx.x == 0 && a.seq_len_out != nullptr)
     for (int b = threadIdx.x; b < a.B; b += blockDim.x)
       a.seq_len_out[b] = a.seq_len[b] - a.N_v + a.keep;
@@ -404,11 +406,11 @@ __global__ void __launch_bounds__(kCompactThreadsSmall) compact_kernel(const Com
 // same loads, one transaction).
 constexpr int kVecThreads = 128;
 constexpr int kVecPieces = 8;
-__global__ void __launch_bounds__(kVecThreads) compact_vec_kernel(const CompactArgs a) {
+__global__ void __launch_bounds__(kVecThreads) compact_vec_kernel(const CompactArgs a, int early) {
   const int lane = threadIdx.x & 31;
   const long long warp = (long long)blockIdx.x * (kVecThreads / 32) + (threadIdx.x >> 5);
   const long long n_warps = (long long)gridDim.x * (kVecThreads / 32);
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (!early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (blockIdx.x == 0 && a.seq_len_out != nullptr)
     for (int b = threadIdx.x; b < a.B; b += blockDim.x) a.seq_len_out[b] = a.seq_len[b] - a.N_v + a.keep;
   const int n16[3] = {a.n_tensors > 0 ? (int)(a.row_bytes[0] / 16) : 0,
@@ -468,7 +470,7 @@ __global__ void __launch_bounds__(kVecThreads) compact_vec_kernel(const CompactA
 }  // namespace
 
 cudaError_t compact_launch(const CompactArgs& a, int num_sms, cudaStream_t s, bool pdl, bool allow_deep,
-                           bool concurrent, bool host_rows) {
+                           bool concurrent, bool host_rows, bool early) {
   if (host_rows) {
     // rows in mapped host memory: plain vector copies over the whole GPU
     const long long rows = (long long)a.B * a.L_out;
@@ -484,7 +486,7 @@ cudaError_t compact_launch(const CompactArgs& a, int num_sms, cudaStream_t s, bo
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, compact_vec_kernel, a);
+    return cudaLaunchKernelEx(&cfg, compact_vec_kernel, a, early ? 1 : 0);
   }
   static std::atomic<bool> configured[64];  // per device, zero-initialised
   int dev = 0;
@@ -535,8 +537,8 @@ cudaError_t compact_launch(const CompactArgs& a, int num_sms, cudaStream_t s, bo
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
   const int alone = pdl ? 0 : 1;
-  return deep ? cudaLaunchKernelEx(&cfg, compact_kernel<kSlotsDeep>, a, np[0], np[1], np[2], small, alone)
-              : cudaLaunchKernelEx(&cfg, compact_kernel<kSlotsShort>, a, np[0], np[1], np[2], small, alone);
+  return deep ? cudaLaunchKernelEx(&cfg, compact_kernel<kSlotsDeep>, a, np[0], np[1], np[2], small, alone, early ? 1 : 0)
+              : cudaLaunchKernelEx(&cfg, compact_kernel<kSlotsShort>, a, np[0], np[1], np[2], small, alone, early ? 1 : 0);
 }
 
 }  // namespace provip

@@ -124,6 +124,10 @@ struct TopkArgs {
   // else -1) and pruned_out [B][N - k] (the others, ascending)
   int* kpos_out;
   int* pruned_out;
+  // let the kernel after this one start once the kernel before is done instead of
+  // once the scores have been read (it must not write what this one reads, nor let
+  // a kernel after it do so)
+  int early_next;
   unsigned* err;
 };
 constexpr int kTopkMaxN = 49152;
@@ -158,10 +162,13 @@ struct CompactArgs {
 // head-score CTA per SM, not for the cluster form's larger one). concurrent:
 // other calls run beside this one on other streams, so a small problem takes
 // only the CTAs its bytes fill (otherwise it spreads over every SM).
+// early: the kernel that writes idx let this one start before it read its inputs
+// (TopkArgs), so this one does not let the next start before it completes.
 // host_rows: sources or destinations may be mapped host memory, so every row is
 // copied with 16-byte loads and stores (no bulk copies).
 cudaError_t compact_launch(const CompactArgs& a, int num_sms, cudaStream_t s, bool pdl = false,
-                           bool allow_deep = true, bool concurrent = false, bool host_rows = false);
+                           bool allow_deep = true, bool concurrent = false, bool host_rows = false,
+                           bool early = false);
 
 // ---------------------------------------------------------------------------
 // pre-LLM similarity pass (Sec. 4.2-4.3)

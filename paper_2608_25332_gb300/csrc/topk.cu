@@ -55,6 +55,7 @@ __global__ void __launch_bounds__(kTopkMaxThreads) topk_kernel(const TopkArgs a)
   // scores has completed (which, for overlapped calls, implies the previous
   // compaction has completed too)
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (a.early_next) pdl_allow_next();
   const int b = blockIdx.x;
   uint32_t mn, mx, lo, hi;
   load_sample_keys(a, b, keys, a.scores_out ? a.scores_out + (size_t)b * a.N : nullptr, mn, mx);
@@ -81,6 +82,7 @@ __global__ void __launch_bounds__(kRegMaxThreads) topk_reg_kernel(const TopkArgs
   for (int q = threadIdx.x; q < kSelectBins; q += blockDim.x) sh.hist[0][q] = 0;
   // a programmatic dependent: wait for that kernel
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (a.early_next) pdl_allow_next();
   const int b = blockIdx.x;
   uint32_t key[KPT], mn, mx, lo, hi;
   load_keys_reg<KPT>(a, b, key, mn, mx);
@@ -131,6 +133,7 @@ __global__ void __launch_bounds__(kRankThreads) topk_rank_kernel(const TopkArgs 
   __shared__ int warp_cnt[kRankThreads / 32];
   __shared__ int cta_cnt;
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (a.early_next) pdl_allow_next();
   const uint32_t crank = cluster_ctarank();
   const int b = blockIdx.y, N = a.N;
   // one CTA of the cluster writes the scores
