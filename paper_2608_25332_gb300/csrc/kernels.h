@@ -241,11 +241,12 @@ constexpr int kMergeMaxSplit = 16;
 
 // the merge Gram on pairs of SMs (tcgen05 cta_group::2, merge_pair_tc.cu)
 constexpr int kMergePairHeights = 4;
-// A tile is (512-row group of one sample's pruned rows, range of its kept
+// A tile is (512- or 256-row group of one sample's pruned rows, range of its kept
 // columns); groups x_hi .. Q-1 split the columns into n_lo ranges, groups
 // 0 .. x_hi-1 into n_lo + 1.
 struct MergePairPlan {
-  int n_quads;  // 512-row groups of pruned rows per sample
+  int halves;   // 256-row halves of a group: 2, or 1 (merge_pair_half_plan)
+  int n_quads;  // groups of pruned rows per sample
   int Q;        // groups of the batch: B * n_quads
   int n_lo;     // column ranges of groups x_hi .. Q-1
   int x_hi;     // groups with n_lo + 1 ranges
@@ -254,8 +255,12 @@ struct MergePairPlan {
   int n_slots;  // partial slots per row: n_lo + (x_hi > 0), <= kMergeMaxSplit
   int n_heights;                     // distinct B rows per CTA (N / 2) of the tiles
   int heights[kMergePairHeights];
+  double clocks;                     // the busiest pair's, by the plan's model
 };
+// groups of 512 rows; of 256; and the form with the fewer clocks
 bool merge_pair_plan(int B, int n_pruned, int keep, int D, int num_sms, MergePairPlan* p);
+bool merge_pair_half_plan(int B, int n_pruned, int keep, int D, int num_sms, MergePairPlan* p);
+bool merge_pair_best(int B, int n_pruned, int keep, int D, int num_sms, MergePairPlan* p);
 // bf16, the pair form enabled, and a two-CTA cluster of it fits on this device
 bool merge_pair_usable(const SimArgs& a);
 void merge_pair_enable(int on);

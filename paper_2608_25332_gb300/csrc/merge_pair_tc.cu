@@ -23,6 +23,11 @@
 // and share its A rows through L2. Each CTA loads only the N/2 kept rows its
 // half of the MMA reads (one tensor map per distinct N/2 of the plan).
 //
+// Where 512-row groups are too few for the pairs of SMs (a few hundred pruned rows
+// per sample), groups of 256 rows, one M = 256 half each, make twice the tiles
+// (kHalves = 1): a K slice is then at most 32 KiB per SM, and six stages fit.
+// merge_pair_best takes the form whose busiest pair has the fewest clocks.
+//
 // The epilogue (eight warps: two per TMEM lane quadrant, each taking half of
 // the 32-column pieces, their tensor-memory loads double-buffered) scales
 // column k by 1/|e_k| and keeps per row the running (max, first index) over
@@ -50,11 +55,12 @@ namespace {
 
 using namespace tcg;
 
-constexpr int kPairQuadRows = 4 * kBM;             // pruned rows of a quad (two M = 256 halves)
 constexpr int kPairMaxN = 256;                     // columns of a tile
-constexpr int kPairStages = 4;
-constexpr int kPairStageBytes = 3 * kABytes;       // A0 rows | A1 rows | B rows of this CTA: 48 KiB
-constexpr uint32_t kPairTmemCols = 2 * kPairMaxN;  // one accumulator per half
+// by the M = 256 halves of a group (1 or 2): ring depth, bytes of a stage (A0 rows
+// | A1 rows | B rows of this CTA), one accumulator per half
+__host__ __device__ constexpr int pair_stages(int halves) { return halves == 2 ? 4 : 6; }
+__host__ __device__ constexpr int pair_stage_bytes(int halves) { return (halves + 1) * kABytes; }
+__host__ __device__ constexpr uint32_t pair_tmem_cols(int halves) { return (uint32_t)halves * kPairMaxN; }
 constexpr int kPairEpiWarps = 8;                   // two per TMEM lane quadrant, splitting the columns
 constexpr int kPairThreads = 64 + 32 * kPairEpiWarps;
 
@@ -79,9 +85,10 @@ struct PairMaps {
   CUtensorMap b[kMergePairHeights];
 };
 
+template <int kStages>
 struct PairPipe {
-  uint64_t full[kPairStages];   // even CTA: both CTAs' boxes of the stage have landed
-  uint64_t empty[kPairStages];  // each CTA: the MMAs that read its stage are done
+  uint64_t full[kStages];   // even CTA: both CTAs' boxes of the stage have landed
+  uint64_t empty[kStages];  // each CTA: the MMAs that read its stage are done
   uint64_t acc_full;            // each CTA: the tile's accumulators are complete
   uint64_t acc_empty;           // even CTA: both CTAs' epilogues have read them
   uint32_t tmem;
@@ -217,8 +224,8 @@ __host__ __device__ __forceinline__ PairTile pair_tile(const MergePairPlan& p, i
     g.t = (k - n_wide) % g.n;
   }
   g.b = quad / p.n_quads;
-  g.m0 = (quad % p.n_quads) * kPairQuadRows;
-  g.has1 = g.m0 + 2 * kBM < n_pruned;  // the second half holds pruned rows
+  g.m0 = (quad % p.n_quads) * p.halves * 2 * kBM;
+  g.has1 = p.halves == 2 && g.m0 + 2 * kBM < n_pruned;  // the second half holds pruned rows
   g.c0 = pair_range_start(g.t, g.n, keep);
   g.nv = pair_range_start(g.t + 1, g.n, keep) - g.c0;
   g.N = (g.nv + 31) / 32 * 32;         // MMA width: N / 2 rows of B per CTA, a multiple of 16
@@ -233,10 +240,14 @@ __host__ __device__ __forceinline__ int pair_deal_tile(const MergePairPlan& p, i
   return k < p.T ? k : -1;
 }
 
+template <int kHalves>
 __global__ void __launch_bounds__(kPairThreads, 1)
     merge_argmax_pair_tc(const PairArgs a, const __grid_constant__ PairMaps maps) {
+  constexpr int kPairStages = pair_stages(kHalves), kPairStageBytes = pair_stage_bytes(kHalves);
+  constexpr uint32_t kPairTmemCols = pair_tmem_cols(kHalves);
+  constexpr uint32_t kBOff = kHalves * kABytes;  // B rows in a stage
   extern __shared__ uint8_t smem_raw[];
-  __shared__ PairPipe pipe;
+  __shared__ PairPipe<kPairStages> pipe;
   __shared__ int sidx[2 * kBM];      // original rows of this CTA's A0 and A1 rows (-1: none)
   __shared__ float skinv[kPairMaxN];  // 1/|e_k| of the tile's kept columns
   __shared__ float xbest[2][kBM];     // the upper column half's (max, position) per row
@@ -304,8 +315,8 @@ __global__ void __launch_bounds__(kPairThreads, 1)
           const int x = kb * kBK;
           if (rank == 0) mbar_arrive_expect_tx(&pipe.full[s], tx);
           tma_load_2d_pair(sa, &maps.a, x, row_a, fb);
-          if (g.has1) tma_load_2d_pair(sa + kABytes, &maps.a, x, row_a + 2 * kBM, fb);
-          tma_load_2d_pair(sa + 2 * kABytes, mapB, x, row_b, fb);
+          if (kHalves == 2 && g.has1) tma_load_2d_pair(sa + kABytes, &maps.a, x, row_a + 2 * kBM, fb);
+          tma_load_2d_pair(sa + kBOff, mapB, x, row_b, fb);
         }
       }
       // the MMAs' releases of the last stages land in this CTA before it may exit
@@ -330,13 +341,13 @@ __global__ void __launch_bounds__(kPairThreads, 1)
           }
           tc_fence_after();
           const uint32_t sa = smem_u32(stages + (size_t)s * kPairStageBytes);
-          const uint32_t sb = sa + 2 * kABytes;
+          const uint32_t sb = sa + kBOff;
 #pragma unroll
           for (int k = 0; k < kBK / 16; ++k) {
             const uint32_t acc = (kb > 0 || k > 0) ? 1u : 0u;
             const uint64_t bd = smem_desc_sw128(sb + k * 32);
             mma_pair_bf16(pipe.tmem, smem_desc_sw128(sa + k * 32), bd, idesc, acc);
-            if (g.has1) mma_pair_bf16(pipe.tmem + kPairMaxN, smem_desc_sw128(sa + kABytes + k * 32), bd, idesc, acc);
+            if (kHalves == 2 && g.has1) mma_pair_bf16(pipe.tmem + kPairMaxN, smem_desc_sw128(sa + kABytes + k * 32), bd, idesc, acc);
           }
           commit_pair(&pipe.empty[s]);  // frees stage s in both CTAs
         }
@@ -360,7 +371,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
       const PairTile g = pair_tile(pl, a.n_pruned, a.keep, k);
       const int* pr = a.pruned + (size_t)g.b * a.n_pruned;
       const int* kp = a.keep_idx + (size_t)g.b * a.keep;
-      for (int i = et; i < 2 * kBM; i += 32 * kPairEpiWarps) {
+      for (int i = et; i < kHalves * kBM; i += 32 * kPairEpiWarps) {
         const int pos = g.m0 + (i < kBM ? 0 : 2 * kBM) + (int)rank * kBM + (i & (kBM - 1));
         sidx[i] = pos < a.n_pruned ? pr[pos] : -1;
       }
@@ -385,7 +396,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         const int cb0 = half ? mid : 0, cb1 = half ? ncb : mid;
         // 32-column pieces (chunk cb of A0, then of A1 when the group has a
         // second half), double-buffered: piece j + 1 loads while j is reduced
-        const int sh = g.has1 ? 1 : 0;
+        const int sh = kHalves == 2 && g.has1 ? 1 : 0;
         const int npc = (cb1 - cb0) << sh;
         auto piece = [&](int j, float* v) {
           tmem_ld32(taddr + (uint32_t)((j & sh) * kPairMaxN + (cb0 + (j >> sh)) * 32), v);
@@ -444,7 +455,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         // the last range of a quad with fewer ranges than slots also fills the
         // spare slot with an entry that never wins
         const bool spare = g.t + 1 == g.n && g.n < pl.n_slots;
-        const int j0 = sidx[r], j1 = sidx[kBM + r];
+        const int j0 = sidx[r];
         if (j0 >= 0) {
           a.ws_best[o + j0] = best0;
           a.ws_bidx[o + j0] = bidx0;
@@ -453,12 +464,15 @@ __global__ void __launch_bounds__(kPairThreads, 1)
             a.ws_bidx[o + slot + j0] = 0x7fffffff;
           }
         }
-        if (g.has1 && j1 >= 0) {
-          a.ws_best[o + j1] = best1;
-          a.ws_bidx[o + j1] = bidx1;
-          if (spare) {
-            a.ws_best[o + slot + j1] = -INFINITY;
-            a.ws_bidx[o + slot + j1] = 0x7fffffff;
+        if constexpr (kHalves == 2) {
+          const int j1 = sidx[kBM + r];
+          if (g.has1 && j1 >= 0) {
+            a.ws_best[o + j1] = best1;
+            a.ws_bidx[o + j1] = bidx1;
+            if (spare) {
+              a.ws_best[o + slot + j1] = -INFINITY;
+              a.ws_bidx[o + slot + j1] = 0x7fffffff;
+            }
           }
         }
       }
@@ -471,9 +485,9 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   if (warp == 0) tmem_dealloc_pair(pipe.tmem, kPairTmemCols);
 }
 
-size_t pair_smem() { return (size_t)kPairStages * kPairStageBytes + 1024; }
+size_t pair_smem(int halves) { return (size_t)pair_stages(halves) * pair_stage_bytes(halves) + 1024; }
 
-// per device: 0 = not checked, 1 = two-CTA clusters of this kernel fit, 2 = they do not
+// per device: 0 = not checked, 1 = two-CTA clusters of both forms fit, 2 = they do not
 std::atomic<int> g_pair_ok[64];
 std::atomic<int> g_pair_enabled{1};
 
@@ -485,13 +499,16 @@ void merge_pair_enable(int on) { g_pair_enabled.store(on ? 1 : 0); }
 // of width D on num_sms SMs: among splits that give 1 to 4 tiles per pair of
 // SMs (and the even splits), the one whose busiest pair has the fewest clocks
 // by a model of a tile of N columns: per 64-element K slice the larger of its
-// MMA clocks (4N with both halves of the group, 2N with one) and 960 (the
-// ring's pace: a stage's loads take about 2700 clocks from issue to landing,
-// and four stages fit in shared memory), plus 9000 clocks of epilogue and
-// refill per tile.
-static bool merge_pair_search(int B, int n_pruned, int keep, int D, int num_sms, MergePairPlan* p) {
+// MMA clocks (4N with both halves of the group, 2N with one) and the ring's pace
+// (a stage's loads take about 2700 clocks from issue to landing: 960 with four
+// stages of 48 KiB in shared memory, kHalfPace measured with six of at most 32),
+// plus 9000 clocks of epilogue and refill per tile.
+constexpr double kHalfPace = 850.0;
+static bool merge_pair_search(int halves, int B, int n_pruned, int keep, int D, int num_sms, MergePairPlan* p) {
   if (B < 1 || n_pruned < 1 || keep < 1 || D < 1 || num_sms < 2) return false;
-  const int n_quads = (n_pruned + kPairQuadRows - 1) / kPairQuadRows;
+  const int quad_rows = halves * 2 * kBM;
+  const int n_quads = (n_pruned + quad_rows - 1) / quad_rows;
+  const double pace = halves == 2 ? 960.0 : kHalfPace;
   const long long Q = (long long)B * n_quads;
   const int max_pairs = num_sms / 2;
   const long long n_k = (D + kBK - 1) / kBK;
@@ -502,6 +519,7 @@ static bool merge_pair_search(int B, int n_pruned, int keep, int D, int num_sms,
     const int n_hi = n_lo + (x_hi > 0 ? 1 : 0);
     if (n_lo < 1 || n_hi > kMergeMaxSplit || x_hi < 0 || x_hi >= Q) return;
     MergePairPlan c;
+    c.halves = halves;
     c.n_quads = n_quads;
     c.Q = (int)Q;
     c.n_lo = n_lo;
@@ -528,13 +546,14 @@ static bool merge_pair_search(int B, int n_pruned, int keep, int D, int num_sms,
     for (int pr = 0; pr < c.P; ++pr) {
       for (int r = 0, k; (k = pair_deal_tile(c, pr, r)) >= 0; ++r) {
         const PairTile g = pair_tile(c, n_pruned, keep, k);
-        load[pr] += (double)n_k * fmax((g.has1 ? 4.0 : 2.0) * g.N, 960.0) + 9000.0;
+        load[pr] += (double)n_k * fmax((g.has1 ? 4.0 : 2.0) * g.N, pace) + 9000.0;
       }
     }
     double worst = 0.0;
     for (double l : load) worst = fmax(worst, l);
     if (best < 0 || worst < best) {
       best = worst;
+      c.clocks = worst;
       *p = c;
     }
   };
@@ -549,12 +568,12 @@ static bool merge_pair_search(int B, int n_pruned, int keep, int D, int num_sms,
 }
 
 // The search simulates every candidate's deal (tens to hundreds of
-// microseconds of host time): its results are kept per shape, the last
-// kPlanCache shapes, for the calls that follow.
+// microseconds of host time): its results are kept per shape and form, the last
+// kPlanCache of them, for the calls that follow.
 namespace {
-constexpr int kPlanCache = 16;
+constexpr int kPlanCache = 32;
 struct PlanEntry {
-  int B, n_pruned, keep, D, num_sms;
+  int halves, B, n_pruned, keep, D, num_sms;
   bool ok;
   MergePairPlan plan;
 };
@@ -563,26 +582,46 @@ PlanEntry g_plans[kPlanCache];
 int g_plan_n = 0, g_plan_next = 0;
 }  // namespace
 
-bool merge_pair_plan(int B, int n_pruned, int keep, int D, int num_sms, MergePairPlan* p) {
+static bool plan_of(int halves, int B, int n_pruned, int keep, int D, int num_sms, MergePairPlan* p) {
   {
     std::lock_guard<std::mutex> lock(g_plan_mu);
     for (int i = 0; i < g_plan_n; ++i) {
       const PlanEntry& e = g_plans[i];
-      if (e.B == B && e.n_pruned == n_pruned && e.keep == keep && e.D == D && e.num_sms == num_sms) {
+      if (e.halves == halves && e.B == B && e.n_pruned == n_pruned && e.keep == keep && e.D == D &&
+          e.num_sms == num_sms) {
         if (e.ok) *p = e.plan;
         return e.ok;
       }
     }
   }
   MergePairPlan plan;
-  const bool ok = merge_pair_search(B, n_pruned, keep, D, num_sms, &plan);
+  const bool ok = merge_pair_search(halves, B, n_pruned, keep, D, num_sms, &plan);
   std::lock_guard<std::mutex> lock(g_plan_mu);
   PlanEntry& e = g_plans[g_plan_next];
-  e = PlanEntry{B, n_pruned, keep, D, num_sms, ok, plan};
+  e = PlanEntry{halves, B, n_pruned, keep, D, num_sms, ok, plan};
   g_plan_next = (g_plan_next + 1) % kPlanCache;
   if (g_plan_n < kPlanCache) ++g_plan_n;
   if (ok) *p = plan;
   return ok;
+}
+
+bool merge_pair_plan(int B, int n_pruned, int keep, int D, int num_sms, MergePairPlan* p) {
+  return plan_of(2, B, n_pruned, keep, D, num_sms, p);
+}
+bool merge_pair_half_plan(int B, int n_pruned, int keep, int D, int num_sms, MergePairPlan* p) {
+  return plan_of(1, B, n_pruned, keep, D, num_sms, p);
+}
+
+// Measured: 16 samples of 288 pruned by 288 kept rows, 64 tiles of 256 rows on the 76
+// pairs instead of 32 of 512: 41 -> 31 us; 4 of 962 by 481: 41 -> 30; 32 of 384 by
+// 192 (width 5120): 50 -> 44. 8 of 1920 by 960 keep 512-row groups (84 us): 256-row
+// tiles would take four rounds of the pairs instead of two.
+bool merge_pair_best(int B, int n_pruned, int keep, int D, int num_sms, MergePairPlan* p) {
+  MergePairPlan half;
+  const bool two = merge_pair_plan(B, n_pruned, keep, D, num_sms, p);
+  const bool one = merge_pair_half_plan(B, n_pruned, keep, D, num_sms, &half);
+  if (one && (!two || half.clocks < p->clocks)) *p = half;
+  return two || one;
 }
 
 bool merge_pair_usable(const SimArgs& a) {
@@ -592,10 +631,9 @@ bool merge_pair_usable(const SimArgs& a) {
   int st = g_pair_ok[dev].load(std::memory_order_acquire);
   if (st == 0) {
     st = 2;
-    const size_t smem = pair_smem();
-    cudaError_t e = cudaFuncSetAttribute(merge_argmax_pair_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e == cudaSuccess) {
+    auto fits = [](auto kernel, size_t smem) {
+      cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
       cudaLaunchConfig_t cfg = {};
       cudaLaunchAttribute attr[1];
       attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -608,9 +646,12 @@ bool merge_pair_usable(const SimArgs& a) {
       cfg.attrs = attr;
       cfg.numAttrs = 1;
       int n = 0;
-      e = cudaOccupancyMaxActiveClusters(&n, merge_argmax_pair_tc, &cfg);
-      if (e == cudaSuccess && n > 0) st = 1;
-    }
+      e = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
+      return e == cudaSuccess && n < 1 ? cudaErrorInvalidConfiguration : e;
+    };
+    cudaError_t e = fits(merge_argmax_pair_tc<2>, pair_smem(2));
+    if (e == cudaSuccess) e = fits(merge_argmax_pair_tc<1>, pair_smem(1));
+    if (e == cudaSuccess) st = 1;
     // a refused attribute or query falls back to the single-SM form: clear the
     // error it left (only then, so that no earlier error of the caller is lost)
     if (e != cudaSuccess) cudaGetLastError();
@@ -652,11 +693,12 @@ cudaError_t merge_argmax_pair_launch(const SimArgs& a, const int* keep_idx, int 
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.gridDim = dim3((unsigned)(2 * plan.P), 1, 1);
   cfg.blockDim = dim3(kPairThreads, 1, 1);
-  cfg.dynamicSmemBytes = pair_smem();
+  cfg.dynamicSmemBytes = pair_smem(plan.halves);
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, merge_argmax_pair_tc, m, maps);
+  return plan.halves == 2 ? cudaLaunchKernelEx(&cfg, merge_argmax_pair_tc<2>, m, maps)
+                          : cudaLaunchKernelEx(&cfg, merge_argmax_pair_tc<1>, m, maps);
 }
 
 }  // namespace provip

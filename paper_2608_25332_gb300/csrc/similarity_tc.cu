@@ -868,7 +868,7 @@ cudaError_t merge_argmax_tc_launch(const SimArgs& a, const int* keep_idx, int ke
                                    cudaStream_t s) {
   const int n_pruned = a.N_v - keep;  // pruned: the rows not kept, ascending (merge_index_kernel)
   MergePairPlan plan;
-  const bool pairs = merge_pair_usable(a) && merge_pair_plan(a.B, n_pruned, keep, a.D, num_sms, &plan);
+  const bool pairs = merge_pair_usable(a) && merge_pair_best(a.B, n_pruned, keep, a.D, num_sms, &plan);
   cudaError_t e = cudaSuccess;
   if (!pairs) {
     static std::atomic<bool> smem_set[64];  // per device, zero-initialised
