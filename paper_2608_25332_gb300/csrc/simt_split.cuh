@@ -9,8 +9,8 @@
 // CTA multiplies half of a step (two warps per scheduler: one alone waits for
 // its own shared-memory reads), and the halves are added at the end. Thread
 // (rg = tid / 16 % 8, kg = tid % 16) of a half owns rows rg + 8 i (i < 8) and
-// columns kg + 16 j (j < 4). The 128 x 64 tile without the split or
-// the ring (simt_gemm.cuh) took 2.4 us per step and had all of K to itself:
+// columns kg + 16 j (j < 4). A 128 x 64 tile without the split or
+// the ring took 2.4 us per step and had all of K to itself:
 // 311 us for the Gram of 64 text rows of 4096 elements, 367 for their products
 // with 576 visual rows, 411 for 384 pruned by 192 kept rows, on 1, 9 and 15 CTAs;
 // this form takes 21, 25 and 37 (8, 72 and 144 CTAs), about 42% of the issue slots
@@ -170,6 +170,18 @@ __device__ __forceinline__ float4 sum_parts(const uint8_t* ring, int r, int c, i
       s.w += v[q].w;
     }
   return s;
+}
+
+// reductions across the 16 lanes that share a row of a tile
+__device__ __forceinline__ float row16_max(float v) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+__device__ __forceinline__ float row16_sum(float v) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
 // CTAs per cluster for `tiles` clusters over kdim elements: the most that keep
