@@ -26,7 +26,14 @@
 // chunk into one of two 128-column TMEM accumulators and commits, warps 0-7
 // (two per TMEM lane quadrant, 64 columns each) turn accumulators into
 // statistics and release them. The loads, the MMAs and the softmax work of
-// consecutive chunks overlap. Two CTAs per SM (their shared memory rules out a
+// consecutive chunks overlap; clock stamps show the keys always there in time and
+// the round of an accumulator as the bound: freed, 8 MMAs issued (about 650 clocks),
+// done and seen by the workers (1200 more beside the other CTA's MMAs), worked on
+// (1200 to 2300). Descriptors formed for each MMA, waits polled by one lane for its
+// warp and a maximum in one chain had made that round longer: every head of 4 samples
+// of 1003 visual tokens under long texts 58.2 -> 57.2 us for the step, visual heads of
+// 8 x 960 73.0 -> 70.6, the schedule of 16 images 241 -> 236. Sixteen worker warps of
+// 32 columns each were no faster (56 registers a thread, twice the barriers). Two CTAs per SM (their shared memory rules out a
 // third), so the two accumulators of each never wait for tensor memory.
 // Every wait is bounded; a timeout sets the device error word.
 #include "common.cuh"
@@ -165,7 +172,13 @@ __global__ void __launch_bounds__(kThreads, 2)
     if (lane == 0) {
       bool live = mbar_wait(&ctl.q_ready, 0, a.err);
       if (!live) ctl.fail = 1;
-      const uint32_t qa = smem_u32(qs);
+      // operand descriptors of the first K step; a later step adds its byte offset
+      // (16-byte units in the low bits), so that this one lane, which shares its
+      // scheduler with busy workers, issues a chunk in few instructions
+      const uint64_t qd = smem_desc_sw128(smem_u32(qs));
+      uint64_t kd[kStages];
+#pragma unroll
+      for (int s = 0; s < kStages; ++s) kd[s] = smem_desc_sw128(smem_u32(ks + (size_t)s * kTileBytes));
       for (int it = 0; it < n_it && live; ++it) {
         const int s = it % kStages, buf = it & 1;
         const uint32_t ph_k = (uint32_t)(it / kStages) & 1u, ph_a = (uint32_t)(it >> 1) & 1u;
@@ -175,17 +188,17 @@ __global__ void __launch_bounds__(kThreads, 2)
           break;
         }
         tc_fence_after();
-        const uint32_t ka = smem_u32(ks + (size_t)s * kTileBytes);
+        const uint64_t kds = s == 0 ? kd[0] : kd[1];
+        static_assert(kStages == 2, "kds picks one of two");
         const uint32_t acc = ctl.tmem + (uint32_t)(buf * kTile);
         // pass A: S = Q K^T (lane = text row); pass B: S^T = K Q^T (lane =
         // key), so a key's sum over the rows stays in its thread
         const bool tr = it >= nA;
-        const uint32_t opa = tr ? ka : qa, opb = tr ? qa : ka;
+        const uint64_t opa = tr ? kds : qd, opb = tr ? qd : kds;
 #pragma unroll
         for (int kstep = 0; kstep < 8; ++kstep) {
-          const uint32_t off = (kstep >> 2) * kHalfBytes + (kstep & 3) * 32;
-          tc_mma_bf16(acc, smem_desc_sw128(opa + off), smem_desc_sw128(opb + off), kIdesc,
-                      kstep > 0 ? 1u : 0u);
+          const uint64_t off = (uint64_t)((kstep >> 2) * kHalfBytes + (kstep & 3) * 32) >> 4;
+          tc_mma_bf16(acc, opa + off, opb + off, kIdesc, kstep > 0 ? 1u : 0u);
         }
         tc_commit(&ctl.k_empty[s]);
         tc_commit(&ctl.acc_full[buf]);
@@ -198,7 +211,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     const int j = rb * kTile + r;
     const bool rv = j < tl && (a.row_mask == nullptr || a.row_mask[(size_t)b * a.N_t_max + j] != 0);
     const int t = ts + j;
-    const uint32_t tbase = ctl.tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * 64);
+    const uint32_t tbase = ctl.tmem + ((uint32_t)(quad * 32) << 16);
     const float sc = a.scale_log2;
     const int t_first = ts + rb * kTile;  // every row of the block sits at or after it
     bool failed = !warp_mbar_wait(&ctl.q_full, 0, a.err);  // warp-uniform from here on
@@ -220,7 +233,8 @@ __global__ void __launch_bounds__(kThreads, 2)
     float cn = 0.f, cmean = 0.f, cm2 = 0.f;
     for (int it = 0; it < n_it; ++it) {
       const int buf = it & 1;
-      if (!failed) failed = !warp_mbar_wait(&ctl.acc_full[buf], (uint32_t)(it >> 1) & 1u, a.err);
+      if (!failed) failed = !mbar_wait(&ctl.acc_full[buf], (uint32_t)(it >> 1) & 1u, a.err);
+      __syncwarp();
       tc_fence_after();
       if (it == nA) {
         // the row's global (max, sum) from the two column halves
@@ -256,7 +270,8 @@ __global__ void __launch_bounds__(kThreads, 2)
         if (half == 0) crow[r] = (rv && L > 0.f) ? c : INFINITY;  // 2^-inf = 0
         workers_sync();
       }
-      const uint32_t tacc = tbase + (uint32_t)(buf * kTile);
+      const uint32_t taccb = tbase + (uint32_t)(buf * kTile);  // this quadrant's lanes, first column
+      const uint32_t tacc = taccb + (uint32_t)(half * 64);
       if (it < nA) {
 #pragma unroll
         for (int cb = 0; cb < 2; ++cb) {
@@ -266,17 +281,14 @@ __global__ void __launch_bounds__(kThreads, 2)
           const int k0 = it * kTile + half * 64 + cb * 32;
           if (rv) {
             // keys before the block's first row are causal for every row
-            float bm = -INFINITY;
-            if (k0 + 31 <= t_first) {
+            if (k0 + 31 > t_first) {
 #pragma unroll
-              for (int i = 0; i < 32; ++i) bm = fmaxf(bm, v[i]);
-            } else {
-#pragma unroll
-              for (int i = 0; i < 32; ++i) {
-                v[i] = k0 + i <= t ? v[i] : -INFINITY;
-                bm = fmaxf(bm, v[i]);
-              }
+              for (int i = 0; i < 32; ++i) v[i] = k0 + i <= t ? v[i] : -INFINITY;
             }
+            float b4[4] = {v[0], v[1], v[2], v[3]};  // four chains: the same maximum, sooner
+#pragma unroll
+            for (int i = 4; i < 32; ++i) b4[i & 3] = fmaxf(b4[i & 3], v[i]);
+            const float bm = fmaxf(fmaxf(b4[0], b4[1]), fmaxf(b4[2], b4[3]));
             const float mn = fmaxf(m, bm * sc);  // sc > 0: the max commutes with the scale
             if (mn != -INFINITY) {
               float s4[4] = {0.f, 0.f, 0.f, 0.f};
@@ -327,16 +339,19 @@ __global__ void __launch_bounds__(kThreads, 2)
           }
         }
       } else {
-        // transposed: thread = key kk of the chunk, 64 text rows per warp
+        // transposed: thread = key kk of the chunk; the 32-row pieces that hold rows
+        // are shared out between the two warps of a quadrant (with two pieces each
+        // or none, their sums are the same additions)
         const int par = (it - nA) & 1;
         const int kk = quad * 32 + lane, key = a.vis_start + (it - nA) * kTile + kk;
         const bool all_causal = a.vis_start + (it - nA) * kTile + kTile - 1 <= t_first;
         float csum = 0.f;
-#pragma unroll
-        for (int cb = 0; cb < 2; ++cb) {
-          const int i0 = half * 64 + cb * 32;  // first row of the block
+        const int n_pc = (rows + 31) / 32, pc1 = half ? n_pc : (n_pc + 1) / 2;
+#pragma unroll 1
+        for (int pc = half ? (n_pc + 1) / 2 : 0; pc < pc1; ++pc) {
+          const int i0 = pc * 32;  // first row of the piece
           float v[32];
-          tmem_ld32(tacc + cb * 32, v);
+          tmem_ld32(taccb + i0, v);
           tc_wait_ld();
           float s4[4] = {0.f, 0.f, 0.f, 0.f};
           const float4* cr = reinterpret_cast<const float4*>(crow + i0);
