@@ -122,11 +122,9 @@ __global__ void __launch_bounds__(kThreads, CPC == 1 ? 3 : (CPC == 2 ? 2 : 1))
   const int hi = blockIdx.y % a.H_sel, rb = blockIdx.y / a.H_sel;
   const int b = blockIdx.z;
   const int h = a.heads[hi], g = h / (a.H_q / a.H_kv);
+  // the lengths arrive while the keys, which do not depend on them, are on their way
   const int ts = a.text_start[b], sl = a.seq_len[b];
   int tl = a.text_len[b];
-  const bool ok = ts >= 0 && tl >= 0 && tl <= a.N_t_max && sl <= a.L_max && ts + tl <= sl &&
-                  a.vis_start + a.N_v <= sl;
-  if (!ok) tl = 0;
   const int key0 = (int)rank * CPC * kTile;  // first key of this CTA
 
   // shared memory: Q tile then CPC key tiles, 1024-byte aligned
@@ -143,16 +141,19 @@ __global__ void __launch_bounds__(kThreads, CPC == 1 ? 3 : (CPC == 2 ? 2 : 1))
     fence_mbar_init();
     // the loads need no TMEM: issue them before the allocation
     mbar_arrive_expect_tx(&ctl.tma_bar, (uint32_t)(1 + CPC) * kTileBytes);
-    const int yq = b * a.L_max + ts + rb * kTile, xq = h * kHeadDim;
-    tma_load_2d(qs, &tmQ, xq, yq, &ctl.tma_bar);
-    tma_load_2d(qs + kHalfBytes, &tmQ, xq + 64, yq, &ctl.tma_bar);
 #pragma unroll
     for (int c = 0; c < CPC; ++c) {
       const int yk = b * a.L_max + key0 + c * kTile, xk = g * kHeadDim;
       tma_load_2d(ks + c * kTileBytes, &tmK, xk, yk, &ctl.tma_bar);
       tma_load_2d(ks + c * kTileBytes + kHalfBytes, &tmK, xk + 64, yk, &ctl.tma_bar);
     }
+    const int yq = b * a.L_max + ts + rb * kTile, xq = h * kHeadDim;
+    tma_load_2d(qs, &tmQ, xq, yq, &ctl.tma_bar);
+    tma_load_2d(qs + kHalfBytes, &tmQ, xq + 64, yq, &ctl.tma_bar);
   }
+  const bool ok = ts >= 0 && tl >= 0 && tl <= a.N_t_max && sl <= a.L_max && ts + tl <= sl &&
+                  a.vis_start + a.N_v <= sl;
+  if (!ok) tl = 0;
   // warp 1 allocates the tensor memory while thread 0 issues the loads
   if (threadIdx.x >= 32 && threadIdx.x < 64) {
     tmem_alloc(&ctl.tmem, kCols);
@@ -166,15 +167,15 @@ __global__ void __launch_bounds__(kThreads, CPC == 1 ? 3 : (CPC == 2 ? 2 : 1))
     if (!ok && rank == 0 && blockIdx.y == 0) set_error(a.err, kErrBadDeviceArg);
     if (mbar_wait(&ctl.tma_bar, 0, a.err)) {
       tc_fence_after();
-      const uint32_t qa = smem_u32(qs);
+      // a K step adds its byte offset, in 16-byte units, to the first one's descriptors
+      const uint64_t qd = smem_desc_sw128(smem_u32(qs)), kd = smem_desc_sw128(smem_u32(ks));
 #pragma unroll
       for (int c = 0; c < CPC; ++c) {
-        const uint32_t ka = smem_u32(ks + c * kTileBytes);
 #pragma unroll
         for (int kstep = 0; kstep < 8; ++kstep) {
-          const uint32_t off = (kstep >> 2) * kHalfBytes + (kstep & 3) * 32;
-          tc_mma_bf16(ctl.tmem + c * kTile, smem_desc_sw128(qa + off), smem_desc_sw128(ka + off),
-                      kIdesc, kstep > 0 ? 1u : 0u);
+          const uint64_t off = (uint64_t)((kstep >> 2) * kHalfBytes + (kstep & 3) * 32) >> 4;
+          tc_mma_bf16(ctl.tmem + c * kTile, qd + off, kd + off + (uint64_t)(c * kTileBytes >> 4), kIdesc,
+                      kstep > 0 ? 1u : 0u);
         }
       }
       tc_commit(&ctl.mma_bar);
@@ -220,17 +221,14 @@ __global__ void __launch_bounds__(kThreads, CPC == 1 ? 3 : (CPC == 2 ? 2 : 1))
       float mn = m;
       if (rv) {
         // keys before the block's first row are causal for every row
-        float bm = -INFINITY;
-        if (k0 + 31 <= t_first) {
+        if (k0 + 31 > t_first) {
 #pragma unroll
-          for (int i = 0; i < 32; ++i) bm = fmaxf(bm, v[i]);
-        } else {
-#pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            v[i] = k0 + i <= t ? v[i] : -INFINITY;
-            bm = fmaxf(bm, v[i]);
-          }
+          for (int i = 0; i < 32; ++i) v[i] = k0 + i <= t ? v[i] : -INFINITY;
         }
+        float b4[4] = {v[0], v[1], v[2], v[3]};  // four chains: the same maximum, sooner
+#pragma unroll
+        for (int i = 4; i < 32; ++i) b4[i & 3] = fmaxf(b4[i & 3], v[i]);
+        const float bm = fmaxf(fmaxf(b4[0], b4[1]), fmaxf(b4[2], b4[3]));
         mn = fmaxf(m, bm * sc);  // sc > 0: the max commutes with the scale
       }
       if (mn != -INFINITY) {
