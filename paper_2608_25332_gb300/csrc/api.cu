@@ -934,11 +934,9 @@ extern "C" int provip_prune(const void* Q, const void* K, const void* V, const v
     return rc;
   // the compaction is a programmatic dependent of the selection: the rows that
   // do not depend on idx are copied before the selection is done
-  DevInfo* d;
-  if ((rc = dev_info(&d))) return rc;
   CompactArgs ca = compact_args(idx_out, B, N_v, keep, hidden, D, K, V, H_kv, d_h, pos, P, seq_len,
                                 L_max, vis_start, dtype, hidden_out, K_out, V_out, pos_out,
-                                seq_len_out, d->status);
+                                seq_len_out, nullptr);
   const size_t nb = (size_t)B * sizeof(int);
   const bool early = early_compaction(
       flags, ca, {{ws, ws_bytes}, {text_len, nb}, {row_mask_or_null, (size_t)B * N_t_max}});
@@ -947,6 +945,9 @@ extern "C" int provip_prune(const void* Q, const void* K, const void* V, const v
                       idx_out, scores_out_or_null, ws, ws_bytes, stream,
                       (flags & PROVIP_PRUNE_OVERLAP_PREVIOUS) != 0, early);
   if (rc) return rc;
+  DevInfo* d;
+  if ((rc = dev_info(&d))) return rc;
+  ca.err = d->status;
   // the next step's head scores overlap this compaction: the deeper ring only
   // beside the streaming form
   const int form = tc_form(resolve_algo(algo, dtype), B, H_sel, hs_shape(L_max, N_t_max, N_v, algo).n_rb,
@@ -1074,11 +1075,9 @@ extern "C" int provip_prune_visual_heads(
                             K, V, H_kv, d_h, pos, P, seq_len, L_max, vis_start, dtype, hidden_out,
                             K_out, V_out, pos_out);
   if (rc) return rc;
-  DevInfo* d;
-  if ((rc = dev_info(&d))) return rc;
   CompactArgs ca = compact_args(idx_out, B, N_v, keep, hidden, D, K, V, H_kv, d_h, pos, P, seq_len,
                                 L_max, vis_start, dtype, hidden_out, K_out, V_out, pos_out,
-                                seq_len_out, d->status);
+                                seq_len_out, nullptr);
   const size_t nb = (size_t)B * sizeof(int);
   const bool early = early_compaction(flags, ca, {{ws, ws_bytes}, {text_len, nb}});
   rc = visual_heads_impl(Q, K, B, L_max, H_q, H_kv, d_h, text_start, text_len, crit_mask_or_null,
@@ -1087,6 +1086,9 @@ extern "C" int provip_prune_visual_heads(
                          ws_bytes, stream, (flags & PROVIP_PRUNE_OVERLAP_PREVIOUS) != 0, early,
                          "prune_visual_heads");
   if (rc) return rc;
+  DevInfo* d;
+  if ((rc = dev_info(&d))) return rc;
+  ca.err = d->status;
   // every head is scored: the streaming form unless the units are fewer than the SMs
   const int form = tc_form(resolve_algo(algo, dtype), B, H_q, hs_shape(L_max, N_t_max, N_v, algo).n_rb,
                            d->sms);
