@@ -669,48 +669,38 @@ __global__ void merge_assign_kernel(const SimArgs a, const int* kpos, int n_spli
 // The member lists come from a counting sort per sample: counts (atomics),
 // exclusive offsets, unordered fill, and a list of the centroids with more than
 // kMeanShort members (n_long of them over the batch, in no particular order).
-// A centroid with few members takes one CTA, which orders them by rank
-// (ascending row index, so the sum order is fixed), fetches the member rows with
-// bulk copies (cp.async.bulk, one thread issuing) into shared-memory row slots,
-// SLOTS rows per batch, and sums them slot by slot in rank order, each thread
-// over its 16-byte pieces of the row. Each such CTA is a short chain of
-// dependent steps, so the configuration is chosen for CTAs resident per SM: rows
-// of at most 8 KiB take 128 threads with 4 pieces each (8 CTAs per SM), longer
-// rows 256 threads (up to 8192 elements).
-// The long centroids (background that many tokens resemble) would be that chain
-// many times over in one CTA while the GPU drains, so the grid's first CTAs take
-// them, a 16-byte piece per thread: a column slice of one centroid per CTA (a
-// column's sum needs no other column), the members put in ascending order by a
-// bitmap over windows of kMeanWin rows, and their pieces kept kMeanDeep copies
-// ahead (cp.async) in the thread's own shared-memory slots, with no block
-// barrier between rows. With every list in its one CTA, a bf16 batch of 8 x 2880
-// rows whose largest centroids gather some hundreds took 143 us here where the
-// 253 MB it moves take 37; the whole pre-LLM pass went 356 -> 280 us (32 x 576
-// of width 5120: 262 -> 252, one fp32 image: 981 -> 946), the sums unchanged bit
-// for bit, and a video without such centroids stayed as it was (194 -> 192 us).
-constexpr int kMeanShort = 16;  // members of a centroid that one CTA sums row by row
-constexpr int kMeanDeep = 12;   // pieces in flight per thread for the others
+// A task is a column slice of 128 16-byte pieces, one per thread (a column's sum
+// needs no other column), of kMeanGroup consecutive centroids: their member lists
+// are one contiguous run, ordered within each centroid by rank (ascending row index,
+// so the sum order is fixed) into one list of rows, and every thread streams its
+// piece of those rows kMeanDeep copies ahead (cp.async) through its own
+// shared-memory slots, with no block barrier between rows, closing a centroid's
+// mean where its last row passes. The index chain (offsets, members, ranks) is paid
+// once for the group, and the loads run on across its centroids. With a CTA per
+// centroid, its whole rows fetched three at a time, 576 centroids of 32 samples of
+// width 5120 took 56 us (240 MB, 4.3 TB/s), 2304 of one sample 31 us, and take 45 us
+// (5.3 TB/s) and 25 us; groups of 16 and of 4 were within 2% or slower.
+// Centroids with more than kMeanShort members (background that many tokens
+// resemble) would hold a group's CTA while the GPU drains, so the grid's first CTAs
+// take them, a slice of one centroid each, their members put in ascending order by
+// rank or, where there are many, by a bitmap over windows of kMeanWin rows. With
+// every list in one CTA, a bf16 batch of 8 x 2880 rows whose largest centroids gather
+// some hundreds took 143 us here where the 253 MB it moves take 37.
+constexpr int kMeanShort = 16;  // members of a centroid that a group's CTA takes
+constexpr int kMeanGroup = 8;   // centroids of a group
+constexpr int kMeanDeep = 12;   // pieces in flight per thread
+constexpr int kMeanRank = 256;  // members of a long centroid that are ordered by rank
 constexpr int kMeanWin = 1024;
-template <int THR, int PIECES, int SLOTS, int MINB>
-struct MeanCfg {
-  static constexpr int kThreads = THR, kPieces = PIECES, kSlots = SLOTS, kMinBlocks = MINB;
-};
-using MeanSmall = MeanCfg<128, 4, 3, 8>;  // row bytes <= 128 * 4 * 16
-using MeanBf16 = MeanCfg<256, 4, 4, 4>;   // bf16 rows <= 8192 elements
-using MeanF32 = MeanCfg<256, 8, 4, 2>;    // fp32 rows <= 8192 elements
-constexpr int kMeanSmallRowBytes = 128 * 4 * 16;
+constexpr int kMeanThreads = 128;
+constexpr size_t kMeanSmem = (size_t)kMeanDeep * kMeanThreads * 16;
 constexpr int kSortSmemKeep = 6144;  // centroids whose counters the sort keeps in shared memory (48 KiB)
-template <typename C> size_t merge_mean_smem(int row_bytes) {
-  const size_t rows = (size_t)C::kSlots * row_bytes, ring = (size_t)kMeanDeep * C::kThreads * 16;
-  return rows > ring ? rows : ring;
-}
 
 // Counting sort of one sample's rows by centroid (one CTA of 1024 threads):
 // count[b][a] = rows assigned to a, offset[b][.] its exclusive scan, and
 // members[b][offset[a] ..] the rows of a in no particular order (the means
 // rank them), and b * keep + a of every centroid with more than kMeanShort rows
-// appended to long_list (*n_long entries over the batch). The block-wide barriers order the phases (global memory of this
-// block only).
+// appended to long_list (*n_long entries over the batch). The block-wide barriers
+// order the phases (global memory of this block only).
 template <bool kSmem>
 __global__ void __launch_bounds__(1024) merge_sort_kernel(const int* assign, int N_v, int keep, int* count,
                                                           int* offset, int* cursor, int* members, int* n_long,
@@ -857,22 +847,58 @@ __device__ __forceinline__ void cp_async_wait() {
 // + a, whose n members lie unordered at mem[0..n). ring: kMeanDeep pieces per
 // thread. Called by every thread of the block; false where a thread's sums are to
 // be taken again in a wider type.
-template <typename T, typename Acc, typename C>
+template <typename T, typename Acc>
 __device__ __forceinline__ bool mean_long(const SimArgs& a, int b, int n, const int* mem, int slice, uint4* ring,
                                           uint32_t* bits, int* pre, uint16_t* list, T* out) {
   constexpr int kVec = 16 / (int)sizeof(T);
-  const int pc = slice * C::kThreads + (int)threadIdx.x;
+  const int pc = slice * kMeanThreads + (int)threadIdx.x;
   const bool has = pc < a.D / kVec;
   const T* E = static_cast<const T*>(a.emb_v) + (size_t)b * a.N_v * a.D + (size_t)(has ? pc : 0) * kVec;
   uint4* mine = ring + threadIdx.x;
   Acc acc[kVec];
 #pragma unroll
   for (int e = 0; e < kVec; ++e) acc_zero(acc[e]);
-  for (int w0 = 0; w0 < a.N_v; w0 += kMeanWin) {
+  // adds rows at[0..cnt) of base in order
+  auto stream = [&](const T* base, const auto* at, int cnt) {
+    // one group per row, empty past the last, so that a fixed count is in flight
+    auto fetch = [&](int i) {
+      if (has && i < cnt) cp_async16(mine + (i % kMeanDeep) * kMeanThreads, base + (size_t)at[i] * a.D);
+      cp_async_commit();
+    };
+#pragma unroll 1
+    for (int i = 0; i < kMeanDeep - 1; ++i) fetch(i);
+#pragma unroll 1
+    for (int i = 0; i < cnt; ++i) {
+      fetch(i + kMeanDeep - 1);
+      cp_async_wait<kMeanDeep - 1>();
+      if (has) add16(acc, mine[(i % kMeanDeep) * kMeanThreads], E);
+    }
+    cp_async_wait<0>();
+  };
+  if (n <= kMeanRank) {
+    int* un = reinterpret_cast<int*>(list);
+    int* sorted = un + kMeanRank;
+    const int n4 = (n + 3) / 4;
+    __syncthreads();  // the previous task's list has been read
+    for (int m = threadIdx.x; m < 4 * n4; m += kMeanThreads) un[m] = m < n ? mem[m] : 0x7fffffff;
+    __syncthreads();
+    for (int m = threadIdx.x; m < n; m += kMeanThreads) {
+      const int v = un[m];
+      int rank = 0;  // the number of smaller row indices (they are distinct)
+      for (int q = 0; q < n4; ++q) {
+        const int4 x = reinterpret_cast<const int4*>(un)[q];
+        rank += (x.x < v) + (x.y < v) + (x.z < v) + (x.w < v);
+      }
+      sorted[rank] = v;
+    }
+    __syncthreads();
+    stream(E, sorted, n);
+  }
+  for (int w0 = 0; n > kMeanRank && w0 < a.N_v; w0 += kMeanWin) {
     __syncthreads();  // the previous window's list has been read
     if (threadIdx.x < kMeanWin / 32) bits[threadIdx.x] = 0u;
     __syncthreads();
-    for (int m = threadIdx.x; m < n; m += C::kThreads) {
+    for (int m = threadIdx.x; m < n; m += kMeanThreads) {
       const int j = mem[m] - w0;
       if (j >= 0 && j < kMeanWin) atomicOr(&bits[j >> 5], 1u << (j & 31));
     }
@@ -889,27 +915,13 @@ __device__ __forceinline__ bool mean_long(const SimArgs& a, int b, int n, const 
       if (threadIdx.x == 31) pre[32] = incl;
     }
     __syncthreads();
-    for (int j = threadIdx.x; j < kMeanWin; j += C::kThreads) {
+    for (int j = threadIdx.x; j < kMeanWin; j += kMeanThreads) {
       const uint32_t w = bits[j >> 5];
       if (w >> (j & 31) & 1u) list[pre[j >> 5] + __popc(w & ((1u << (j & 31)) - 1u))] = (uint16_t)j;
     }
     __syncthreads();
     const int cnt = pre[32];
-    const T* Ew = E + (size_t)w0 * a.D;
-    // one group per row, empty past the last, so that a fixed count is in flight
-    auto fetch = [&](int i) {
-      if (has && i < cnt) cp_async16(mine + (i % kMeanDeep) * C::kThreads, Ew + (size_t)list[i] * a.D);
-      cp_async_commit();
-    };
-#pragma unroll 1
-    for (int i = 0; i < kMeanDeep - 1; ++i) fetch(i);
-#pragma unroll 1
-    for (int i = 0; i < cnt; ++i) {
-      fetch(i + kMeanDeep - 1);
-      cp_async_wait<kMeanDeep - 1>();
-      if (has) add16(acc, mine[(i % kMeanDeep) * C::kThreads], E);
-    }
-    cp_async_wait<0>();
+    stream(E + (size_t)w0 * a.D, list, cnt);
   }
   bool ok = true;
   if (has) {
@@ -921,110 +933,112 @@ __device__ __forceinline__ bool mean_long(const SimArgs& a, int b, int n, const 
   return ok;
 }
 
-template <typename T, typename Acc, typename C>
-__global__ void __launch_bounds__(C::kThreads, C::kMinBlocks)
+template <typename T, typename Acc>
+__global__ void __launch_bounds__(kMeanThreads, 8)
     merge_mean_kernel(const SimArgs a, const int* count, const int* offset, const int* members_all, int keep,
                       void* merged, const int* n_long, const int* long_list, int long_ctas) {
-  constexpr int kMeanThreads = C::kThreads, kMeanSlots = C::kSlots;
-  static_assert(kMeanWin / 32 == 32 && kMeanShort <= 32, "a word of the window per lane, a member per lane");
-  extern __shared__ __align__(128) uint8_t slots[];  // kMeanSlots rows, or the long centroids' ring
-  __shared__ int members[kMeanShort];
+  static_assert(kMeanWin / 32 == 32, "a word of the window per lane");
+  static_assert(2 * kMeanRank * sizeof(int) <= kMeanWin * sizeof(uint16_t), "the ranked lists take the window's place");
+  static_assert(kMeanGroup * kMeanShort == kMeanThreads, "a member of the group per thread");
+  extern __shared__ __align__(128) uint4 mean_ring[];  // kMeanDeep pieces per thread
   __shared__ uint32_t bits[kMeanWin / 32];
   __shared__ int pre[kMeanWin / 32 + 1];
-  __shared__ uint16_t list[kMeanWin];
-  __shared__ __align__(8) uint64_t bar;
+  __shared__ __align__(16) uint16_t list[kMeanWin];
+  __shared__ int unsorted[kMeanThreads], rows[kMeanThreads];
+  __shared__ int gcount[kMeanGroup], gstart[kMeanGroup + 1];
+  __shared__ bool gbrief[kMeanGroup];
   constexpr int kVec = 16 / (int)sizeof(T);  // elements per 16-byte piece
-  constexpr int kPieces = C::kPieces;
+  const int n_slices = (a.D / kVec + kMeanThreads - 1) / kMeanThreads;
+  const int tid = threadIdx.x;
   pdl_wait_prior();  // the member lists come from the sort before
   if ((int)blockIdx.x < long_ctas) {
-    const int n_slices = (a.D / kVec + kMeanThreads - 1) / kMeanThreads;
     const long long n_tasks = (long long)*n_long * n_slices;
     for (long long t = blockIdx.x; t < n_tasks; t += long_ctas) {
       const int cen = long_list[t / n_slices], b = cen / keep, n = count[cen];
       const int* mem = members_all + (size_t)b * a.N_v + offset[cen];
-      uint4* ring = reinterpret_cast<uint4*>(slots);
       T* out = static_cast<T*>(merged) + (size_t)cen * a.D;
-      const bool ok = mean_long<T, Acc, C>(a, b, n, mem, (int)(t % n_slices), ring, bits, pre, list, out);
+      const bool ok = mean_long<T, Acc>(a, b, n, mem, (int)(t % n_slices), mean_ring, bits, pre, list, out);
       if constexpr (sizeof(T) == 4)
         if (__syncthreads_or(!ok))
-          mean_long<T, double, C>(a, b, n, mem, (int)(t % n_slices), ring, bits, pre, list, out);
+          mean_long<T, double>(a, b, n, mem, (int)(t % n_slices), mean_ring, bits, pre, list, out);
     }
     return;
   }
-  const int cen = (int)blockIdx.x - long_ctas, b = cen / keep;
-  const T* E = static_cast<const T*>(a.emb_v) + (size_t)b * a.N_v * a.D;
-  T* out = static_cast<T*>(merged) + (size_t)cen * a.D;
-  const uint32_t row_bytes = (uint32_t)a.D * (uint32_t)sizeof(T);
-  const int n_pieces = a.D / kVec;
-  // count and offset issued together: the member list depends on both
-  const int n_all = count[cen];
-  const int off0 = offset[cen];
-  if (n_all > kMeanShort) return;  // among the long ones
-  Acc acc[kPieces][kVec];
-#pragma unroll
-  for (int k = 0; k < kPieces; ++k)
-#pragma unroll
-    for (int e = 0; e < kVec; ++e) acc_zero(acc[k][e]);
-  if (threadIdx.x < 32) {
-    if (threadIdx.x == 0) {
-      mbar_init(&bar, 1);
-      fence_mbar_init();
-    }
-    // rank = number of smaller row indices (they are distinct)
-    const int lane = threadIdx.x;
-    const int v = lane < n_all ? members_all[(size_t)b * a.N_v + off0 + lane] : 0x7fffffff;
-    int rank = 0;
-#pragma unroll
-    for (int q = 0; q < kMeanShort; ++q) rank += __shfl_sync(0xffffffffu, v, q) < v;
-    if (lane < n_all) members[rank] = v;
+  const int n_groups = (keep + kMeanGroup - 1) / kMeanGroup;
+  const int task = (int)blockIdx.x - long_ctas;
+  const int slice = task % n_slices, grp = task / n_slices;
+  const int b = grp / n_groups, a0 = (grp - b * n_groups) * kMeanGroup, ng = min(kMeanGroup, keep - a0);
+  const size_t cen0 = (size_t)b * keep + a0;
+  // this thread's slot of the group: member q of its centroid g (as many slots as a
+  // short centroid may have members); counts and offsets arrive together
+  const int g = tid / kMeanShort, q = tid % kMeanShort;
+  const int n_g = g < ng ? count[cen0 + g] : 0, off_g = g < ng ? offset[cen0 + g] : 0;
+  const bool brief = n_g <= kMeanShort;  // the others are among the long ones
+  const int v = brief && q < n_g ? members_all[(size_t)b * a.N_v + off_g + q] : 0x7fffffff;
+  unsorted[tid] = v;
+  if (q == 0) {
+    gcount[g] = brief ? n_g : 0;
+    gbrief[g] = brief;
   }
   __syncthreads();
-  bool ok = true;
-  uint32_t phase = 0;
-  // adds rows members[0..n_all) in order: batches of kMeanSlots bulk copies
-  for (int m0 = 0; m0 < n_all; m0 += kMeanSlots) {
-    const int nb = min(kMeanSlots, n_all - m0);
-    if (threadIdx.x == 0 && ok) {
-      const uint64_t pol = policy_evict_first();
-      mbar_arrive_expect_tx(&bar, (uint32_t)nb * row_bytes);
-      for (int q = 0; q < nb; ++q)
-        bulk_g2s(slots + (size_t)q * row_bytes, E + (size_t)members[m0 + q] * a.D, row_bytes, &bar, pol);
-    }
-    if (ok && !mbar_wait(&bar, phase, a.err)) ok = false;
-    phase ^= 1u;
-    if (ok) {
-      for (int q = 0; q < nb; ++q) {
-        const uint8_t* row = slots + (size_t)q * row_bytes;
+  int before = 0;  // rows of the group's earlier centroids
 #pragma unroll
-        for (int k = 0; k < kPieces; ++k) {
-          const int pc = k * kMeanThreads + (int)threadIdx.x;
-          if (pc < n_pieces) add16(acc[k], *reinterpret_cast<const uint4*>(row + (size_t)pc * 16), E);
-        }
-      }
-    }
-    __syncthreads();  // the slots may be refilled
+  for (int h = 0; h < kMeanGroup; ++h) before += h < g ? gcount[h] : 0;
+  if (brief && q < n_g) {
+    int rank = 0;  // the number of smaller row indices (they are distinct)
+#pragma unroll
+    for (int h = 0; h < kMeanShort; ++h) rank += unsorted[g * kMeanShort + h] < v;
+    rows[before + rank] = v;
   }
+  if (q == 0) {
+    gstart[g] = before;
+    if (g == kMeanGroup - 1) gstart[kMeanGroup] = before + gcount[g];
+  }
+  __syncthreads();
+  const int n_rows = gstart[kMeanGroup];
+  const int pc = slice * kMeanThreads + tid;
+  if (pc >= a.D / kVec) return;  // no barrier follows
+  const T* E = static_cast<const T*>(a.emb_v) + (size_t)b * a.N_v * a.D + (size_t)pc * kVec;
+  T* out = static_cast<T*>(merged) + cen0 * a.D + (size_t)pc * kVec;
+  uint4* mine = mean_ring + tid;
+  // one group per row, empty past the last, so that a fixed count is in flight
+  auto fetch = [&](int i) {
+    if (i < n_rows) cp_async16(mine + (i % kMeanDeep) * kMeanThreads, E + (size_t)rows[i] * a.D);
+    cp_async_commit();
+  };
+#pragma unroll 1
+  for (int i = 0; i < kMeanDeep - 1; ++i) fetch(i);
+  int i = 0;
+#pragma unroll 1
+  for (int c = 0; c < ng; ++c) {
+    const int end = gstart[c + 1], n = end - i;
+    if (!gbrief[c]) continue;  // among the long ones
+    Acc acc[kVec];
 #pragma unroll
-  for (int k = 0; k < kPieces; ++k) {
-    const int pc = k * kMeanThreads + (int)threadIdx.x;
-    if (pc >= n_pieces) continue;
-    float v[kVec];
+    for (int e = 0; e < kVec; ++e) acc_zero(acc[e]);
+#pragma unroll 1
+    for (; i < end; ++i) {
+      fetch(i + kMeanDeep - 1);
+      cp_async_wait<kMeanDeep - 1>();
+      add16(acc, mine[(i % kMeanDeep) * kMeanThreads], E);
+    }
+    float m[kVec];
     bool fine = true;
 #pragma unroll
-    for (int e = 0; e < kVec; ++e) v[e] = n_all > 0 ? acc_mean(acc[k][e], n_all, fine) : 0.f;
+    for (int e = 0; e < kVec; ++e) m[e] = n > 0 ? acc_mean(acc[e], n, fine) : 0.f;
     if constexpr (sizeof(T) == 4) {
       if (!fine) {
         double d[kVec];
 #pragma unroll
         for (int e = 0; e < kVec; ++e) d[e] = 0.0;
-        for (int m = 0; m < n_all; ++m)
-          add16(d, *reinterpret_cast<const uint4*>(E + (size_t)members[m] * a.D + (size_t)pc * kVec), E);
+        for (int r = end - n; r < end; ++r) add16(d, *reinterpret_cast<const uint4*>(E + (size_t)rows[r] * a.D), E);
 #pragma unroll
-        for (int e = 0; e < kVec; ++e) v[e] = acc_mean(d[e], n_all, fine);
+        for (int e = 0; e < kVec; ++e) m[e] = acc_mean(d[e], n, fine);
       }
     }
-    store16(out + (size_t)pc * kVec, v);
+    store16(out + (size_t)c * a.D, m);
   }
+  cp_async_wait<0>();
 }
 
 }  // namespace
@@ -1244,40 +1258,21 @@ cudaError_t merge_launch(const SimArgs& a, const int* keep_idx, int keep, const 
                          : launch_pdl(merge_sort_kernel<false>, dim3(a.B), dim3(1024), 0, s, (const int*)assign,
                                       a.N_v, keep, cnt, off, cur, mem, n_long, lng);
     if (es != cudaSuccess) return es;
-    static std::atomic<bool> configured[64];  // per device, zero-initialised
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && !configured[dev]) {
-      cudaError_t e = cudaFuncSetAttribute(merge_mean_kernel<float, Sum2, MeanF32>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)merge_mean_smem<MeanF32>(8192 * 4));
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(merge_mean_kernel<__nv_bfloat16, float, MeanBf16>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)merge_mean_smem<MeanBf16>(8192 * 2));
-      if (e != cudaSuccess) return e;
-      configured[dev] = true;
-    }
-    const int row_bytes = a.D * (a.dtype == 0 ? 4 : 2);
-    // CTAs for the long centroids: two per SM (they leave at once where none is
-    // long), one where so few rows are pruned that none can be with a valid keep_idx
-    const int n_lc = n_pruned >= kMeanShort ? 2 * num_sms : 1;
-    const dim3 gm((unsigned)((size_t)a.B * keep + n_lc));
-    cudaError_t em;
-    auto go = [&](auto kernel, unsigned threads, size_t smem) {
-      return launch_pdl(kernel, gm, dim3(threads), smem, s, a, (const int*)cnt, (const int*)off, (const int*)mem,
-                        keep, merged, (const int*)n_long, (const int*)lng, n_lc);
+    const int vec = a.dtype == 0 ? 4 : 8, n_slices = (a.D / vec + kMeanThreads - 1) / kMeanThreads;
+    const int group_tasks = a.B * ((keep + kMeanGroup - 1) / kMeanGroup) * n_slices;
+    // CTAs for the long centroids, which leave at once where none is long: one where
+    // so few rows are pruned that none can be with a valid keep_idx, else two per SM,
+    // and four beside 16 or more groups per SM, which cover the idle ones: at 25 groups
+    // per SM 254 us a pass with many long centroids against 264, at 7.6 without any
+    // 187 against 183.
+    const int n_lc = n_pruned < kMeanShort ? 1 : (group_tasks >= 16 * num_sms ? 4 : 2) * num_sms;
+    const dim3 gm((unsigned)(group_tasks + n_lc));
+    auto go = [&](auto kernel) {
+      return launch_pdl(kernel, gm, dim3(kMeanThreads), kMeanSmem, s, a, (const int*)cnt, (const int*)off,
+                        (const int*)mem, keep, merged, (const int*)n_long, (const int*)lng, n_lc);
     };
-    if (row_bytes <= kMeanSmallRowBytes) {
-      const size_t smem = merge_mean_smem<MeanSmall>(row_bytes);
-      em = a.dtype == 0 ? go(merge_mean_kernel<float, Sum2, MeanSmall>, MeanSmall::kThreads, smem)
-                        : go(merge_mean_kernel<__nv_bfloat16, float, MeanSmall>, MeanSmall::kThreads, smem);
-    } else if (a.dtype == 0) {
-      em = go(merge_mean_kernel<float, Sum2, MeanF32>, MeanF32::kThreads, merge_mean_smem<MeanF32>(row_bytes));
-    } else {
-      em = go(merge_mean_kernel<__nv_bfloat16, float, MeanBf16>, MeanBf16::kThreads,
-              merge_mean_smem<MeanBf16>(row_bytes));
-    }
+    const cudaError_t em = a.dtype == 0 ? go(merge_mean_kernel<float, Sum2>)
+                                        : go(merge_mean_kernel<__nv_bfloat16, float>);
     if (em != cudaSuccess) return em;
   }
   return cudaGetLastError();
