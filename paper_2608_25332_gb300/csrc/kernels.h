@@ -228,9 +228,9 @@ cudaError_t relevance_tc_launch(const SimArgs& a, const uint8_t* mask, const flo
                                 cudaEvent_t mask_ready = nullptr);
 bool merge_tc_supported(const SimArgs& a, int keep, int n_split);
 // pruned: the rows not kept, ascending ([B][N_v - keep], from merge_index_kernel)
-// Writes the permuted copy perm, then runs the Gram on pairs of SMs when they
-// are usable (*n_split_out = its column ranges), else on single SMs with n_split
-// column splits (*n_split_out = n_split).
+// Runs the Gram on pairs of SMs when they are usable (*n_split_out = its column
+// ranges), else on single SMs with n_split column splits (*n_split_out = n_split),
+// after writing the permuted copy perm unless the plan reads the rows directly.
 cudaError_t merge_argmax_tc_launch(const SimArgs& a, const int* keep_idx, int keep,
                                    const float* inv_v, const int* pruned, void* perm,
                                    int n_split, float* ws_best, int* ws_bidx, int num_sms,
@@ -246,6 +246,7 @@ constexpr int kMergePairHeights = 4;
 // 0 .. x_hi-1 into n_lo + 1.
 struct MergePairPlan {
   int halves;   // 256-row halves of a group: 2, or 1 (merge_pair_half_plan)
+  bool direct;  // the rows are read where they lie, not from the permuted copy
   int n_quads;  // groups of pruned rows per sample
   int Q;        // groups of the batch: B * n_quads
   int n_lo;     // column ranges of groups x_hi .. Q-1

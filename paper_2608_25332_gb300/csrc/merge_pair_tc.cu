@@ -2,8 +2,10 @@
 // kept token. The pruned x kept Gram fused with the row argmax, on pairs of SMs
 // (tcgen05 cta_group::2).
 //
-// The operands are contiguous rows of the per-sample copy of E_v permuted to
-// [pruned | kept] (gather_perm_kernel). A unit of work is a tile (sample b,
+// The operands are rows of E_v, fetched where they lie (direct), or contiguous rows
+// of a per-sample copy of E_v permuted to [pruned | kept] (gather_perm_kernel): the
+// copy reads and writes all of E_v, the direct form loads slower (see
+// merge_pair_search). A unit of work is a tile (sample b,
 // 512-row group q of its pruned positions, range t of its kept positions):
 // the group's rows as two M = 256 halves (A0 = the first 256, A1 = the next
 // 256) against the range's kept rows c0 .. c0+N-1 (N <= 256). The two CTAs of
@@ -21,7 +23,7 @@
 // pair_deal_tile), so that the busiest pair of SMs gets as little work as the
 // ranges allow, and the tiles of one group run side by side on different pairs
 // and share its A rows through L2. Each CTA loads only the N/2 kept rows its
-// half of the MMA reads (one tensor map per distinct N/2 of the plan).
+// half of the MMA reads (of the copy: one tensor map per distinct N/2 of the plan).
 //
 // Where 512-row groups are too few for the pairs of SMs (a few hundred pruned rows
 // per sample), groups of 256 rows, one M = 256 half each, make twice the tiles
@@ -62,7 +64,12 @@ __host__ __device__ constexpr int pair_stages(int halves) { return halves == 2 ?
 __host__ __device__ constexpr int pair_stage_bytes(int halves) { return (halves + 1) * kABytes; }
 __host__ __device__ constexpr uint32_t pair_tmem_cols(int halves) { return (uint32_t)halves * kPairMaxN; }
 constexpr int kPairEpiWarps = 8;                   // two per TMEM lane quadrant, splitting the columns
-constexpr int kPairThreads = 64 + 32 * kPairEpiWarps;
+// warps that load: warp 0, and with rows fetched where they lie those past the
+// epilogue's
+__host__ __device__ constexpr int pair_load_warps(bool direct) { return direct ? 11 : 1; }
+__host__ __device__ constexpr int pair_threads(bool direct) {
+  return 32 * (1 + kPairEpiWarps + pair_load_warps(direct));
+}
 
 struct PairArgs {
   const int* pruned;    // [B][n_pruned] original row of each pruned position
@@ -79,7 +86,7 @@ struct PairArgs {
 
 // tensor maps of the permuted copy: A boxes of 128 rows, B boxes of each
 // distinct half-width of the plan's tiles (so that a CTA loads only the N/2
-// kept rows its half of the MMA reads)
+// kept rows its half of the MMA reads); direct: a, of E_v, its boxes one row high
 struct PairMaps {
   CUtensorMap a;
   CUtensorMap b[kMergePairHeights];
@@ -153,6 +160,15 @@ __device__ __forceinline__ void tma_load_2d_pair(void* smem_dst, const CUtensorM
       "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
       "[%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(smem_dst)),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
+      : "memory");
+}
+// rows y0 .. y3 of 64 columns from x, 128 bytes each, one after the other
+__device__ __forceinline__ void tma_gather4_pair(void* smem_dst, const CUtensorMap* map, int x, int y0, int y1, int y2,
+                                                 int y3, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(smem_u32(smem_dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y0), "r"(y1), "r"(y2), "r"(y3), "r"(bar)
       : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
@@ -240,8 +256,8 @@ __host__ __device__ __forceinline__ int pair_deal_tile(const MergePairPlan& p, i
   return k < p.T ? k : -1;
 }
 
-template <int kHalves>
-__global__ void __launch_bounds__(kPairThreads, 1)
+template <int kHalves, bool kDirect>
+__global__ void __launch_bounds__(pair_threads(kDirect), 1)
     merge_argmax_pair_tc(const PairArgs a, const __grid_constant__ PairMaps maps) {
   constexpr int kPairStages = pair_stages(kHalves), kPairStageBytes = pair_stage_bytes(kHalves);
   constexpr uint32_t kPairTmemCols = pair_tmem_cols(kHalves);
@@ -263,7 +279,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
 
   if (threadIdx.x == 0) {
     prefetch_tmap(&maps.a);
-    for (int j = 0; j < pl.n_heights; ++j) prefetch_tmap(&maps.b[j]);
+    for (int j = 0; !kDirect && j < pl.n_heights; ++j) prefetch_tmap(&maps.b[j]);
     for (int s = 0; s < kPairStages; ++s) {
       mbar_init(&pipe.full[s], 1);
       mbar_init(&pipe.empty[s], 1);
@@ -280,12 +296,74 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   tc_fence_before();
   pair_cluster_sync();  // both CTAs' barriers initialised, the pair's tensor memory allocated
   tc_fence_after();
-  // launched as a programmatic dependent of the gather: the set-up above ran
-  // under its tail; the permuted copy and the index tables are read after this
+  // launched as a programmatic dependent of the kernel before: the set-up above ran
+  // under its tail; the rows' copy and the index tables are read after this
   pdl_wait_prior();
   pdl_allow_next();
 
-  if (warp == 0) {
+  // the MMAs' releases of the last stages land in this CTA before it may exit
+  auto drain = [&](int it) {
+    for (int i = it; i < it + kPairStages && !pipe.fail; ++i)
+      if (!mbar_wait(&pipe.empty[i % kPairStages], ((uint32_t)(i / kPairStages) & 1u) ^ 1u, a.err)) pipe.fail = 1;
+  };
+  // loader warps: 0, then those past the epilogue's (2 .. 1 + kPairEpiWarps)
+  const int loader = warp == 0 ? 0 : (warp >= 2 + kPairEpiWarps ? warp - 1 - kPairEpiWarps : -1);
+  if (kDirect && loader >= 0) {
+    // Both CTAs load their rows of every stage, four to a load: 32 loads for the 128
+    // rows of each half, then N / 8 for the B rows, dealt to the loaders' lanes (one
+    // each); completion counts on the even CTA's full barrier, which expects the bytes
+    // of both. Positions past the last pruned or kept row repeat it (computed, never
+    // stored).
+    constexpr int kLoaders = pair_load_warps(true), kLoads = 32 * (kHalves + 1);
+    constexpr int kPer = (kLoads + kLoaders - 1) / kLoaders;
+    static_assert(kPer <= 32, "a load per lane");
+    const int unit = loader * kPer + lane, area = unit / 32;
+    const bool used = lane < kPer && unit < kLoads, bs = area == kHalves;
+    auto rows_of = [&](int k, int* y) {
+      const PairTile g = pair_tile(pl, a.n_pruned, a.keep, k);
+      const int* list = bs ? a.keep_idx + (size_t)g.b * a.keep : a.pruned + (size_t)g.b * a.n_pruned;
+      const int last = (bs ? a.keep : a.n_pruned) - 1;
+      const int p0 = (bs ? g.c0 + (int)rank * (g.N / 2) : g.m0 + area * 2 * kBM + (int)rank * kBM) + 4 * (unit % 32);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        int j = list[min(p0 + e, last)];
+        if (j < 0 || j >= a.N_v) {
+          set_error(a.err, kErrBadDeviceArg);
+          j = 0;
+        }
+        y[e] = g.b * a.N_v + j;
+      }
+    };
+    const uint32_t full0 = cluster_addr(&pipe.full[0], 0);
+    int it = 0;
+    bool ok = true;
+    int next[4] = {0, 0, 0, 0};
+    int k = pair_deal_tile(pl, pair, 0);
+    if (k >= 0 && used) rows_of(k, next);
+    for (int rd = 1; k >= 0 && ok; ++rd) {
+      const PairTile g = pair_tile(pl, a.n_pruned, a.keep, k);
+      const int y0 = next[0], y1 = next[1], y2 = next[2], y3 = next[3];
+      k = pair_deal_tile(pl, pair, rd);
+      if (k >= 0 && used) rows_of(k, next);  // the next tile's rows, under this one's loads
+      const bool mine = used && (bs ? unit % 32 < g.N / 8 : (area == 0 || g.has1));
+      const uint32_t tx = 2u * (uint32_t)((g.has1 ? 2 : 1) * kABytes + (g.N / 2) * kBK * 2);
+      for (int kb = 0; kb < n_k; ++kb, ++it) {
+        const int s = it % kPairStages;
+        const uint32_t ph = (uint32_t)(it / kPairStages) & 1u;
+        if (lane == 0) ok = !pipe.fail && mbar_wait(&pipe.empty[s], ph ^ 1u, a.err);
+        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+        if (!ok) {
+          pipe.fail = 1;
+          break;
+        }
+        if (loader == 0 && rank == 0 && lane == 0) mbar_arrive_expect_tx(&pipe.full[s], tx);
+        if (mine)
+          tma_gather4_pair(stages + (size_t)s * kPairStageBytes + unit * (4 * kBK * 2), &maps.a, kb * kBK, y0, y1, y2,
+                           y3, full0 + 8u * (uint32_t)s);
+      }
+    }
+    if (loader == 0 && lane == 0) drain(it);
+  } else if (!kDirect && warp == 0) {
     if (lane == 0) {
       // both CTAs load their rows of every stage; completion counts on the
       // even CTA's full barrier, which expects the bytes of both
@@ -319,9 +397,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
           tma_load_2d_pair(sa + kBOff, mapB, x, row_b, fb);
         }
       }
-      // the MMAs' releases of the last stages land in this CTA before it may exit
-      for (int i = it; i < it + kPairStages && !pipe.fail; ++i)
-        if (!mbar_wait(&pipe.empty[i % kPairStages], ((uint32_t)(i / kPairStages) & 1u) ^ 1u, a.err)) pipe.fail = 1;
+      drain(it);
     }
   } else if (warp == 1) {
     if (rank == 0 && lane == 0) {
@@ -499,16 +575,30 @@ void merge_pair_enable(int on) { g_pair_enabled.store(on ? 1 : 0); }
 // of width D on num_sms SMs: among splits that give 1 to 4 tiles per pair of
 // SMs (and the even splits), the one whose busiest pair has the fewest clocks
 // by a model of a tile of N columns: per 64-element K slice the larger of its
-// MMA clocks (4N with both halves of the group, 2N with one) and the ring's pace
-// (a stage's loads take about 2700 clocks from issue to landing: 960 with four
-// stages of 48 KiB in shared memory, kHalfPace measured with six of at most 32),
-// plus 9000 clocks of epilogue and refill per tile.
-constexpr double kHalfPace = 850.0;
-static bool merge_pair_search(int halves, int B, int n_pruned, int keep, int D, int num_sms, MergePairPlan* p) {
+// MMA clocks (4N with both halves of the group, 2N with one) and the ring's pace,
+// plus 9000 clocks of epilogue and refill per tile, plus the copy's clocks where the
+// rows are not read where they lie. The pace of boxes of the copy: a stage's loads
+// take about 2700 clocks from issue to landing, 960 with four stages of 48 KiB in
+// shared memory; 760 to 800 measured with six of at most 32. Rows fetched four to a
+// load come slower (paces of 900 to 1100 and of 1300 to 1500 measured): it takes a
+// warp some 150 clocks to issue a load, so that many warps share them, and the SM
+// begins one every 14 clocks at best. The pass of 32 images (576 rows of width 5120)
+// took 196, 181, 178, 172 and 174 us with 4, 6, 8, 11 and 12 of them; on the copy,
+// which alone takes 52 (378 MB), 219. 8 of 2880 rows of width 4096: 256 -> 216; 16
+// images of width 4096: 231 -> 221; 4 of 1443 rows: 135 -> 132. A video of 9216 rows
+// of width 3584 keeps the copy (179 us against 182). Slower than either: 16-byte
+// cp.async by eight warps (243 us for the 32 images: too few requests fit in flight
+// beside the ring), and copying the kept rows alone (191 us).
+constexpr double kBoxPace[2] = {780.0, 960.0};        // by halves
+constexpr double kDirectPace[2] = {1090.0, 1400.0};
+constexpr double kCopyClocksPerByte = 1.9 / 7200;     // 7.2 TB/s, read and write, at 1.9 GHz
+static bool merge_pair_search(int halves, bool direct, int B, int n_pruned, int keep, int D, int num_sms,
+                              MergePairPlan* p) {
   if (B < 1 || n_pruned < 1 || keep < 1 || D < 1 || num_sms < 2) return false;
   const int quad_rows = halves * 2 * kBM;
   const int n_quads = (n_pruned + quad_rows - 1) / quad_rows;
-  const double pace = halves == 2 ? 960.0 : kHalfPace;
+  const double pace = direct ? kDirectPace[halves - 1] : kBoxPace[halves - 1];
+  const double copy = direct ? 0.0 : kCopyClocksPerByte * 4.0 * B * (n_pruned + keep) * (double)D;
   const long long Q = (long long)B * n_quads;
   const int max_pairs = num_sms / 2;
   const long long n_k = (D + kBK - 1) / kBK;
@@ -520,6 +610,7 @@ static bool merge_pair_search(int halves, int B, int n_pruned, int keep, int D, 
     if (n_lo < 1 || n_hi > kMergeMaxSplit || x_hi < 0 || x_hi >= Q) return;
     MergePairPlan c;
     c.halves = halves;
+    c.direct = direct;
     c.n_quads = n_quads;
     c.Q = (int)Q;
     c.n_lo = n_lo;
@@ -551,6 +642,7 @@ static bool merge_pair_search(int halves, int B, int n_pruned, int keep, int D, 
     }
     double worst = 0.0;
     for (double l : load) worst = fmax(worst, l);
+    worst += copy;
     if (best < 0 || worst < best) {
       best = worst;
       c.clocks = worst;
@@ -595,7 +687,12 @@ static bool plan_of(int halves, int B, int n_pruned, int keep, int D, int num_sm
     }
   }
   MergePairPlan plan;
-  const bool ok = merge_pair_search(halves, B, n_pruned, keep, D, num_sms, &plan);
+  bool ok = merge_pair_search(halves, false, B, n_pruned, keep, D, num_sms, &plan);
+  MergePairPlan direct;
+  if (merge_pair_search(halves, true, B, n_pruned, keep, D, num_sms, &direct) && (!ok || direct.clocks < plan.clocks)) {
+    plan = direct;
+    ok = true;
+  }
   std::lock_guard<std::mutex> lock(g_plan_mu);
   PlanEntry& e = g_plans[g_plan_next];
   e = PlanEntry{halves, B, n_pruned, keep, D, num_sms, ok, plan};
@@ -613,8 +710,8 @@ bool merge_pair_half_plan(int B, int n_pruned, int keep, int D, int num_sms, Mer
 }
 
 // Measured: 16 samples of 288 pruned by 288 kept rows, 64 tiles of 256 rows on the 76
-// pairs instead of 32 of 512: 41 -> 31 us; 4 of 962 by 481: 41 -> 30; 32 of 384 by
-// 192 (width 5120): 50 -> 44. 8 of 1920 by 960 keep 512-row groups (84 us): 256-row
+// pairs instead of 32 of 512: 41 -> 31 us (of the copy); 4 of 962 by 481: 41 -> 30;
+// 32 of 384 by 192 (width 5120): 50 -> 44. 8 of 1920 by 960 keep 512-row groups (84 us): 256-row
 // tiles would take four rounds of the pairs instead of two.
 bool merge_pair_best(int B, int n_pruned, int keep, int D, int num_sms, MergePairPlan* p) {
   MergePairPlan half;
@@ -631,7 +728,8 @@ bool merge_pair_usable(const SimArgs& a) {
   int st = g_pair_ok[dev].load(std::memory_order_acquire);
   if (st == 0) {
     st = 2;
-    auto fits = [](auto kernel, size_t smem) {
+    auto fits = [](auto kernel, int halves, bool direct) {
+      const size_t smem = pair_smem(halves);
       cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
       cudaLaunchConfig_t cfg = {};
@@ -641,7 +739,7 @@ bool merge_pair_usable(const SimArgs& a) {
       attr[0].val.clusterDim.y = 1;
       attr[0].val.clusterDim.z = 1;
       cfg.gridDim = dim3(2, 1, 1);
-      cfg.blockDim = dim3(kPairThreads, 1, 1);
+      cfg.blockDim = dim3(pair_threads(direct), 1, 1);
       cfg.dynamicSmemBytes = smem;
       cfg.attrs = attr;
       cfg.numAttrs = 1;
@@ -649,8 +747,10 @@ bool merge_pair_usable(const SimArgs& a) {
       e = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
       return e == cudaSuccess && n < 1 ? cudaErrorInvalidConfiguration : e;
     };
-    cudaError_t e = fits(merge_argmax_pair_tc<2>, pair_smem(2));
-    if (e == cudaSuccess) e = fits(merge_argmax_pair_tc<1>, pair_smem(1));
+    cudaError_t e = fits(merge_argmax_pair_tc<2, false>, 2, false);
+    if (e == cudaSuccess) e = fits(merge_argmax_pair_tc<1, false>, 1, false);
+    if (e == cudaSuccess) e = fits(merge_argmax_pair_tc<2, true>, 2, true);
+    if (e == cudaSuccess) e = fits(merge_argmax_pair_tc<1, true>, 1, true);
     if (e == cudaSuccess) st = 1;
     // a refused attribute or query falls back to the single-SM form: clear the
     // error it left (only then, so that no earlier error of the caller is lost)
@@ -665,9 +765,10 @@ cudaError_t merge_argmax_pair_launch(const SimArgs& a, const int* keep_idx, int 
                                      float* ws_best, int* ws_bidx, cudaStream_t s) {
   PairMaps maps;
   const uint64_t rows = (uint64_t)a.B * a.N_v;
-  if (make_tmap_bf16_2d(&maps.a, perm, rows, (uint64_t)a.D, (uint64_t)a.D * 2, kBM))
+  if (make_tmap_bf16_2d(&maps.a, plan.direct ? a.emb_v : perm, rows, (uint64_t)a.D, (uint64_t)a.D * 2,
+                        plan.direct ? 1 : kBM))
     return cudaErrorInvalidValue;
-  for (int j = 0; j < plan.n_heights; ++j)
+  for (int j = 0; !plan.direct && j < plan.n_heights; ++j)
     if (make_tmap_bf16_2d(&maps.b[j], perm, rows, (uint64_t)a.D, (uint64_t)a.D * 2, (uint32_t)plan.heights[j]))
       return cudaErrorInvalidValue;
   PairArgs m;
@@ -692,13 +793,14 @@ cudaError_t merge_argmax_pair_launch(const SimArgs& a, const int* keep_idx, int 
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.gridDim = dim3((unsigned)(2 * plan.P), 1, 1);
-  cfg.blockDim = dim3(kPairThreads, 1, 1);
+  cfg.blockDim = dim3(pair_threads(plan.direct), 1, 1);
   cfg.dynamicSmemBytes = pair_smem(plan.halves);
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return plan.halves == 2 ? cudaLaunchKernelEx(&cfg, merge_argmax_pair_tc<2>, m, maps)
-                          : cudaLaunchKernelEx(&cfg, merge_argmax_pair_tc<1>, m, maps);
+  auto go = [&](auto kernel) { return cudaLaunchKernelEx(&cfg, kernel, m, maps); };
+  if (plan.direct) return plan.halves == 2 ? go(merge_argmax_pair_tc<2, true>) : go(merge_argmax_pair_tc<1, true>);
+  return plan.halves == 2 ? go(merge_argmax_pair_tc<2, false>) : go(merge_argmax_pair_tc<1, false>);
 }
 
 }  // namespace provip

@@ -878,8 +878,9 @@ cudaError_t merge_argmax_tc_launch(const SimArgs& a, const int* keep_idx, int ke
     if (e != cudaSuccess) return e;
   }
   dim3 gg((a.N_v + 7) / 8, a.B);
-  e = launch_pdl(gather_perm_kernel, gg, dim3(256), 0, s, static_cast<const __nv_bfloat16*>(a.emb_v), pruned,
-                 keep_idx, n_pruned, keep, a.N_v, a.D, static_cast<__nv_bfloat16*>(perm), a.err);
+  if (!pairs || !plan.direct)
+    e = launch_pdl(gather_perm_kernel, gg, dim3(256), 0, s, static_cast<const __nv_bfloat16*>(a.emb_v), pruned,
+                   keep_idx, n_pruned, keep, a.N_v, a.D, static_cast<__nv_bfloat16*>(perm), a.err);
   if (e != cudaSuccess) return e;
   if (pairs) {
     *n_split_out = plan.n_slots;
