@@ -680,10 +680,16 @@ extern "C" int provip_similarity_reduce(const void* emb_v, int B, int N_v, int D
   uint8_t* mask_dst = mask_out_or_null ? mask_out_or_null : w.mask;
   cudaError_t e = cudaSuccess;
   cudaEvent_t mask_ready = nullptr;
-  if (!mask) {
-    // the critical text rows (their Gram and threshold) run on a side stream
-    // beside the relevance Gram, which reads no mask; the stream waits for
-    // them before the kernel that takes the max over the critical rows
+  // the critical text rows run beside the relevance Gram, which reads no mask: first on
+  // the stream, the text norms and the relevance starting under them as programmatic
+  // dependents (crit_leads says where)
+  const bool chain = !mask && crit_leads(a, d->sms);
+  if (chain) {
+    e = crit_text_launch(a, mask_dst, nullptr, w.G, d->sms, s, true);
+    mask = mask_dst;
+  } else if (!mask) {
+    // else on a side stream; the stream waits for them before the kernel that takes
+    // the max over the critical rows
     SideStream* side;
     if ((rc = side_stream(&side))) return rc;
     e = cudaEventRecord(side->fork, s);
@@ -697,7 +703,7 @@ extern "C" int provip_similarity_reduce(const void* emb_v, int B, int N_v, int D
   }
   float* p = p_out_or_null ? p_out_or_null : w.p;
   if (e == cudaSuccess) {
-    e = relevance_launch(a, mask, w.inv_v, p, w.sum, w.mu, w.invt, rel_splits(B, N_v), d->sms, s, mask_ready);
+    e = relevance_launch(a, mask, w.inv_v, p, w.sum, w.mu, w.invt, rel_splits(B, N_v), d->sms, s, mask_ready, chain);
     if (e != cudaSuccess && mask_ready != nullptr) cudaStreamWaitEvent(s, mask_ready, 0);  // join even so
   }
   if (e == cudaSuccess) {

@@ -184,8 +184,11 @@ struct SimArgs {
 // Sec. 4.2: mask[b][j] (and r) from the text self-similarity. ws: G, [B][Ntm][Ntm]
 // f32; Ntm <= kCritMaxNt.
 constexpr int kCritMaxNt = 4096;
+// early (only where crit_leads holds): the next kernel of the stream, launched as a
+// programmatic dependent, may start at once
+bool crit_leads(const SimArgs& a, int num_sms);
 cudaError_t crit_text_launch(const SimArgs& a, uint8_t* mask, float* r_out, float* G, int num_sms,
-                             cudaStream_t s);
+                             cudaStream_t s, bool early = false);
 // inverse L2 norms of every visual row (0 for a zero row): inv_v [B][N_v]
 cudaError_t vis_inv_norm_launch(const SimArgs& a, float* inv_v, cudaStream_t s);
 // the same for the kept rows keep_idx [B][keep] only (inv_v[b][keep_idx[b][q]]),
@@ -199,10 +202,12 @@ cudaError_t kept_inv_norm_launch(const SimArgs& a, const int* keep_idx, int keep
 // mask_ready (optional): an event recorded where the mask is written (another
 // stream); s waits for it before the first kernel that reads the mask, so that
 // the kernels before that one run beside the mask's producer.
+// after_crit (bf16, relevance_tc_supported): the kernel before on s is the critical
+// rows' (crit_text_launch, early), beside which the first kernels run.
 cudaError_t relevance_launch(const SimArgs& a, const uint8_t* mask, float* inv_v,
                              float* p, float* ws_sum, float* ws_mu, float* ws_invt,
                              int n_split, int num_sms, cudaStream_t s,
-                             cudaEvent_t mask_ready = nullptr);
+                             cudaEvent_t mask_ready = nullptr, bool after_crit = false);
 // Sec. 4.3 merge: assign[b][j] and merged[b][a][:]
 // ws_best, ws_bidx: kMergeMaxSplit x [B][N_v]; ws_pruned: [B][N_v] ints; ws_perm:
 // [B][N_v][D] bf16 for the tcgen05 path (null: CUDA-core path); num_sms for the
@@ -217,7 +222,7 @@ cudaError_t merge_launch(const SimArgs& a, const int* keep_idx, int keep, const 
 // tcgen05 forms of the pre-LLM Grams (bf16), used by the launchers above
 // the text Gram into G (bf16), or, up to 128 text rows (*whole), the mask and r at once
 cudaError_t crit_gram_tc_launch(const SimArgs& a, uint8_t* mask, float* r_out, float* G, int num_sms, bool* whole,
-                                cudaStream_t s);
+                                cudaStream_t s, bool early);
 bool relevance_tc_supported(const SimArgs& a);
 // workspace floats of the tensor-core relevance (cosines + per-tile sums)
 size_t relevance_fused_floats(int B, int N_v, int N_t_max);

@@ -201,6 +201,9 @@ __global__ void __launch_bounds__(256) inv_norm_kernel(const void* X, size_t row
   }
   s = warp_sum(s);
   if (lane == 0) inv[row] = s > 0.f ? 1.f / sqrtf(s) : 0.f;
+  // completes after the kernel before it (the critical rows, when it runs beside them),
+  // so that what waits for this grid finds that one's results too
+  pdl_wait_prior();
 }
 
 // ---------------------------------------------------------------------------
@@ -1048,7 +1051,7 @@ __global__ void __launch_bounds__(kMeanThreads, 8)
 }  // namespace
 
 cudaError_t crit_text_launch(const SimArgs& a, uint8_t* mask, float* r_out, float* G, int num_sms,
-                             cudaStream_t s) {
+                             cudaStream_t s, bool early) {
   if (a.dtype == 0) {
     const int nt = (a.N_t_max + split::kTile - 1) / split::kTile;
     const int C = split::cluster_size((long long)a.B * nt * nt, a.D, num_sms);
@@ -1057,7 +1060,7 @@ cudaError_t crit_text_launch(const SimArgs& a, uint8_t* mask, float* r_out, floa
     if (e != cudaSuccess) return e;
   } else {
     bool whole = false;
-    cudaError_t e = crit_gram_tc_launch(a, mask, r_out, G, num_sms, &whole, s);
+    cudaError_t e = crit_gram_tc_launch(a, mask, r_out, G, num_sms, &whole, s, early);
     if (e != cudaSuccess || whole) return e;
   }
   static std::atomic<bool> configured[64];  // per device, zero-initialised
@@ -1138,13 +1141,19 @@ cudaError_t vis_inv_norm_launch(const SimArgs& a, float* inv_v, cudaStream_t s) 
 
 cudaError_t relevance_launch(const SimArgs& a, const uint8_t* mask, float* inv_v, float* p,
                              float* ws_sum, float* ws_mu, float* ws_invt, int n_split,
-                             int num_sms, cudaStream_t s, cudaEvent_t mask_ready) {
+                             int num_sms, cudaStream_t s, cudaEvent_t mask_ready, bool after_crit) {
   // bf16 (up to 4096 text rows): the text rows' inverse norms, one
   // tensor-core read of the visual rows (norms, cosines and de-meaning sums)
   // and a small max kernel
   if (relevance_tc_supported(a)) {
     const size_t rows = (size_t)a.B * a.N_t_max;
-    inv_norm_kernel<__nv_bfloat16><<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(a.emb_t, rows, a.D, ws_invt);
+    if (after_crit) {
+      const cudaError_t e = launch_pdl(inv_norm_kernel<__nv_bfloat16>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0,
+                                       s, a.emb_t, rows, a.D, ws_invt);
+      if (e != cudaSuccess) return e;
+    } else {
+      inv_norm_kernel<__nv_bfloat16><<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(a.emb_t, rows, a.D, ws_invt);
+    }
     return relevance_tc_launch(a, mask, ws_invt, inv_v, p, ws_sum, num_sms, s, mask_ready);
   }
   const int chunk = (a.N_v + n_split - 1) / n_split;

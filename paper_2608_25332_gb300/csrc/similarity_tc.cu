@@ -438,6 +438,7 @@ __global__ void __launch_bounds__(kThreads, 2 / kAcc)
     s_invt[r] = tb0 + r < a.N_t_max ? a.inv_t[(size_t)b * a.N_t_max + tb0 + r] : 0.f;
     asm volatile("bar.sync 1, 128;" ::: "memory");  // s_invt complete (epilogue warps)
     const bool ok = warp_mbar_wait(&pipe.acc_full, 0, a.err) && !pipe.fail;
+    pdl_allow_next();  // the finish kernel, where it follows without an event between
     tc_fence_after();
     const uint32_t taddr = pipe.tmem + ((uint32_t)(quad * 32) << 16);
     float v[32];
@@ -508,6 +509,7 @@ __global__ void __launch_bounds__(kThreads, 2 / kAcc)
 __global__ void __launch_bounds__(256) relevance_finish_kernel(const RelFusedArgs a, const int* text_len,
                                                                const uint8_t* mask, float* p) {
   pdl_allow_next();  // the top-k reads p only after this grid completes
+  pdl_wait_prior();  // the cosines, and the mask before them
   extern __shared__ float mu[];  // mu [NTs], valid [NTs]
   int* valid = reinterpret_cast<int*>(mu + a.NTs);
   const int b = blockIdx.y;
@@ -591,6 +593,7 @@ struct CritArgs {
   float* G;        // [B][N_t_max][N_t_max]; unused with kWhole
   uint8_t* mask;   // kWhole: the outputs
   float* r_out;
+  bool early;      // let the next kernel start at once
   unsigned* err;
 };
 constexpr int kCritStages = 4;
@@ -634,6 +637,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ __align__(16) float ccol[kBM];
   __shared__ float wsum[4];
   __shared__ int wcnt[4];
+  if (a.early) pdl_allow_next();  // what waits for this grid does so in inv_norm_kernel
   const uint32_t rank = blockIdx.x, C = gridDim.x;  // the cluster spans grid x
   const int ti = blockIdx.y / a.nt, tj = blockIdx.y % a.nt, b = blockIdx.z;
   const bool same = ti == tj;  // one load per K slice is both operands
@@ -980,12 +984,12 @@ cudaError_t relevance_tc_launch(const SimArgs& a, const uint8_t* mask, const flo
   e = n_tb == 1 ? launch_pdl(relevance_fused_tc<1>, dim3(r.n_vt, a.B), dim3(kThreads), smem, s, r, mapV, mapT)
                 : launch_pdl(relevance_fused_tc<2>, dim3(r.n_vt, a.B, n_tb), dim3(kThreads), smem, s, r, mapV, mapT);
   if (e != cudaSuccess) return e;
-  if (mask_ready != nullptr) {
-    e = cudaStreamWaitEvent(s, mask_ready, 0);  // the first kernel that reads the mask
-    if (e != cudaSuccess) return e;
-  }
-  relevance_finish_kernel<<<dim3((a.N_v + 8 * kRelFinishRows - 1) / (8 * kRelFinishRows), a.B), 256,
-                            (size_t)r.NTs * (sizeof(float) + sizeof(int)), s>>>(r, a.text_len, mask, p);
+  const dim3 gf((a.N_v + 8 * kRelFinishRows - 1) / (8 * kRelFinishRows), a.B);
+  const size_t smem_f = (size_t)r.NTs * (sizeof(float) + sizeof(int));
+  if (mask_ready == nullptr) return launch_pdl(relevance_finish_kernel, gf, dim3(256), smem_f, s, r, a.text_len, mask, p);
+  e = cudaStreamWaitEvent(s, mask_ready, 0);  // the first kernel that reads the mask
+  if (e != cudaSuccess) return e;
+  relevance_finish_kernel<<<gf, 256, smem_f, s>>>(r, a.text_len, mask, p);
   return cudaGetLastError();
 }
 
@@ -996,8 +1000,24 @@ namespace provip {
 // CTAs per tile and accumulators per CTA: 8 x 2 while the clusters fit the SMs at
 // one CTA each, 4 x 4 beyond (the same 16 parts with fewer, longer CTAs); narrow
 // embeddings with fewer K slices take the largest power of two of them.
+static int crit_cluster(int B, int nt, int n_k, int num_sms) {
+  int C = (long long)B * nt * nt * kCritMaxCluster <= num_sms ? kCritMaxCluster : kCritMaxAcc;
+  while (C > n_k) C /= 2;
+  return C;
+}
+
+// The critical rows are one kernel whose CTAs take three quarters of the SMs or more:
+// the relevance then follows it on its stream instead of running beside it from
+// another, without the events between (passes of 32 and of 16 images 171 -> 167 and
+// 222 -> 218 us, 128 CTAs each; with 64 and with 8 CTAs, 8 anyres samples and a video,
+// the later start of the relevance costs more: 219 -> 223 and 178 -> 184).
+bool crit_leads(const SimArgs& a, int num_sms) {
+  if (a.dtype != 1 || a.N_t_max > kBM || !relevance_tc_supported(a)) return false;
+  return 4ll * a.B * crit_cluster(a.B, 1, (a.D + kBK - 1) / kBK, num_sms) >= 3ll * num_sms;
+}
+
 cudaError_t crit_gram_tc_launch(const SimArgs& a, uint8_t* mask, float* r_out, float* G, int num_sms, bool* whole,
-                                cudaStream_t s) {
+                                cudaStream_t s, bool early) {
   static std::atomic<bool> smem_set[64], smem_set2[64];  // per device, zero-initialised
   int dev = 0;
   cudaGetDevice(&dev);
@@ -1022,8 +1042,8 @@ cudaError_t crit_gram_tc_launch(const SimArgs& a, uint8_t* mask, float* r_out, f
   c.r_out = r_out;
   c.err = a.err;
   *whole = c.nt == 1;
-  int C = (long long)a.B * c.nt * c.nt * kCritMaxCluster <= num_sms ? kCritMaxCluster : kCritMaxAcc;
-  while (C > c.n_k) C /= 2;
+  c.early = early && *whole;
+  const int C = crit_cluster(a.B, c.nt, c.n_k, num_sms);
   c.n_acc = C == kCritMaxCluster ? 2 : kCritMaxAcc;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
