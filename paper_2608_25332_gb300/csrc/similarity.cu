@@ -27,8 +27,8 @@ __device__ __forceinline__ const T* row_ptr(const void* base, size_t row, int D)
 // ---------------------------------------------------------------------------
 // Sec. 4.2
 // ---------------------------------------------------------------------------
-// the fp32 text Gram: a cluster per 64 x 64 tile (simt_split.cuh), CTA c of it
-// writing rows [c * 64 / C, ..)
+// the fp32 text Gram: a cluster per 64 x 64 tile and part of K (simt_split.cuh;
+// gridDim.z parts, each its own G), CTA c of it writing rows [c * 64 / C, ..)
 __global__ void __launch_bounds__(split::kThreads, split::kCtasPerSm) crit_gram_kernel(const SimArgs a, int C, float* G) {
   extern __shared__ __align__(128) uint8_t ring[];
   __shared__ const float* arow[split::kTile];
@@ -46,8 +46,9 @@ __global__ void __launch_bounds__(split::kThreads, split::kCtasPerSm) crit_gram_
   }
   __syncthreads();
   int k0, k1;
-  split::share(a.D, rank, C, k0, k1);
+  split::share(a.D, blockIdx.z * C + rank, gridDim.z * C, k0, k1);
   split::tile_part<float>(arow, brow, k0, k1, ring, a.emb_t);
+  G += (size_t)blockIdx.z * a.B * a.N_t_max * a.N_t_max;
   split::cluster_sync();
   const int n_rows = split::kTile / C, c = c0 + (threadIdx.x & 15) * 4;
   for (int i = threadIdx.x >> 4; i < n_rows; i += split::kThreads / 16) {
@@ -72,6 +73,8 @@ __global__ void __launch_bounds__(split::kThreads, split::kCtasPerSm) crit_gram_
 // the CTAs are added in order. One CTA of 1024 threads per sample took 34 us for
 // 300 text rows.
 constexpr int kFinishCtas = 8;
+constexpr int kCritMaxParts = 2;  // parts of K that the fp32 text Gram may leave to this kernel,
+constexpr int kPartsReg = 4;      // for at most 32 * kPartsReg text rows
 constexpr int kFinishWarps = 8;
 constexpr size_t finish_smem(int N_t_max) { return (size_t)(kFinishWarps + 2) * N_t_max * sizeof(float); }
 __device__ __forceinline__ void finish_cluster_sync() {
@@ -79,7 +82,7 @@ __device__ __forceinline__ void finish_cluster_sync() {
                "barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 template <int kReg>
-__global__ void __launch_bounds__(32 * kFinishWarps) crit_finish_kernel(const SimArgs a, const float* G,
+__global__ void __launch_bounds__(32 * kFinishWarps) crit_finish_kernel(const SimArgs a, const float* G, int parts,
                                                                         uint8_t* mask, float* r_out) {
   extern __shared__ float sh[];  // part[kFinishWarps][Ntm], col[Ntm], rr[Ntm]
   float* col = sh + (size_t)kFinishWarps * a.N_t_max;
@@ -104,6 +107,19 @@ __global__ void __launch_bounds__(32 * kFinishWarps) crit_finish_kernel(const Si
       float v[kReg], m = -INFINITY, z = 0.f;
 #pragma unroll
       for (int q = 0; q < kReg; ++q) v[q] = lane + 32 * q < n ? Gb[(size_t)i * a.N_t_max + lane + 32 * q] : 0.f;
+      if constexpr (kReg <= kPartsReg) {
+        float w[kCritMaxParts - 1][kReg];  // the further parts, added in order
+#pragma unroll
+        for (int p = 1; p < kCritMaxParts; ++p)
+#pragma unroll
+          for (int q = 0; q < kReg; ++q)
+            w[p - 1][q] = p < parts && lane + 32 * q < n
+                              ? Gb[((size_t)p * a.B * a.N_t_max + i) * a.N_t_max + lane + 32 * q] : 0.f;
+#pragma unroll
+        for (int p = 1; p < kCritMaxParts; ++p)
+#pragma unroll
+          for (int q = 0; q < kReg; ++q) v[q] += w[p - 1][q];
+      }
 #pragma unroll
       for (int q = 0; q < kReg; ++q)
         if (lane + 32 * q < n) m = fmaxf(m, v[q]);
@@ -1052,11 +1068,20 @@ __global__ void __launch_bounds__(kMeanThreads, 8)
 
 cudaError_t crit_text_launch(const SimArgs& a, uint8_t* mask, float* r_out, float* G, int num_sms,
                              cudaStream_t s, bool early) {
+  int parts = 1;
   if (a.dtype == 0) {
     const int nt = (a.N_t_max + split::kTile - 1) / split::kTile;
     const int C = split::cluster_size((long long)a.B * nt * nt, a.D, num_sms);
+    // where the largest clusters leave SMs idle, K in two parts, by the clusters' own rule
+    // (at least 1024 elements a part, so that G's region holds them): the relevance of one
+    // image waits for its 64 x 64 Gram over 4096 elements, and the pass went from 104.7 to
+    // 98.5 us (four parts: the same, the relevance no longer waits)
+    while (C == split::kMaxCluster && a.N_t_max <= 32 * kPartsReg && parts < kCritMaxParts &&
+           2ll * parts * C * a.B * nt * nt <= (long long)split::kCtasPerSm * num_sms &&
+           a.D / (2 * parts * C) >= 4 * split::kKT)
+      parts *= 2;
     static std::atomic<bool> set[64];  // per device, zero-initialised
-    const cudaError_t e = split::launch(crit_gram_kernel, split::kSmem<float>, set, dim3((unsigned)(C * nt * nt), (unsigned)a.B), C, s, a, C, G);
+    const cudaError_t e = split::launch(crit_gram_kernel, split::kSmem<float>, set, dim3((unsigned)(C * nt * nt), (unsigned)a.B, (unsigned)parts), C, s, a, C, G);
     if (e != cudaSuccess) return e;
   } else {
     bool whole = false;
@@ -1084,9 +1109,9 @@ cudaError_t crit_text_launch(const SimArgs& a, uint8_t* mask, float* r_out, floa
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (a.N_t_max <= 32 * 4) return cudaLaunchKernelEx(&cfg, crit_finish_kernel<4>, a, G, mask, r_out);
-  if (a.N_t_max <= 32 * 16) return cudaLaunchKernelEx(&cfg, crit_finish_kernel<16>, a, G, mask, r_out);
-  return cudaLaunchKernelEx(&cfg, crit_finish_kernel<0>, a, G, mask, r_out);
+  if (a.N_t_max <= 32 * 4) return cudaLaunchKernelEx(&cfg, crit_finish_kernel<4>, a, G, parts, mask, r_out);
+  if (a.N_t_max <= 32 * 16) return cudaLaunchKernelEx(&cfg, crit_finish_kernel<16>, a, G, parts, mask, r_out);
+  return cudaLaunchKernelEx(&cfg, crit_finish_kernel<0>, a, G, parts, mask, r_out);
 }
 
 // 1/|e_j| (0 for a zero row) of the kept rows j = keep_idx[b][q] only, into

@@ -13,8 +13,8 @@
 // the ring took 2.4 us per step and had all of K to itself:
 // 311 us for the Gram of 64 text rows of 4096 elements, 367 for their products
 // with 576 visual rows, 411 for 384 pruned by 192 kept rows, on 1, 9 and 15 CTAs;
-// this form takes 21, 25 and 37 (8, 72 and 144 CTAs), about 42% of the issue slots
-// between the ring's start and the last step. The shorter sums are closer to 64
+// this form takes 21 (8 CTAs; the Gram now takes two parts of 8), 25 and 37 (72 and 144
+// CTAs), about 42% of the issue slots between the ring's start and the last step. The shorter sums are closer to 64
 // bits: p to 1.2e-7 where it was 1.1e-6.
 #pragma once
 

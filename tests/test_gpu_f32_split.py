@@ -92,3 +92,30 @@ def test_merge_bf16_past_the_tensor_core_form():
     a_ref, mg_ref = oracle.merge(Evn, keeps[0])
     check_merge(Evn, keeps[0], assign[0].cpu().numpy(), merged[0].double().cpu().numpy(), "bf16", "merge bf16 FFMA",
                 a_ref, np.setdiff1d(np.arange(N_v), keeps[0]), mg_ref=mg_ref)
+
+
+@pytest.mark.parametrize("tls,T,D", [
+    ((64,), 64, 2048),        # one tile, K in two parts of eight shares
+    ((65, 40), 65, 2056),     # four tiles, shares that end inside a K step
+    ((128, 1, 0), 128, 4096),
+    ((20,), 20, 1024),        # shares too short for parts
+    ((129,), 129, 4096),      # more text rows than the finish adds parts for
+])
+def test_critical_rows_f32(tls, T, D):
+    rng = np.random.default_rng(T + D)
+    # rows whose products stay near 1, so that the softmax is no row's own diagonal
+    et = torch.from_numpy((rng.standard_normal((len(tls), T, D)) / D ** 0.5).astype(np.float32))
+    for b, t in enumerate(tls):
+        et[b, t:] = float("nan")
+    mask, r = P.provip_crit_text(et.to(DEV), torch.tensor(tls, dtype=torch.int32, device=DEV), want_r=True)
+    torch.cuda.synchronize()
+    for b, t in enumerate(tls):
+        assert not mask[b, t:].any()
+        if t == 0:
+            continue
+        x = et[b, :t].double()
+        ref = torch.softmax(x @ x.T, 1).mean(0).numpy()
+        assert_close_rel(r[b, :t].cpu().numpy(), ref, 1e-5, f"r T={T} D={D} [{b}]")
+        sure = np.abs(ref - ref.mean()) > 1e-5 * ref.mean()
+        got = mask[b, :t].cpu().numpy().astype(bool)
+        assert np.array_equal(got[sure], (ref > ref.mean())[sure]) or t == 1
