@@ -593,7 +593,7 @@ struct CritArgs {
   float* G;        // [B][N_t_max][N_t_max]; unused with kWhole
   uint8_t* mask;   // kWhole: the outputs
   float* r_out;
-  bool early;      // let the next kernel start at once
+  bool early;      // let the next kernel start beside this one
   unsigned* err;
 };
 constexpr int kCritStages = 4;
@@ -637,7 +637,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ __align__(16) float ccol[kBM];
   __shared__ float wsum[4];
   __shared__ int wcnt[4];
-  if (a.early) pdl_allow_next();  // what waits for this grid does so in inv_norm_kernel
   const uint32_t rank = blockIdx.x, C = gridDim.x;  // the cluster spans grid x
   const int ti = blockIdx.y / a.nt, tj = blockIdx.y % a.nt, b = blockIdx.z;
   const bool same = ti == tj;  // one load per K slice is both operands
@@ -664,6 +663,12 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // Only now that this CTA has its tensor memory: the text norms that this lets start
+  // let the relevance start, whose CTAs take tensor memory and keep it until the
+  // norms, and through them this grid, have completed. A CTA of this grid that still
+  // waited for its own could wait for ever. What waits for this grid does so in
+  // inv_norm_kernel.
+  if (a.early) pdl_allow_next();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float* tile = reinterpret_cast<float*>(stages);  // [128][kCritLd], once the MMAs are done
   if (warp == 0) {

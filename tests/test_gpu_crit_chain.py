@@ -16,6 +16,7 @@ DEV = "cuda:0"
     (20, 300, 128, 256, 100),  # clusters of 4 (as many K slices): 80 CTAs, the side stream
     (29, 257, 128, 264, 64),   # clusters of 4: 116 CTAs; a ragged last K slice and visual tile
     (120, 40, 7, 64, 9),       # one K slice, one CTA a sample
+    (64, 70, 128, 256, 20),    # clusters of 4, 512 columns of tensor memory each: 256 CTAs, more than SMs
 ])
 def test_pass_gives_the_bits_of_separate_calls(B, N_v, N_t, D, keep):
     __graft_entry__.build()
