@@ -351,6 +351,7 @@ __global__ void __launch_bounds__(pair_threads(kDirect), 1)
         const int s = it % kPairStages;
         const uint32_t ph = (uint32_t)(it / kPairStages) & 1u;
         if (lane == 0) ok = !pipe.fail && mbar_wait(&pipe.empty[s], ph ^ 1u, a.err);
+        __syncwarp();  // orders the other lanes' loads after lane 0's wait; the shuffle alone does not
         ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
         if (!ok) {
           pipe.fail = 1;
