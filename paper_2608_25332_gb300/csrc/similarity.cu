@@ -712,7 +712,10 @@ constexpr int kMeanRank = 256;  // members of a long centroid that are ordered b
 constexpr int kMeanWin = 1024;
 constexpr int kMeanThreads = 128;
 constexpr size_t kMeanSmem = (size_t)kMeanDeep * kMeanThreads * 16;
-constexpr int kSortSmemKeep = 6144;  // centroids whose counters the sort keeps in shared memory (48 KiB)
+// centroids whose counters the sort keeps in shared memory: 8 bytes each beside the
+// warps' totals, in the 48 KiB that a kernel has without an attribute
+constexpr int kSortWarps = 32;
+constexpr int kSortSmemKeep = (48 * 1024 - kSortWarps * (int)sizeof(int)) / (2 * (int)sizeof(int));
 
 // Counting sort of one sample's rows by centroid (one CTA of 1024 threads):
 // count[b][a] = rows assigned to a, offset[b][.] its exclusive scan, and
@@ -727,7 +730,7 @@ __global__ void __launch_bounds__(1024) merge_sort_kernel(const int* assign, int
                                                           int* offset, int* cursor, int* members, int* n_long,
                                                           int* long_list) {
   extern __shared__ int sort_sm[];  // kSmem: counts [keep], then offsets / cursors [keep]
-  __shared__ int warp_tot[32];
+  __shared__ int warp_tot[kSortWarps];
   pdl_wait_prior();  // the assignment comes from the kernel before
   pdl_allow_next();
   const int b = blockIdx.x;
