@@ -166,9 +166,9 @@ int provip_topk(const float *scores, int B, int N, int k, int *idx_out, void *st
  *   assign_out [B, N_v] int32: position in keep_idx of row j's centroid (kept
  *              rows map to their own position).
  *   merged_out [B, keep, D] dtype or NULL (assignment only). fp32 sums are
- *              accumulated as pairs of floats with every rounding error kept
- *              (in double where a sum is not finite in fp32), bf16 sums in
- *              float, both in ascending row order; the mean is rounded to
+ *              accumulated as triples of floats, no less accurately than in
+ *              double (in double where a sum is not finite in fp32), bf16 sums
+ *              in float, both in ascending row order; the mean is rounded to
  *              nearest-even.
  * Requires D % 8 == 0, D <= 8192. */
 size_t provip_merge_workspace_size(int B, int N_v, int D, int keep);

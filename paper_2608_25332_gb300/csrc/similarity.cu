@@ -816,37 +816,72 @@ __device__ __forceinline__ void add16(double* acc, const uint4& u, const float*)
   acc[2] += (double)__uint_as_float(u.z);
   acc[3] += (double)__uint_as_float(u.w);
 }
-// The running sum of fp32 values as an unevaluated pair hi + lo: every addition's
-// rounding error is recovered exactly (Knuth's TwoSum) and kept in lo, so the sum
-// is good to about 2^-48, and its mean, rounded once, to the same half ulp as one
-// taken in double. The GPU adds 128 floats per SM clock but only two doubles: in
-// double, with a division per element, the means of one fp32 image (576 rows of
-// 4096) took 66 us; this takes 14, every mean still correctly rounded. A sum that leaves fp32's range or meets an infinity or a NaN
-// is taken again in double.
-struct Sum2 {
-  float hi, lo;
+// The running sum of fp32 values as an unevaluated hi + mid + lo: the rounding error of
+// every addition to hi is recovered exactly (Knuth's TwoSum) and added to mid, that
+// addition's error to lo. lo itself is rounded, and settle(), every 256 rows, keeps it
+// below an ulp of mid, so n rows are added to within n 2^-56 of the largest partial
+// sum, where double allows n 2^-53; and acc_mean rounds the quotient once. Sums of
+// 1 to 9000 rows, spread over 2^60, cancelling or subnormal, were all correctly
+// rounded; in double 1 in 500 of those that cancel to 1e-7 of their largest partial
+// were not, and as pairs of floats 1 in 4. The GPU adds 128 floats per SM clock but
+// only two doubles: in double, with a division per element, the means of one fp32 image
+// (576 rows of 4096) took 66 us; as pairs or triples they take 14, and as triples the
+// merge of 16 such images takes 322 us where pairs took 314. A sum that leaves fp32's
+// range or meets an infinity or a NaN is taken again in double.
+struct Sum3 {
+  float hi, mid, lo;
 };
-__device__ __forceinline__ void two_sum(Sum2& s, float x) {
-  const float t = s.hi + x, z = t - s.hi;
-  s.lo += (s.hi - (t - z)) + (x - z);
-  s.hi = t;
+// a + b = the returned sum + e, exactly
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+  const float t = a + b, z = t - a;
+  e = (a - (t - z)) + (b - z);
+  return t;
 }
-__device__ __forceinline__ void add16(Sum2* acc, const uint4& u, const float*) {
-  two_sum(acc[0], __uint_as_float(u.x));
-  two_sum(acc[1], __uint_as_float(u.y));
-  two_sum(acc[2], __uint_as_float(u.z));
-  two_sum(acc[3], __uint_as_float(u.w));
+__device__ __forceinline__ void add1(Sum3& s, float x) {
+  float e, f;
+  s.hi = two_sum(s.hi, x, e);
+  s.mid = two_sum(s.mid, e, f);
+  s.lo += f;
+}
+__device__ __forceinline__ void add16(Sum3* acc, const uint4& u, const float*) {
+  add1(acc[0], __uint_as_float(u.x));
+  add1(acc[1], __uint_as_float(u.y));
+  add1(acc[2], __uint_as_float(u.z));
+  add1(acc[3], __uint_as_float(u.w));
+}
+constexpr int kSettleRows = 256;
+__device__ __forceinline__ void settle(float&) {}
+__device__ __forceinline__ void settle(double&) {}
+__device__ __forceinline__ void settle(Sum3& s) {
+  float e;
+  s.hi = two_sum(s.hi, s.mid, e);
+  s.mid = two_sum(e, s.lo, s.lo);
+  s.hi = two_sum(s.hi, s.mid, s.mid);
+  s.mid = two_sum(s.mid, s.lo, s.lo);
 }
 __device__ __forceinline__ void acc_zero(float& a) { a = 0.f; }
 __device__ __forceinline__ void acc_zero(double& a) { a = 0.0; }
-__device__ __forceinline__ void acc_zero(Sum2& a) { a.hi = a.lo = 0.f; }
-// sum / n; a pair that is not finite clears ok
+__device__ __forceinline__ void acc_zero(Sum3& a) { a.hi = a.mid = a.lo = 0.f; }
+// sum / n; a triple that is not finite clears ok
 __device__ __forceinline__ float acc_mean(float a, int n, bool&) { return a / (float)n; }
 __device__ __forceinline__ float acc_mean(double a, int n, bool&) { return (float)(a / (double)n); }
-__device__ __forceinline__ float acc_mean(const Sum2& a, int n, bool& ok) {
-  if (!(fabsf(a.hi) <= 3.0e38f && fabsf(a.lo) <= 3.0e38f)) ok = false;
-  const float fn = (float)n, q = a.hi / fn;
-  return q + (fmaf(-q, fn, a.hi) + a.lo) / fn;  // the quotient's remainder is exact
+__device__ __forceinline__ float acc_mean(Sum3 a, int n, bool& ok) {
+  if (!(fabsf(a.hi) <= 3.0e38f && fabsf(a.mid) <= 3.0e38f && fabsf(a.lo) <= 3.0e38f)) ok = false;
+  settle(a);
+  if (!(fabsf(a.hi) >= 0x1p-90f)) {  // the remainders below could be subnormal
+    return a.hi == 0.f ? 0.f : (float)(((double)a.hi + (double)a.mid + (double)a.lo) / (double)n);
+  }
+  // q, the quotient of hi to about an ulp; c, of what q leaves (an exact remainder, as
+  // n < 2^22) and of mid; d, of what both leave
+  const float fn = (float)n, inv = 1.f / fn, q = a.hi * inv;
+  float t, e;
+  const float r = two_sum(fmaf(-q, fn, a.hi), a.mid, t), c = r * inv;
+  const float d = (fmaf(-c, fn, r) + (t + a.lo)) * inv;
+  // c + d rounded to odd, so that q + (c + d), rounded to nearest, is rounded only once
+  const float u = two_sum(c, d, e);
+  int bits = __float_as_int(u);
+  if (e != 0.f && (bits & 1) == 0) bits += (e > 0.f) == (u > 0.f) ? 1 : -1;
+  return q + __int_as_float(bits);
 }
 // 16 bytes of a row from fp32 values, rounded to nearest even
 __device__ __forceinline__ void store16(__nv_bfloat16* p, const float* v) {
@@ -898,7 +933,12 @@ __device__ __forceinline__ bool mean_long(const SimArgs& a, int b, int n, const 
       fetch(i + kMeanDeep - 1);
       cp_async_wait<kMeanDeep - 1>();
       if (has) add16(acc, mine[(i % kMeanDeep) * kMeanThreads], E);
+      if ((i + 1) % kSettleRows == 0)
+#pragma unroll
+        for (int e = 0; e < kVec; ++e) settle(acc[e]);
     }
+#pragma unroll
+    for (int e = 0; e < kVec; ++e) settle(acc[e]);
     cp_async_wait<0>();
   };
   if (n <= kMeanRank) {
@@ -1312,7 +1352,7 @@ cudaError_t merge_launch(const SimArgs& a, const int* keep_idx, int keep, const 
       return launch_pdl(kernel, gm, dim3(kMeanThreads), kMeanSmem, s, a, (const int*)cnt, (const int*)off,
                         (const int*)mem, keep, merged, (const int*)n_long, (const int*)lng, n_lc);
     };
-    const cudaError_t em = a.dtype == 0 ? go(merge_mean_kernel<float, Sum2>)
+    const cudaError_t em = a.dtype == 0 ? go(merge_mean_kernel<float, Sum3>)
                                         : go(merge_mean_kernel<__nv_bfloat16, float>);
     if (em != cudaSuccess) return em;
   }

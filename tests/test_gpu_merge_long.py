@@ -2,6 +2,8 @@
 own CTAs, a column slice each): member counts at the limit between the two
 paths and past one window of the ordering bitmap, rows of every configuration
 and of a partial last slice, against the oracle."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -84,3 +86,34 @@ def test_fp32_means_of_huge_and_non_finite_values(keep, D):
     assert np.array_equal(ref[~fin & ~np.isnan(ref)], got[~fin & ~np.isnan(ref)])
     # one unit in the last place (the sums' own rounding is 2^-24 below it)
     assert np.all(np.abs(got[fin] - ref[fin]) <= np.spacing(np.abs(ref[fin]).astype(np.float32)))
+
+
+@pytest.mark.parametrize("n", [2, 3, 16, 17, 256, 257, 700, 1500])
+@pytest.mark.parametrize("D", [264, 2056])
+def test_fp32_means_are_correctly_rounded(n, D):
+    """One centroid that gathers n rows (its group's list, ranked, and by windows): columns
+    that cancel to a small part of their largest partial sum, columns spread over 2^60,
+    whole numbers (ties) and subnormals. Every mean is the exact one rounded once: half a
+    unit in the last place, with 2^-50 for the reference's own two roundings."""
+    rng = np.random.default_rng(100 * n + D)
+    Ev = rng.standard_normal((n, D)).astype(np.float32)
+    first, last = rng.permutation(n)[:2]
+    for c in range(D):
+        k = c % 4
+        if k == 0:
+            big = np.float32(10.0 ** rng.uniform(4, 12))
+            Ev[first, c], Ev[last, c] = big, -big
+        elif k == 1:
+            Ev[:, c] = np.ldexp(Ev[:, c], rng.integers(-30, 31, n))
+        elif k == 2:
+            Ev[:, c] = rng.integers(0, 8192, n)
+        elif c < 32:
+            Ev[:, c] = np.ldexp(Ev[:, c], rng.integers(-140, -120, n))
+    keeps = np.array([[int(rng.integers(0, n))]], np.int32)
+    _, merged = P.provip_merge(torch.from_numpy(Ev[None]).to(DEV), torch.from_numpy(keeps).to(DEV))
+    torch.cuda.synchronize()
+    got = merged[0, 0].cpu().numpy()
+    for c in range(D):
+        ref = math.fsum(Ev[:, c].astype(np.float64).tolist()) / n
+        ulp = float(np.spacing(np.abs(np.float32(ref))))
+        assert abs(float(got[c]) - ref) <= 0.5 * ulp + 2.0 ** -50 * abs(ref), (n, c, got[c], ref)
