@@ -49,6 +49,7 @@
 
 #include <math.h>
 
+#include <algorithm>
 #include <mutex>
 #include <vector>
 
@@ -590,28 +591,33 @@ void merge_pair_enable(int on) { g_pair_enabled.store(on ? 1 : 0); }
 // of width 3584 keeps the copy (179 us against 182). Slower than either: 16-byte
 // cp.async by eight warps (243 us for the 32 images: too few requests fit in flight
 // beside the ring), and copying the kept rows alone (191 us).
-constexpr double kBoxPace[2] = {780.0, 960.0};        // by halves
-constexpr double kDirectPace[2] = {1090.0, 1400.0};
+constexpr long long kBoxPace[2] = {780, 960};         // by halves
+constexpr long long kDirectPace[2] = {1090, 1400};
 constexpr double kCopyClocksPerByte = 1.9 / 7200;     // 7.2 TB/s, read and write, at 1.9 GHz
-static bool merge_pair_search(int halves, bool direct, int B, int n_pruned, int keep, int D, int num_sms,
-                              MergePairPlan* p) {
-  if (B < 1 || n_pruned < 1 || keep < 1 || D < 1 || num_sms < 2) return false;
+// plan[0]: the best split for boxes of the copy, plan[1]: for rows read where they lie
+// (ok: found). Both forms share each candidate's deal, which is walked tile by tile, and
+// only where the mean load of its pairs is below the best busiest pair so far.
+static void merge_pair_search(int halves, int B, int n_pruned, int keep, int D, int num_sms, MergePairPlan* plan,
+                              bool* ok) {
+  ok[0] = ok[1] = false;
+  if (B < 1 || n_pruned < 1 || keep < 1 || D < 1 || num_sms < 2) return;
   const int quad_rows = halves * 2 * kBM;
   const int n_quads = (n_pruned + quad_rows - 1) / quad_rows;
-  const double pace = direct ? kDirectPace[halves - 1] : kBoxPace[halves - 1];
-  const double copy = direct ? 0.0 : kCopyClocksPerByte * 4.0 * B * (n_pruned + keep) * (double)D;
+  const long long pace[2] = {kBoxPace[halves - 1], kDirectPace[halves - 1]};
+  const double copy[2] = {kCopyClocksPerByte * 4.0 * B * (n_pruned + keep) * (double)D, 0.0};
   const long long Q = (long long)B * n_quads;
   const int max_pairs = num_sms / 2;
   const long long n_k = (D + kBK - 1) / kBK;
-  if (Q > (1 << 20)) return false;
-  double best = -1.0;
-  std::vector<double> load;
+  if (Q > (1 << 20)) return;
+  // whether the last group of a sample, or every group, holds one half
+  const bool last_one = halves == 1 || n_pruned - (n_quads - 1) * quad_rows <= 2 * kBM, all_one = halves == 1;
+  long long best[2] = {0, 0};
+  std::vector<long long> load[2];
   auto consider = [&](int n_lo, long long x_hi) {
     const int n_hi = n_lo + (x_hi > 0 ? 1 : 0);
     if (n_lo < 1 || n_hi > kMergeMaxSplit || x_hi < 0 || x_hi >= Q) return;
     MergePairPlan c;
     c.halves = halves;
-    c.direct = direct;
     c.n_quads = n_quads;
     c.Q = (int)Q;
     c.n_lo = n_lo;
@@ -622,32 +628,69 @@ static bool merge_pair_search(int halves, bool direct, int B, int n_pruned, int 
     c.P = (int)(T < max_pairs ? T : max_pairs);
     c.n_slots = n_hi;
     c.n_heights = 0;
+    // clocks of a range's tile by form, number of ranges (n_lo, n_hi) and halves of its
+    // group, and of a group's tiles together
+    long long cost[2][2][2][kMergeMaxSplit], row[2][2][2] = {};
     for (int n = n_lo; n <= n_hi; ++n)
       for (int t = 0; t < n; ++t) {
         const int nv = pair_range_start(t + 1, n, keep) - pair_range_start(t, n, keep);
         if (nv < 1 || nv > kPairMaxN) return;
-        const int h = (nv + 31) / 32 * 16;  // B rows per CTA
+        const int N = (nv + 31) / 32 * 32, h = N / 2;  // B rows per CTA
         int j = 0;
         while (j < c.n_heights && c.heights[j] != h) ++j;
         if (j == c.n_heights) {
           if (j == kMergePairHeights) return;
           c.heights[c.n_heights++] = h;
         }
+        for (int f = 0; f < 2; ++f)
+          for (int two = 0; two < 2; ++two) {
+            const long long v = n_k * std::max((two ? 4ll : 2ll) * N, pace[f]) + 9000;
+            cost[f][n - n_lo][two][t] = v;
+            row[f][n - n_lo][two] += v;
+          }
       }
-    load.assign(c.P, 0.0);
-    for (int pr = 0; pr < c.P; ++pr) {
-      for (int r = 0, k; (k = pair_deal_tile(c, pr, r)) >= 0; ++r) {
-        const PairTile g = pair_tile(c, n_pruned, keep, k);
-        load[pr] += (double)n_k * fmax((g.has1 ? 4.0 : 2.0) * g.N, pace) + 9000.0;
+    // groups of one half among the first x_hi and among the others
+    const long long one_hi = all_one ? x_hi : (last_one ? x_hi / n_quads : 0);
+    const long long one_lo = (all_one ? Q : (last_one ? B : 0)) - one_hi;
+    bool try_form[2];
+    for (int f = 0; f < 2; ++f) {
+      const int hi = n_hi - n_lo;
+      const long long total = one_hi * row[f][hi][0] + (x_hi - one_hi) * row[f][hi][1] + one_lo * row[f][0][0] +
+                              (Q - x_hi - one_lo) * row[f][0][1];
+      try_form[f] = !ok[f] || total < best[f] * c.P;  // else its busiest pair has at least best[f]
+    }
+    if (!try_form[0] && !try_form[1]) return;
+    // the tiles in order (pair_tile), dealt in snake order (pair_deal_tile)
+    for (int f = 0; f < 2; ++f) load[f].assign((size_t)c.P, 0);
+    int pr = 0, step = 1;
+    for (int part = 0; part < 2; ++part) {
+      const long long q0 = part == 0 ? x_hi : 0, q1 = part == 0 ? Q : x_hi;
+      int in_sample = (int)(q0 % n_quads);
+      for (long long q = q0; q < q1; ++q) {
+        const int two = !(all_one || (last_one && in_sample == n_quads - 1));
+        if (++in_sample == n_quads) in_sample = 0;
+        const long long *c0 = cost[0][part][two], *c1 = cost[1][part][two];
+        for (int t = 0; t < n_lo + part; ++t) {
+          load[0][pr] += c0[t];
+          load[1][pr] += c1[t];
+          pr += step;
+          if (pr == c.P || pr < 0) {
+            step = -step;
+            pr += step;
+          }
+        }
       }
     }
-    double worst = 0.0;
-    for (double l : load) worst = fmax(worst, l);
-    worst += copy;
-    if (best < 0 || worst < best) {
-      best = worst;
-      c.clocks = worst;
-      *p = c;
+    for (int f = 0; f < 2; ++f) {
+      if (!try_form[f]) continue;
+      const long long worst = *std::max_element(load[f].begin(), load[f].end());
+      if (!ok[f] || worst < best[f]) {
+        ok[f] = true;
+        best[f] = worst;
+        plan[f] = c;
+        plan[f].direct = f == 1;
+        plan[f].clocks = (double)worst + copy[f];
+      }
     }
   };
   for (int n_lo = (keep + kPairMaxN - 1) / kPairMaxN; n_lo <= kMergeMaxSplit; ++n_lo) {
@@ -657,52 +700,52 @@ static bool merge_pair_search(int halves, bool direct, int B, int n_pruned, int 
       if (x_hi > 0 && x_hi < Q) consider(n_lo, x_hi);
     }
   }
-  return best >= 0;
 }
 
-// The search simulates every candidate's deal (tens to hundreds of
-// microseconds of host time): its results are kept per shape and form, the last
-// kPlanCache of them, for the calls that follow.
+// The searches take 3 to 7 us of host time for the shapes above and 7 for 64 x 2880 rows
+// (four searches that dealt every candidate took 120, 400 and 2600): their results are
+// kept per shape, the last kPlanCache shapes, for the calls that follow.
 namespace {
-constexpr int kPlanCache = 32;
+constexpr int kPlanCache = 16;
 struct PlanEntry {
-  int halves, B, n_pruned, keep, D, num_sms;
-  bool ok;
-  MergePairPlan plan;
+  int B, n_pruned, keep, D, num_sms;
+  bool ok[2];             // by halves - 1
+  MergePairPlan plan[2];
 };
 std::mutex g_plan_mu;
 PlanEntry g_plans[kPlanCache];
 int g_plan_n = 0, g_plan_next = 0;
 }  // namespace
 
-static bool plan_of(int halves, int B, int n_pruned, int keep, int D, int num_sms, MergePairPlan* p) {
+// both group sizes' plans, each in the form with the fewer clocks
+static PlanEntry plans_of(int B, int n_pruned, int keep, int D, int num_sms) {
   {
     std::lock_guard<std::mutex> lock(g_plan_mu);
     for (int i = 0; i < g_plan_n; ++i) {
       const PlanEntry& e = g_plans[i];
-      if (e.halves == halves && e.B == B && e.n_pruned == n_pruned && e.keep == keep && e.D == D &&
-          e.num_sms == num_sms) {
-        if (e.ok) *p = e.plan;
-        return e.ok;
-      }
+      if (e.B == B && e.n_pruned == n_pruned && e.keep == keep && e.D == D && e.num_sms == num_sms) return e;
     }
   }
-  MergePairPlan plan;
-  bool ok = merge_pair_search(halves, false, B, n_pruned, keep, D, num_sms, &plan);
-  MergePairPlan direct;
-  if (merge_pair_search(halves, true, B, n_pruned, keep, D, num_sms, &direct) && (!ok || direct.clocks < plan.clocks)) {
-    plan = direct;
-    ok = true;
+  PlanEntry e{B, n_pruned, keep, D, num_sms, {}, {}};
+  for (int h = 0; h < 2; ++h) {
+    MergePairPlan form[2];
+    bool ok[2];
+    merge_pair_search(h + 1, B, n_pruned, keep, D, num_sms, form, ok);
+    e.ok[h] = ok[0] || ok[1];
+    if (e.ok[h]) e.plan[h] = ok[1] && (!ok[0] || form[1].clocks < form[0].clocks) ? form[1] : form[0];
   }
   std::lock_guard<std::mutex> lock(g_plan_mu);
-  PlanEntry& e = g_plans[g_plan_next];
-  e = PlanEntry{halves, B, n_pruned, keep, D, num_sms, ok, plan};
+  g_plans[g_plan_next] = e;
   g_plan_next = (g_plan_next + 1) % kPlanCache;
   if (g_plan_n < kPlanCache) ++g_plan_n;
-  if (ok) *p = plan;
-  return ok;
+  return e;
 }
 
+static bool plan_of(int halves, int B, int n_pruned, int keep, int D, int num_sms, MergePairPlan* p) {
+  const PlanEntry e = plans_of(B, n_pruned, keep, D, num_sms);
+  if (e.ok[halves - 1]) *p = e.plan[halves - 1];
+  return e.ok[halves - 1];
+}
 bool merge_pair_plan(int B, int n_pruned, int keep, int D, int num_sms, MergePairPlan* p) {
   return plan_of(2, B, n_pruned, keep, D, num_sms, p);
 }
@@ -715,11 +758,13 @@ bool merge_pair_half_plan(int B, int n_pruned, int keep, int D, int num_sms, Mer
 // 32 of 384 by 192 (width 5120): 50 -> 44. 8 of 1920 by 960 keep 512-row groups (84 us): 256-row
 // tiles would take four rounds of the pairs instead of two.
 bool merge_pair_best(int B, int n_pruned, int keep, int D, int num_sms, MergePairPlan* p) {
-  MergePairPlan half;
-  const bool two = merge_pair_plan(B, n_pruned, keep, D, num_sms, p);
-  const bool one = merge_pair_half_plan(B, n_pruned, keep, D, num_sms, &half);
-  if (one && (!two || half.clocks < p->clocks)) *p = half;
-  return two || one;
+  const PlanEntry e = plans_of(B, n_pruned, keep, D, num_sms);
+  if (e.ok[0] && (!e.ok[1] || e.plan[0].clocks < e.plan[1].clocks)) {
+    *p = e.plan[0];
+  } else if (e.ok[1]) {
+    *p = e.plan[1];
+  }
+  return e.ok[0] || e.ok[1];
 }
 
 bool merge_pair_usable(const SimArgs& a) {

@@ -38,6 +38,30 @@ def test_chosen_forms(checker):
     assert _forms(checker, [(*s, 152) for s, _ in FORMS]) == [f for _, f in FORMS]
 
 
+def _search(checker, shapes):
+    r = subprocess.run([checker, "search", *(str(v) for s in shapes for v in s)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+    return [float(line.split()[1]) for line in r.stdout.splitlines()]
+
+
+def test_plans_are_the_full_searchs(checker):
+    """Both group sizes' plans are those of a search that deals every candidate's tiles."""
+    rng = np.random.default_rng(11)
+    shapes = [(*s, 152) for s, _ in FORMS] + [(3, 257, 1, 64, 152), (2, 513, 256, 64, 152), (1, 600, 1, 64, 2)]
+    for _ in range(60):
+        N_v = int(rng.integers(2, 6000))
+        shapes.append((int(rng.integers(1, 40)), N_v, int(rng.integers(1, min(N_v - 1, 5000) + 1)),
+                       8 * int(rng.integers(1, 600)), 2 * int(rng.integers(1, 90))))
+    assert len(_search(checker, shapes)) == len(shapes)
+
+
+def test_a_new_shape_costs_less_than_one_full_search(checker):
+    """Host time of a shape not seen before against that of one search that deals every
+    candidate's tiles (measured 0.02 to 0.4)."""
+    shapes = [(8, 2880, 960, 4096, 152), (1, 9216, 2304, 3584, 152), (4, 1443, 481, 4096, 152), (64, 2880, 960, 4096, 152)]
+    assert max(_search(checker, shapes)) < 1
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("B,N_v,D,keep,halves", [
     (32, 258, 64, 1, 1),      # a second group of one row; one kept row; one K slice
