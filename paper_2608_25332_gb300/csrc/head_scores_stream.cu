@@ -233,7 +233,9 @@ __global__ void __launch_bounds__(kThreads, 2)
     float cn = 0.f, cmean = 0.f, cm2 = 0.f;
     for (int it = 0; it < n_it; ++it) {
       const int buf = it & 1;
+      // every lane polls; if one gives up, none waits again
       if (!failed) failed = !mbar_wait(&ctl.acc_full[buf], (uint32_t)(it >> 1) & 1u, a.err);
+      failed = __any_sync(0xffffffffu, failed);
       __syncwarp();
       tc_fence_after();
       if (it == nA) {

@@ -1,4 +1,4 @@
-"""Waits that one lane makes for its warp, read from the kernels' source (CPU only)."""
+"""Waits that a warp shares, read from the kernels' source (CPU only)."""
 import glob
 import os
 import re
@@ -24,3 +24,13 @@ def test_a_lanes_wait_is_shared_behind_a_warp_barrier(path):
         share = re.search(r"__shfl_sync\([^;]*\b" + m.group(1) + r"\b", after)
         assert share, m.group(0)
         assert "__syncwarp();" in after[:share.start()], f"{os.path.basename(path)}: {m.group(0)}"
+
+
+def test_a_wait_of_every_lane_is_voted_on():
+    """The streaming head scores' workers poll with every lane and treat the outcome as the
+    warp's: where one lane gives up, no lane may go on waiting at the next chunk."""
+    code = _code(os.path.join(CSRC, "head_scores_stream.cu"))
+    waits = list(re.finditer(r"if \(!failed\) failed = !mbar_wait\([^;]*;", code))
+    assert len(waits) == 1
+    rest = code[waits[0].end():].lstrip()
+    assert rest.startswith("failed = __any_sync(0xffffffffu, failed);")
