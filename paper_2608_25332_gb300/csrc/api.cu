@@ -480,16 +480,9 @@ extern "C" int provip_selftest_wait_timeout(void* stream) {
 // ===========================================================================
 // pre-LLM pass
 // ===========================================================================
-// the text Gram's workspace: 16 parts of it up to 128 text rows, one beyond (what
-// its kernels needed once; they use one part at most, and a caller that kept a
-// size keeps a valid one)
+// the text Gram's workspace
 static size_t crit_gram_floats(int B, int N_t_max, int D) {
-  size_t parts = 1;
-  if (N_t_max <= 128 && D % 8 == 0) {
-    const int n_k = (D + 63) / 64, ns = n_k < 16 ? n_k : 16, per = (n_k + ns - 1) / ns;
-    parts = (size_t)((n_k + per - 1) / per);
-  }
-  return parts * B * N_t_max * N_t_max;
+  return (size_t)crit_gram_parts(N_t_max, D) * B * N_t_max * N_t_max;
 }
 
 extern "C" size_t provip_crit_text_workspace_size(int B, int N_t_max, int D) {

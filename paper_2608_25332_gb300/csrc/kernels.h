@@ -181,9 +181,18 @@ struct SimArgs {
   int dtype;
   unsigned* err;
 };
-// Sec. 4.2: mask[b][j] (and r) from the text self-similarity. ws: G, [B][Ntm][Ntm]
-// f32; Ntm <= kCritMaxNt.
+// Sec. 4.2: mask[b][j] (and r) from the text self-similarity. ws: G, crit_gram_parts x
+// [B][Ntm][Ntm] f32; Ntm <= kCritMaxNt.
 constexpr int kCritMaxNt = 4096;
+// Parts of the text Gram that the workspace holds: up to 128 text rows one for every 64
+// elements of a row, at most 16, each of as many such slices; one beyond. Earlier kernels
+// filled them, and a workspace sized for them stays valid. The fp32 Gram leaves up to two,
+// within this number, the bf16 one at most one.
+inline int crit_gram_parts(int N_t_max, int D) {
+  if (N_t_max > 128 || D % 8 != 0) return 1;
+  const int n_k = (D + 63) / 64, ns = n_k < 16 ? n_k : 16, per = (n_k + ns - 1) / ns;
+  return (n_k + per - 1) / per;
+}
 // early (only where crit_leads holds): the next kernel of the stream, launched as a
 // programmatic dependent, may start at once
 bool crit_leads(const SimArgs& a, int num_sms);

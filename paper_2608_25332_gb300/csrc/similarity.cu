@@ -1116,10 +1116,11 @@ cudaError_t crit_text_launch(const SimArgs& a, uint8_t* mask, float* r_out, floa
     const int nt = (a.N_t_max + split::kTile - 1) / split::kTile;
     const int C = split::cluster_size((long long)a.B * nt * nt, a.D, num_sms);
     // where the largest clusters leave SMs idle, K in two parts, by the clusters' own rule
-    // (at least 1024 elements a part, so that G's region holds them): the relevance of one
+    // (at least 1024 elements a part) and where G's region holds them: the relevance of one
     // image waits for its 64 x 64 Gram over 4096 elements, and the pass went from 104.7 to
     // 98.5 us (four parts: the same, the relevance no longer waits)
-    while (C == split::kMaxCluster && a.N_t_max <= 32 * kPartsReg && parts < kCritMaxParts &&
+    while (C == split::kMaxCluster && a.N_t_max <= 32 * kPartsReg &&
+           2 * parts <= std::min(kCritMaxParts, crit_gram_parts(a.N_t_max, a.D)) &&
            2ll * parts * C * a.B * nt * nt <= (long long)split::kCtasPerSm * num_sms &&
            a.D / (2 * parts * C) >= 4 * split::kKT)
       parts *= 2;

@@ -162,3 +162,13 @@ def test_missing_library_fails_loudly(tmp_path, monkeypatch):
     monkeypatch.setattr(provip, "LIB_PATH", str(tmp_path / "libprovip.so"))
     with pytest.raises(provip.ProvipError, match="not built"):
         provip.lib()
+
+
+def test_text_gram_workspace_holds_its_parts(L):
+    """Up to 128 text rows the text Gram's workspace holds one part per 64 elements of a row,
+    16 at most (the sizes that callers may have kept), beyond one; the fp32 Gram fills two
+    parts from 2048 elements a row."""
+    for N_t, D, parts in [(64, 8, 1), (64, 128, 2), (128, 1024, 16), (128, 2048, 16), (7, 4096, 16), (40, 1088, 9),
+                          (129, 4096, 1), (300, 64, 1)]:
+        need = 3 * N_t * N_t * 4 * parts
+        assert L.provip_crit_text_workspace_size(3, N_t, D) == (need + 255) // 256 * 256, (N_t, D)

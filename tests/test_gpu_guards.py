@@ -190,6 +190,7 @@ def test_head_scores_writes_only_its_outputs(algo):
     ("bf16", 2, 200, 136, (129, 2), 50),
     ("bf16", 2, 150, 136, (40, 7), 60),
     ("f32", 2, 37, 64, (1, 9), 10),
+    ("f32", 1, 60, 2048, (128,), 20),  # the text Gram in two parts of K
 ])
 def test_similarity_reduce_writes_only_its_outputs(dtype, B, N_v, D, tls, keep_pre):
     rng = np.random.default_rng(77)
