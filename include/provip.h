@@ -162,7 +162,8 @@ int provip_topk(const float *scores, int B, int N, int k, int *idx_out, void *st
  * library reads it as: each pruned row j goes to the kept row of largest
  * cosine, ties to the lower kept position; merged = uniform mean of the kept
  * row and its members).
- *   keep_idx   [B, keep] int32, strictly ascending visual indices (device).
+ *   keep_idx   [B, keep] int32, strictly ascending visual indices (device; others are
+ *              reported, and every row still gets a position of the list).
  *   assign_out [B, N_v] int32: position in keep_idx of row j's centroid (kept
  *              rows map to their own position).
  *   merged_out [B, keep, D] dtype or NULL (assignment only). fp32 sums are

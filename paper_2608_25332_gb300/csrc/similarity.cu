@@ -527,10 +527,12 @@ __global__ void __launch_bounds__(split::kThreads, split::kCtasPerSm) relevance_
 // Sec. 4.3 merge
 // ---------------------------------------------------------------------------
 // Per sample (one CTA of 1024 threads): the kept-position map kpos[b][j] =
-// a if j == keep[b][a], else -1, and, when `pruned` is given, the rows not
-// kept in ascending order, pruned[b][0 .. N_v - keep) (ballot compaction).
+// a if j == keep[b][a], else -1, and the rows not kept in ascending order,
+// pruned[b][0 .. cap) (ballot compaction), -1 past the last one. cap is N_v - keep, which a
+// valid keep_idx fills, or N_v. With an invalid one (reported) more rows are not kept; those
+// past cap are marked -2 in the map.
 __global__ void __launch_bounds__(1024) merge_index_kernel(const int* keep_idx, int keep, int N_v, int* kpos,
-                                                           int* pruned, unsigned* err) {
+                                                           int* pruned, int cap, unsigned* err) {
   __shared__ int warp_tot[32];
   const int b = blockIdx.x;
   int* kp = kpos + (size_t)b * N_v;
@@ -545,10 +547,8 @@ __global__ void __launch_bounds__(1024) merge_index_kernel(const int* keep_idx, 
     }
     kp[j] = q;
   }
-  if (pruned == nullptr) return;
   __syncthreads();  // the map is complete (global writes of this block)
-  const int n_pruned = N_v - keep;
-  int* out = pruned + (size_t)b * n_pruned;
+  int* out = pruned + (size_t)b * cap;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   int base = 0;
   for (int j0 = 0; j0 < N_v; j0 += blockDim.x) {
@@ -563,10 +563,12 @@ __global__ void __launch_bounds__(1024) merge_index_kernel(const int* keep_idx, 
       tot += warp_tot[w];
     }
     const int pos = base + off + __popc(bal & ((1u << lane) - 1u));
-    if (pr && pos < n_pruned) out[pos] = j;
+    if (pr && pos < cap) out[pos] = j;
+    if (pr && pos >= cap) kp[j] = -2;
     base += tot;
     __syncthreads();
   }
+  for (int i = base + (int)threadIdx.x; i < cap; i += blockDim.x) out[i] = -1;
 }
 __device__ __forceinline__ bool better(float v, int i, float bv, int bi) {
   return v > bv || (v == bv && i < bi);
@@ -574,10 +576,11 @@ __device__ __forceinline__ bool better(float v, int i, float bv, int bi) {
 
 // Argmax over one split of the kept columns for 64 pruned rows: a cluster per
 // (row tile, split) walks the split's 64-column tiles (simt_split.cuh); CTA c of it
-// adds rows [c * 64 / C, ..) and keeps their running (max, lowest position).
+// adds rows [c * 64 / C, ..) and keeps their running (max, lowest position). The list of
+// a sample has room for n_list rows, -1 past the last one.
 template <typename T>
 __global__ void __launch_bounds__(split::kThreads, split::kCtasPerSm) merge_argmax_kernel(const SimArgs a, int C, const int* pruned,
-                                                                       int n_pruned, const int* keep_idx, int keep,
+                                                                       int n_list, const int* keep_idx, int keep,
                                                                        const float* inv_v, int n_split,
                                                                        float* ws_best, int* ws_bidx) {
   extern __shared__ __align__(128) uint8_t ring[];
@@ -590,7 +593,7 @@ __global__ void __launch_bounds__(split::kThreads, split::kCtasPerSm) merge_argm
   const int t0 = (int)((long long)ntile * part / n_split), t1 = (int)((long long)ntile * (part + 1) / n_split);
   const int tid = threadIdx.x, kg = tid & 15;
   if (tid < split::kTile) {
-    const int j = r0 + tid < n_pruned ? pruned[(size_t)b * n_pruned + r0 + tid] : -1;
+    const int j = r0 + tid < n_list ? pruned[(size_t)b * n_list + r0 + tid] : -1;
     const bool ok = j >= 0 && j < a.N_v;
     rowj[tid] = ok ? j : -1;
     arow[tid] = ok ? row_ptr<T>(a.emb_v, (size_t)b * a.N_v + j, a.D) : nullptr;
@@ -616,6 +619,7 @@ __global__ void __launch_bounds__(split::kThreads, split::kCtasPerSm) merge_argm
       kinv[tid] = ok ? inv_v[(size_t)b * a.N_v + j] : 0.f;
     }
     __syncthreads();
+    if (rowj[0] < 0) return;  // every CTA of the cluster: the list ends before the tile
     split::tile_part<T>(arow, brow, k0, k1, ring, a.emb_v);
     split::cluster_sync();
 #pragma unroll
@@ -666,8 +670,8 @@ __global__ void merge_assign_kernel(const SimArgs a, const int* kpos, int n_spli
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (size_t)a.B * a.N_v) return;
   const int kp = kpos[i];
-  if (kp >= 0) {
-    assign[i] = kp;
+  if (kp != -1) {
+    assign[i] = max(kp, 0);  // -2: a row that an invalid keep_idx left out of the pruned list
     return;
   }
   float bv = -INFINITY;
@@ -1297,30 +1301,33 @@ cudaError_t merge_launch(const SimArgs& a, const int* keep_idx, int keep, const 
   const bool tc = ws_perm != nullptr && merge_tc_supported(a, keep, tc_split);
   const int n_pruned = a.N_v - keep;
   int n_split = 1;
-  // the kept-position map and the pruned rows
-  if (!index_ready) merge_index_kernel<<<a.B, 1024, 0, s>>>(keep_idx, keep, a.N_v, kpos, ws_pruned, a.err);
+  // the kept-position map and the pruned rows: the FFMA Gram takes every row that is not
+  // kept (clusters past the last one leave at once), the tensor-core one as many as a valid
+  // keep_idx leaves
+  const int cap = tc || index_ready ? n_pruned : a.N_v;
+  if (!index_ready) merge_index_kernel<<<a.B, 1024, 0, s>>>(keep_idx, keep, a.N_v, kpos, ws_pruned, cap, a.err);
   if (tc) {
     cudaError_t e = merge_argmax_tc_launch(a, keep_idx, keep, inv_v, ws_pruned, ws_perm, tc_split, ws_best,
                                            ws_bidx, num_sms, &n_split, s);
     if (e != cudaSuccess) return e;
-  } else if (n_pruned > 0) {
+  } else if (cap > 0) {
     // column splits until three CTAs per SM are there, then the K split
-    const int rt = (n_pruned + split::kTile - 1) / split::kTile, ct = (keep + split::kTile - 1) / split::kTile;
+    const int rt = std::max(1, (n_pruned + split::kTile - 1) / split::kTile), ct = (keep + split::kTile - 1) / split::kTile;
     n_split = (int)std::min<long long>(std::min(ct, kMergeMaxSplit), 3ll * num_sms / ((long long)rt * a.B));
     if (n_split < 1) n_split = 1;
     const int C = split::cluster_size((long long)rt * a.B * n_split, a.D, num_sms);
-    const dim3 g((unsigned)(C * rt), (unsigned)a.B, (unsigned)n_split);
+    const dim3 g((unsigned)(C * ((cap + split::kTile - 1) / split::kTile)), (unsigned)a.B, (unsigned)n_split);
     static std::atomic<bool> set_f32[64], set_bf16[64];  // per device, zero-initialised
     const cudaError_t e =
-        a.dtype == 0 ? split::launch(merge_argmax_kernel<float>, split::kSmem<float>, set_f32, g, C, s, a, C, (const int*)ws_pruned, n_pruned,
+        a.dtype == 0 ? split::launch(merge_argmax_kernel<float>, split::kSmem<float>, set_f32, g, C, s, a, C, (const int*)ws_pruned, cap,
                                      keep_idx, keep, inv_v, n_split, ws_best, ws_bidx)
                      : split::launch(merge_argmax_kernel<__nv_bfloat16>, split::kSmem<__nv_bfloat16>, set_bf16, g, C, s, a, C, (const int*)ws_pruned,
-                                     n_pruned, keep_idx, keep, inv_v, n_split, ws_best, ws_bidx);
+                                     cap, keep_idx, keep, inv_v, n_split, ws_best, ws_bidx);
     if (e != cudaSuccess) return e;
   }
-  // the counter of the long centroids lies past the pruned list's last entry
-  // (keep >= 1 leaves room), which nothing else uses
-  int* n_long = merged != nullptr ? ws_pruned + (size_t)a.B * n_pruned : nullptr;
+  // the counter of the long centroids is the last entry of the pruned list's room: past the
+  // list (keep >= 1), or in it where that is full length, whose reader is done by then
+  int* n_long = merged != nullptr ? ws_pruned + nb - 1 : nullptr;
   cudaError_t el = launch_pdl(merge_assign_kernel, dim3((unsigned)((nb + 255) / 256)), dim3(256), 0, s, a,
                               (const int*)kpos, n_split, (const float*)ws_best, (const int*)ws_bidx, assign,
                               n_long);
