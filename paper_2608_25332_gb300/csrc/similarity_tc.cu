@@ -946,48 +946,65 @@ static int rel_tile_rows(int B, int N_v, int NT, int n_tb, int num_sms) {
   return best;
 }
 
+// tiles and shared memory of the relevance
+struct RelShape {
+  int NTs, n_tb, NT, R, n_vt, n_stages;
+  bool deep;    // one CTA per SM
+  size_t smem;
+};
+constexpr size_t kRelSmemMax = 200 * 1024;
+static RelShape rel_shape(int B, int N_v, int N_t_max, int num_sms) {
+  RelShape h;
+  h.NTs = rel_nt(N_t_max);
+  h.n_tb = (h.NTs + kBM - 1) / kBM;  // text blocks, of equal rows but for the last
+  h.NT = rel_nt((h.NTs + h.n_tb - 1) / h.n_tb);
+  h.R = rel_tile_rows(B, N_v, h.NT, h.n_tb, num_sms);
+  h.n_vt = (N_v + h.R - 1) / h.R;
+  // one CTA per SM when the tiles do not fill the GPU or there are several text
+  // blocks (deeper ring), else two
+  // the MMA reads 128 A rows (16 KiB) from the start of a stage: the last
+  // stage keeps that much room even when R + NT rows are fewer
+  const size_t st_bytes = (size_t)(h.R + h.NT) * 128;
+  const size_t tail = st_bytes > (size_t)kABytes ? 0 : (size_t)kABytes - st_bytes;
+  h.deep = h.n_tb > 1 || (long long)B * h.n_vt <= num_sms;
+  const size_t budget = (h.deep ? kRelSmemMax - 1024 : 110 * 1024 - 1024) - tail;
+  const int ns = (int)(budget / st_bytes);
+  h.n_stages = ns > kRelMaxStages ? kRelMaxStages : (ns < 2 ? 2 : ns);
+  h.smem = (size_t)h.n_stages * st_bytes + tail + 1024;
+  return h;
+}
+
 cudaError_t relevance_tc_launch(const SimArgs& a, const uint8_t* mask, const float* inv_t, float* inv_v,
                                 float* p, float* ws, int num_sms, cudaStream_t s, cudaEvent_t mask_ready) {
   static std::atomic<bool> smem_set[64], smem_set2[64];  // per device, zero-initialised
   int dev = 0;
   cudaGetDevice(&dev);
-  constexpr size_t kSmemMax = 200 * 1024;
-  cudaError_t e = set_smem(relevance_fused_tc<1>, kSmemMax, &smem_set[dev < 64 ? dev : 0]);
-  if (e == cudaSuccess) e = set_smem(relevance_fused_tc<2>, kSmemMax, &smem_set2[dev < 64 ? dev : 0]);
+  cudaError_t e = set_smem(relevance_fused_tc<1>, kRelSmemMax, &smem_set[dev < 64 ? dev : 0]);
+  if (e == cudaSuccess) e = set_smem(relevance_fused_tc<2>, kRelSmemMax, &smem_set2[dev < 64 ? dev : 0]);
   if (e != cudaSuccess) return e;
   RelFusedArgs r;
   r.B = a.B;
   r.N_v = a.N_v;
   r.D = a.D;
   r.N_t_max = a.N_t_max;
-  r.NTs = rel_nt(a.N_t_max);
-  const int n_tb = (r.NTs + kBM - 1) / kBM;  // text blocks, of equal rows but for the last
-  r.NT = rel_nt((r.NTs + n_tb - 1) / n_tb);
-  r.R = rel_tile_rows(a.B, a.N_v, r.NT, n_tb, num_sms);
-  r.n_vt = (a.N_v + r.R - 1) / r.R;
+  const RelShape h = rel_shape(a.B, a.N_v, a.N_t_max, num_sms);
+  r.NTs = h.NTs;
+  r.NT = h.NT;
+  r.R = h.R;
+  r.n_vt = h.n_vt;
+  r.n_stages = h.n_stages;
   r.inv_t = inv_t;
   r.inv_v = inv_v;
   r.Y = ws;
   r.part = ws + (size_t)a.B * a.N_v * r.NTs;
   r.err = a.err;
-  // one CTA per SM when the tiles do not fill the GPU or there are several text
-  // blocks (deeper ring), else two
-  // the MMA reads 128 A rows (16 KiB) from the start of a stage: the last
-  // stage keeps that much room even when R + NT rows are fewer
-  const size_t st_bytes = (size_t)(r.R + r.NT) * 128;
-  const size_t tail = st_bytes > (size_t)kABytes ? 0 : (size_t)kABytes - st_bytes;
-  const bool deep = n_tb > 1 || (long long)a.B * r.n_vt <= num_sms;
-  const size_t budget = (deep ? kSmemMax - 1024 : 110 * 1024 - 1024) - tail;
-  int ns = (int)(budget / st_bytes);
-  r.n_stages = ns > kRelMaxStages ? kRelMaxStages : (ns < 2 ? 2 : ns);
-  const size_t smem = (size_t)r.n_stages * st_bytes + tail + 1024;
   CUtensorMap mapV, mapT;
   if (make_tmap_bf16_2d(&mapV, a.emb_v, (uint64_t)a.B * a.N_v, (uint64_t)a.D, (uint64_t)a.D * 2, (uint32_t)r.R) ||
       make_tmap_bf16_2d(&mapT, a.emb_t, (uint64_t)a.B * a.N_t_max, (uint64_t)a.D, (uint64_t)a.D * 2,
                         (uint32_t)r.NT))
     return cudaErrorInvalidValue;
-  e = n_tb == 1 ? launch_pdl(relevance_fused_tc<1>, dim3(r.n_vt, a.B), dim3(kThreads), smem, s, r, mapV, mapT)
-                : launch_pdl(relevance_fused_tc<2>, dim3(r.n_vt, a.B, n_tb), dim3(kThreads), smem, s, r, mapV, mapT);
+  e = h.n_tb == 1 ? launch_pdl(relevance_fused_tc<1>, dim3(r.n_vt, a.B), dim3(kThreads), h.smem, s, r, mapV, mapT)
+                  : launch_pdl(relevance_fused_tc<2>, dim3(r.n_vt, a.B, h.n_tb), dim3(kThreads), h.smem, s, r, mapV, mapT);
   if (e != cudaSuccess) return e;
   const dim3 gf((a.N_v + 8 * kRelFinishRows - 1) / (8 * kRelFinishRows), a.B);
   const size_t smem_f = (size_t)r.NTs * (sizeof(float) + sizeof(int));
@@ -1011,14 +1028,35 @@ static int crit_cluster(int B, int nt, int n_k, int num_sms) {
   return C;
 }
 
-// The critical rows are one kernel whose CTAs take three quarters of the SMs or more:
-// the relevance then follows it on its stream instead of running beside it from
-// another, without the events between (passes of 32 and of 16 images 171 -> 167 and
-// 222 -> 218 us, 128 CTAs each; with 64 and with 8 CTAs, 8 anyres samples and a video,
-// the later start of the relevance costs more: 219 -> 223 and 178 -> 184).
+constexpr size_t kCritTileBytes = (size_t)kBM * kCritLd * sizeof(float);
+constexpr size_t kCritRingBytes = (size_t)kCritStages * kABytes;
+constexpr size_t kCritWholeSmem = (kCritRingBytes > kCritTileBytes ? kCritRingBytes : kCritTileBytes) + 1024;
+
+// Whether the critical rows, as one kernel, come first on the stream and the relevance
+// follows instead of running beside them from another, without the events between.
+// * Their CTAs take three quarters of the SMs or more: at 64 and 8 CTAs (8 anyres samples,
+//   a video) the later start of the relevance costs more, 219 -> 223 us a pass and 178 ->
+//   184, and at 80 to 112 it went either way.
+// * The relevance takes at most two CTAs per SM at once: at 29 samples of 1440 rows (435
+//   tiles) 292 -> 297 us and 277 -> 282, at 32 under 128 text rows 311 -> 320.
+// * Where it takes one CTA per SM, on more than seven eighths of them, that CTA does not
+//   fit beside one of the critical rows: where it does, it is put there and both run slower
+//   than in turn. 15 and 16 samples of 576 rows under 32 and 64 text rows (135 and 144
+//   tiles of 64 rows, rings of 98 and 128 KiB): 107 -> 115 us from a graph, 119 -> 119
+//   launched one by one; 15 of width 2048 66 -> 72 and 72 -> 77, 29 of 300 rows (145) 120
+//   -> 126 and 133 -> 133. On fewer SMs (102 to 128 tiles) it gains all the same: 19 samples
+//   of 576 rows under 32 (114) 110..118 -> 106 and 123 -> 111.
+// Elsewhere, over 15 to 38 samples of 300 to 1440 rows of widths 1024 to 5120, it gave 1 to
+// 6%: 16 samples of 576 under 128 text rows 121 -> 119, 17 under 64 118 -> 112, 32 of width
+// 5120 171 -> 167.
 bool crit_leads(const SimArgs& a, int num_sms) {
   if (a.dtype != 1 || a.N_t_max > kBM || !relevance_tc_supported(a)) return false;
-  return 4ll * a.B * crit_cluster(a.B, 1, (a.D + kBK - 1) / kBK, num_sms) >= 3ll * num_sms;
+  if (4ll * a.B * crit_cluster(a.B, 1, (a.D + kBK - 1) / kBK, num_sms) < 3ll * num_sms) return false;
+  const RelShape h = rel_shape(a.B, a.N_v, a.N_t_max, num_sms);
+  const long long tiles = (long long)a.B * h.n_vt;
+  if (!h.deep) return tiles <= 2ll * num_sms;
+  // 228 KiB per SM; 8 KiB for both kernels' static parts and what a CTA reserves
+  return 8 * tiles <= 7ll * num_sms || h.smem + kCritWholeSmem + 8 * 1024 > 228 * 1024;
 }
 
 cudaError_t crit_gram_tc_launch(const SimArgs& a, uint8_t* mask, float* r_out, float* G, int num_sms, bool* whole,
@@ -1026,11 +1064,8 @@ cudaError_t crit_gram_tc_launch(const SimArgs& a, uint8_t* mask, float* r_out, f
   static std::atomic<bool> smem_set[64], smem_set2[64];  // per device, zero-initialised
   int dev = 0;
   cudaGetDevice(&dev);
-  constexpr size_t kTileBytes = (size_t)kBM * kCritLd * sizeof(float);
-  constexpr size_t kWholeBytes = (size_t)kCritStages * kABytes;
-  constexpr size_t smem1 = (kWholeBytes > kTileBytes ? kWholeBytes : kTileBytes) + 1024;
-  constexpr size_t smem2 = (size_t)kCritStages * 2 * kABytes + 1024;
-  static_assert(smem2 >= kTileBytes + 1024, "the tile part fits the stages");
+  constexpr size_t smem1 = kCritWholeSmem, smem2 = (size_t)kCritStages * 2 * kABytes + 1024;
+  static_assert(smem2 >= kCritTileBytes + 1024, "the tile part fits the stages");
   cudaError_t e = set_smem(crit_gram_tc<true>, smem1, &smem_set[dev < 64 ? dev : 0]);
   if (e == cudaSuccess) e = set_smem(crit_gram_tc<false>, smem2, &smem_set2[dev < 64 ? dev : 0]);
   if (e != cudaSuccess) return e;

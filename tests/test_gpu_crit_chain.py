@@ -1,6 +1,6 @@
-"""Pre-LLM pass with the critical rows first on the stream (their CTAs take three
-quarters of the SMs or more) and from the side stream: the mask and p of back-to-back
-passes on one workspace must be the bits of the separate calls."""
+"""Pre-LLM pass with the critical rows first on the stream and from the side stream: the
+mask and p of back-to-back passes on one workspace must be the bits of the separate
+calls."""
 import pytest
 import torch
 
@@ -12,11 +12,14 @@ DEV = "cuda:0"
 
 @pytest.mark.parametrize("B,N_v,N_t,D,keep", [
     (13, 100, 40, 512, 30),    # 104 CTAs: the side stream
-    (15, 100, 40, 512, 30),    # 120 CTAs of clusters of 8
+    (15, 100, 40, 512, 30),    # 120 CTAs of clusters of 8: first on the stream
+    (15, 560, 40, 512, 30),    # the same, but a relevance CTA fits beside each on nearly every SM: the side stream
+    (15, 560, 128, 512, 30),   # one that does not fit: first
     (20, 300, 128, 256, 100),  # clusters of 4 (as many K slices): 80 CTAs, the side stream
-    (29, 257, 128, 264, 64),   # clusters of 4: 116 CTAs; a ragged last K slice and visual tile
-    (120, 40, 7, 64, 9),       # one K slice, one CTA a sample
-    (64, 70, 128, 256, 20),    # clusters of 4, 512 columns of tensor memory each: 256 CTAs, more than SMs
+    (29, 257, 128, 264, 64),   # clusters of 4: 116 CTAs, first; a ragged last K slice and visual tile
+    (120, 40, 7, 64, 9),       # one K slice, one CTA a sample: first
+    (140, 40, 7, 64, 9),       # the same on nearly every SM: the side stream
+    (64, 70, 128, 256, 20),    # clusters of 4, 512 columns of tensor memory each: 256 CTAs, more than SMs; first
 ])
 def test_pass_gives_the_bits_of_separate_calls(B, N_v, N_t, D, keep):
     __graft_entry__.build()
