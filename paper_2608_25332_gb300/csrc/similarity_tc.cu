@@ -316,17 +316,23 @@ __global__ void __launch_bounds__(kMergeThreads, 1)
 //     butterfly, then the four lane quadrants in order).
 // relevance_finish_kernel then forms mu_i = (sum of the tile sums in tile
 // order) / N_v and p_j = max_{i in T} (Y[b][j][i] - mu_i) (Sec. 4.3).
-// More than 128 text rows are split into blocks of at most 128 (grid z); each
+// More than 128 text rows (kLong) are split into blocks of at most 128 (grid z); each
 // block's CTAs read the visual tiles again (from L2, where the first block's
-// loads left them) and form their norms themselves. These CTAs are bound by the
-// latency of their K loop and are few, so they run one per SM with two
-// accumulators (kAcc = 2), each over half of the K slices: the tensor core
-// truncates at every accumulation, and the shorter chains keep p as close to its
-// value as the FFMA kernel that took such texts before (relative error of p
-// against 64 bits over widths 2048 to 5120: 2-7e-7, FFMA 6-12e-7). That kernel
-// took 990 us on 4 x 1443 visual rows under 300 text rows (23 x 4 CTAs, each a
-// chain of 128 K steps of 2.4 us per 128 text rows); the whole pre-LLM pass of
-// that batch went from 1322 to 605 us.
+// loads left them), one CTA per SM with a deep ring. FFMA kernels took such texts
+// before, 990 us for 4 x 1443 visual rows under 300 text rows, and their sums were rounded
+// to nearest where the tensor core truncates at every accumulation: two accumulators
+// over half of the K slices each left p further off than FFMA from width 3584 on
+// (relative error against 64 bits on random rows 8.7e-7 at 4096 and 1.7e-6 at 8192, FFMA
+// 6.0e-7 and 1.0e-6), and 1/|v_j|, which the merge reads on its own, 2.6e-6 and 5.2e-6 (FFMA
+// 0.9e-7 and 1.3e-7). So here
+//   * an accumulator takes kRelChunk slices, two in turn, and the epilogue warps add them up
+//     in registers: p is 1.1e-7 off at widths 512 to 5120 and 2.5e-7 at 8192;
+//   * in the first block, warps of their own add up the squares of the visual rows from the
+//     slices as they pass: 1/|v_j| is 0.4e-7 off at every width.
+// Both cost the K loop some 3%: the pass of the batch above 129.5 -> 131 us, 8 x 2880 rows
+// 335 -> 344, 32 x 576 rows of width 5120 under 512 526 -> 538. Chunks of two and of eight
+// slices: 360 and 342 us for the 8 x 2880; the squares in the epilogue warps, or by all
+// blocks in place of the visual block of the MMA: 349 and 355.
 struct RelFusedArgs {
   int B, N_v, D, N_t_max;
   int NT;        // text rows in the MMA (a block's rows, a multiple of 16)
@@ -345,16 +351,21 @@ constexpr int kRelMaxStages = 8;
 constexpr int kRelFinishRows = 8;  // rows per warp of relevance_finish_kernel
 constexpr uint32_t kRelTmemCols = 256;  // 128 visual + <= 128 text columns
 
+constexpr int kRelChunk = 4;            // K slices of an accumulator with several text blocks
+constexpr int kRelSqWarps = 2;          // then more warps, for the squares of kBM rows
+constexpr int kRelLongThreads = kThreads + 32 * kRelSqWarps;
+
 struct RelPipe {
   uint64_t full[kRelMaxStages];
   uint64_t empty[kRelMaxStages];
-  uint64_t acc_full;
+  uint64_t acc_full[2];   // one accumulator, or two in turn with several text blocks
+  uint64_t acc_empty[2];
   uint32_t tmem;
   volatile int fail;
 };
 
-template <int kAcc>
-__global__ void __launch_bounds__(kThreads, 2 / kAcc)
+template <bool kLong>
+__global__ void __launch_bounds__(kLong ? kRelLongThreads : kThreads, kLong ? 1 : 2)
     relevance_fused_tc(const RelFusedArgs a, const __grid_constant__ CUtensorMap mapV,
                        const __grid_constant__ CUtensorMap mapT) {
   extern __shared__ uint8_t smem_raw[];
@@ -368,6 +379,8 @@ __global__ void __launch_bounds__(kThreads, 2 / kAcc)
   const int n_k = (a.D + kBK - 1) / kBK;
   const int NS = a.n_stages;
   const uint32_t st_bytes = (uint32_t)(R + a.NT) * 128u;
+  constexpr uint32_t kCols = (kLong ? 2 : 1) * kRelTmemCols;
+  const bool squares = kLong && blockIdx.z == 0;
   const uint32_t sbase = smem_u32(smem_raw);
   uint8_t* stages = smem_raw + (((sbase + 1023u) & ~1023u) - sbase);
   if (threadIdx.x == 0) {
@@ -375,14 +388,17 @@ __global__ void __launch_bounds__(kThreads, 2 / kAcc)
     prefetch_tmap(&mapT);
     for (int s = 0; s < NS; ++s) {
       mbar_init(&pipe.full[s], 1);
-      mbar_init(&pipe.empty[s], 1);
+      mbar_init(&pipe.empty[s], squares ? 1 + kRelSqWarps : 1);  // the MMAs, and the warps that add squares
     }
-    mbar_init(&pipe.acc_full, 1);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&pipe.acc_full[s], 1);
+      mbar_init(&pipe.acc_empty[s], 4);  // the epilogue warps
+    }
     pipe.fail = 0;
     fence_mbar_init();
   }
   if (threadIdx.x < 32) {
-    tmem_alloc(&pipe.tmem, kAcc * kRelTmemCols);
+    tmem_alloc(&pipe.tmem, kCols);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -409,66 +425,165 @@ __global__ void __launch_bounds__(kThreads, 2 / kAcc)
   } else if (warp == 1) {
     if (lane == 0) {
       const uint32_t idesc = idesc_bf16_f32(kBM, R + a.NT);
-      const int kb1 = kAcc == 1 ? n_k : (n_k + 1) / 2;  // first slice of the second accumulator
+      // One lane issues every MMA, and at some 800 clocks a slice it, not the loads, set the
+      // pace: so it adds byte offsets, in 16-byte units, to the first stage's descriptor,
+      // counts stages instead of dividing, and looks at the next slice's barriers before it
+      // issues this one's MMAs.
+      const uint64_t desc0 = smem_desc_sw128(smem_u32(stages));
+      uint64_t desc = desc0;
+      int s = 0, in_ch = 0;                // the slice's stage; its place in its accumulator
+      uint32_t ph = 0, buf = 0, ph_a = 1;  // parities of full and, with several blocks, of acc_empty
+      bool there = false, room = false;    // the next slice's loads and accumulator, looked at ahead
       for (int kb = 0; kb < n_k; ++kb) {
-        const int s = kb % NS;
-        const uint32_t ph = (uint32_t)(kb / NS) & 1u;
-        if (pipe.fail || !mbar_wait(&pipe.full[s], ph, a.err)) {
+        if (kLong && in_ch == 0 && !room && !pipe.fail && !mbar_wait(&pipe.acc_empty[buf], ph_a, a.err)) pipe.fail = 1;
+        if (pipe.fail || (!there && !mbar_wait(&pipe.full[s], ph, a.err))) {
           pipe.fail = 1;
           break;
         }
+        const bool wrap = s + 1 == NS, last = kb == n_k - 1, ends = kLong && (in_ch + 1 == kRelChunk || last);
+        const int s1 = wrap ? 0 : s + 1;
+        const uint32_t ph1 = wrap ? ph ^ 1u : ph;
+        there = !last && mbar_test(&pipe.full[s1], ph1);
+        if (ends) room = !last && mbar_test(&pipe.acc_empty[buf ^ 1u], ph_a ^ buf);
         tc_fence_after();
-        const uint32_t sa = smem_u32(stages + (size_t)s * st_bytes);
+        const uint32_t acc = pipe.tmem + buf * kRelTmemCols;
 #pragma unroll
         for (int k = 0; k < kBK / 16; ++k)
-          tc_mma_bf16(pipe.tmem + (kb >= kb1 ? kRelTmemCols : 0u), smem_desc_sw128(sa + k * 32),
-                      smem_desc_sw128(sa + k * 32), idesc, ((kb != 0 && kb != kb1) || k > 0) ? 1u : 0u);
+          tc_mma_bf16(acc, desc + 2 * k, desc + 2 * k, idesc, ((kLong ? in_ch : kb) > 0 || k > 0) ? 1u : 0u);
         tc_commit(&pipe.empty[s]);
+        desc = wrap ? desc0 : desc + (st_bytes >> 4);
+        s = s1;
+        ph = ph1;
+        ++in_ch;
+        if (ends) {
+          tc_commit(&pipe.acc_full[buf]);  // arrives once every MMA above has completed
+          in_ch = 0;
+          ph_a ^= buf;  // the second accumulator's turn ends a round
+          buf ^= 1u;
+        }
       }
-      tc_commit(&pipe.acc_full);  // arrives once every MMA above has completed
+      if (!kLong) tc_commit(&pipe.acc_full[0]);
+    }
+  } else if (kLong && warp >= kThreads / 32) {
+    if (squares) {
+      // 1/|v_j| of the tile's rows for the merge: the squares of row r's slices as they
+      // pass, a slice's 64 in eight chains, the slices by TwoSum (in one chain over the
+      // slices the sum is biased low: squares of bf16 values are 0 or 1 mod 4 in their last
+      // place, so that rounding them to a longer one's goes down more often). A row's eight
+      // 16-byte pieces lie in some order in its 128 bytes, and lane l starts with piece l of
+      // them, so that eight lanes meet every bank.
+      constexpr int kRows = kBM / (32 * kRelSqWarps);  // rows of a lane
+      const int r0 = (warp - kThreads / 32) * 32 + lane;
+      float sum[kRows], rest[kRows];
+#pragma unroll
+      for (int h = 0; h < kRows; ++h) sum[h] = rest[h] = 0.f;
+      int s = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int kb = 0; kb < n_k && ok; ++kb) {
+        ok = warp_mbar_wait(&pipe.full[s], ph, a.err);
+#pragma unroll
+        for (int h = 0; h < kRows; ++h) {
+          const int r = r0 + h * 32 * kRelSqWarps;
+          if (!ok || r >= R) break;  // warp-uniform
+          const uint8_t* row = stages + (size_t)s * st_bytes + (size_t)r * 128;
+          float sq[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const uint4 u = *reinterpret_cast<const uint4*>(row + ((i + lane) & 7) * 16);
+            const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const float lo = __uint_as_float(w[e] << 16), hi = __uint_as_float(w[e] & 0xffff0000u);
+              sq[2 * e] = fmaf(lo, lo, sq[2 * e]);
+              sq[2 * e + 1] = fmaf(hi, hi, sq[2 * e + 1]);
+            }
+          }
+          const float q = ((sq[0] + sq[1]) + (sq[2] + sq[3])) + ((sq[4] + sq[5]) + (sq[6] + sq[7]));
+          const float t = sum[h] + q, z = t - sum[h];
+          rest[h] += (sum[h] - (t - z)) + (q - z);
+          sum[h] = t;
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&pipe.empty[s]);
+        if (++s == NS) {
+          s = 0;
+          ph ^= 1u;
+        }
+      }
+      if (!ok) pipe.fail = 1;
+      pdl_wait_prior();
+#pragma unroll
+      for (int h = 0; h < kRows; ++h) {
+        const int r = r0 + h * 32 * kRelSqWarps, j = n0 + r;
+        const float v = sum[h] + rest[h];
+        if (ok && r < R && j < a.N_v) a.inv_v[(size_t)b * a.N_v + j] = v > 0.f ? 1.f / sqrtf(v) : 0.f;
+      }
     }
   } else {
     const int quad = warp & 3;
     const int r = quad * 32 + lane;
     const int j = n0 + r;
     const bool rv = r < R && j < a.N_v;
+    const uint32_t taddr = pipe.tmem + ((uint32_t)(quad * 32) << 16);
+    const int nt = min(a.NT, a.NTs - tb0);  // the last block may be narrower
+    float v[32];
+    // |v_j|^2: column j of the visual block, i.e. element `lane` of the warp's 32 columns
+    auto diagonal = [&]() {
+      float d = 0.f;
+#pragma unroll
+      for (int i = 0; i < 32; ++i) d = i == lane ? v[i] : d;
+      return d;
+    };
+    bool ok = true;
+    float sqv = 0.f;
+    float sum[kLong ? kBM : 1];  // several text blocks: the products, chunk by chunk
+    if constexpr (kLong) {
+#pragma unroll
+      for (int i = 0; i < kBM; ++i) sum[i] = 0.f;
+      const int n_ch = (n_k + kRelChunk - 1) / kRelChunk;
+      for (int ch = 0; ch < n_ch && ok; ++ch) {
+        ok = warp_mbar_wait(&pipe.acc_full[ch & 1], (uint32_t)(ch >> 1) & 1u, a.err);
+        if (!ok) pipe.fail = 1;
+        tc_fence_after();
+        const uint32_t tch = taddr + ((ch & 1) ? kRelTmemCols : 0u);
+        tmem_ld32(tch + (uint32_t)(quad * 32), v);
+        tc_wait_ld_into(v);
+        sqv += diagonal();
+#pragma unroll
+        for (int cb = 0; cb < kBM / 32; ++cb)
+          if (cb * 32 < nt) {
+            tmem_ld32(tch + (uint32_t)(R + cb * 32), v);
+            tc_wait_ld_into(v);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) sum[cb * 32 + i] += v[i];
+          }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&pipe.acc_empty[ch & 1]);
+      }
+    }
     // launched as a programmatic dependent of the text-row norms: the loads and
     // MMAs ran under that kernel; its output (and every write below) waits here
     pdl_wait_prior();
     s_invt[r] = tb0 + r < a.N_t_max ? a.inv_t[(size_t)b * a.N_t_max + tb0 + r] : 0.f;
     asm volatile("bar.sync 1, 128;" ::: "memory");  // s_invt complete (epilogue warps)
-    const bool ok = warp_mbar_wait(&pipe.acc_full, 0, a.err) && !pipe.fail;
+    if constexpr (!kLong) {
+      ok = warp_mbar_wait(&pipe.acc_full[0], 0, a.err);
+      tc_fence_after();
+    }
+    ok = ok && !pipe.fail;
     pdl_allow_next();  // the finish kernel, where it follows without an event between
-    tc_fence_after();
-    const uint32_t taddr = pipe.tmem + ((uint32_t)(quad * 32) << 16);
-    float v[32];
-    // 32 columns from column c of the accumulator (of both: one K slice has no second)
-    const bool two = kAcc == 2 && n_k > 1;
-    auto load_cols = [&](int c) {
-      tmem_ld32(taddr + (uint32_t)c, v);
-      if (two) {
-        float w[32];
-        tmem_ld32(taddr + kRelTmemCols + (uint32_t)c, w);
-        tc_wait_ld_into(w);
-        tc_wait_ld_into(v);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] += w[i];
-      } else {
-        tc_wait_ld();
-      }
-    };
-    // |v_j|^2: column j of the visual block, i.e. element `lane` of the warp's 32 columns
-    load_cols(quad * 32);
-    float sqv = 0.f;
-#pragma unroll
-    for (int i = 0; i < 32; ++i) sqv = i == lane ? v[i] : sqv;
+    if constexpr (!kLong) {
+      tmem_ld32(taddr + (uint32_t)(quad * 32), v);
+      tc_wait_ld();
+      sqv = diagonal();
+    }
     const float iv = sqv > 0.f ? 1.f / sqrtf(sqv) : 0.f;
-    if (rv && ok && blockIdx.z == 0) a.inv_v[(size_t)b * a.N_v + j] = iv;
-    const int nt = min(a.NT, a.NTs - tb0);  // the last block may be narrower
+    if (!kLong && rv && ok) a.inv_v[(size_t)b * a.N_v + j] = iv;
     float* yrow = a.Y + ((size_t)b * a.N_v + (rv ? j : 0)) * a.NTs + tb0;
-#pragma unroll 1
-    for (int cb = 0; cb * 32 < nt; ++cb) {
-      load_cols(R + cb * 32);
+    // the cosines of text columns [32 cb, ..), from the products in v, and their sums
+    auto columns = [&](int cb) {
 #pragma unroll
       for (int i = 0; i < 32; ++i) v[i] = v[i] * s_invt[cb * 32 + i] * iv;
       if (rv && ok) {
@@ -492,6 +607,22 @@ __global__ void __launch_bounds__(kThreads, 2 / kAcc)
         }
       }
       red[quad][cb * 32 + lane] = v[0];
+    };
+    if constexpr (kLong) {
+#pragma unroll
+      for (int cb = 0; cb < kBM / 32; ++cb)
+        if (cb * 32 < nt) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) v[i] = sum[cb * 32 + i];
+          columns(cb);
+        }
+    } else {
+#pragma unroll 1
+      for (int cb = 0; cb * 32 < nt; ++cb) {
+        tmem_ld32(taddr + (uint32_t)(R + cb * 32), v);
+        tc_wait_ld();
+        columns(cb);
+      }
     }
     tc_fence_before();
     asm volatile("bar.sync 1, 128;" ::: "memory");
@@ -501,7 +632,7 @@ __global__ void __launch_bounds__(kThreads, 2 / kAcc)
   }
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x < 32) tmem_dealloc(pipe.tmem, kAcc * kRelTmemCols);
+  if (threadIdx.x < 32) tmem_dealloc(pipe.tmem, kCols);
 }
 
 // mu_i from the tile sums (tile order; every CTA forms all of mu), then p_j =
@@ -979,8 +1110,8 @@ cudaError_t relevance_tc_launch(const SimArgs& a, const uint8_t* mask, const flo
   static std::atomic<bool> smem_set[64], smem_set2[64];  // per device, zero-initialised
   int dev = 0;
   cudaGetDevice(&dev);
-  cudaError_t e = set_smem(relevance_fused_tc<1>, kRelSmemMax, &smem_set[dev < 64 ? dev : 0]);
-  if (e == cudaSuccess) e = set_smem(relevance_fused_tc<2>, kRelSmemMax, &smem_set2[dev < 64 ? dev : 0]);
+  cudaError_t e = set_smem(relevance_fused_tc<false>, kRelSmemMax, &smem_set[dev < 64 ? dev : 0]);
+  if (e == cudaSuccess) e = set_smem(relevance_fused_tc<true>, kRelSmemMax, &smem_set2[dev < 64 ? dev : 0]);
   if (e != cudaSuccess) return e;
   RelFusedArgs r;
   r.B = a.B;
@@ -1003,8 +1134,8 @@ cudaError_t relevance_tc_launch(const SimArgs& a, const uint8_t* mask, const flo
       make_tmap_bf16_2d(&mapT, a.emb_t, (uint64_t)a.B * a.N_t_max, (uint64_t)a.D, (uint64_t)a.D * 2,
                         (uint32_t)r.NT))
     return cudaErrorInvalidValue;
-  e = h.n_tb == 1 ? launch_pdl(relevance_fused_tc<1>, dim3(r.n_vt, a.B), dim3(kThreads), h.smem, s, r, mapV, mapT)
-                  : launch_pdl(relevance_fused_tc<2>, dim3(r.n_vt, a.B, h.n_tb), dim3(kThreads), h.smem, s, r, mapV, mapT);
+  e = h.n_tb == 1 ? launch_pdl(relevance_fused_tc<false>, dim3(r.n_vt, a.B), dim3(kThreads), h.smem, s, r, mapV, mapT)
+                  : launch_pdl(relevance_fused_tc<true>, dim3(r.n_vt, a.B, h.n_tb), dim3(kRelLongThreads), h.smem, s, r, mapV, mapT);
   if (e != cudaSuccess) return e;
   const dim3 gf((a.N_v + 8 * kRelFinishRows - 1) / (8 * kRelFinishRows), a.B);
   const size_t smem_f = (size_t)r.NTs * (sizeof(float) + sizeof(int));

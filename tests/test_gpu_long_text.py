@@ -56,6 +56,51 @@ def test_relevance_of_long_text(N_v, D, tls):
         assert_close_rel(got, ref, 0.0, f"p N_v={N_v} D={D} tls={tls} [{b}]", atol=1e-5)
 
 
+@pytest.mark.parametrize("N_v,D,T", [(500, 512, 129), (300, 4096, 300), (300, 5120, 129), (300, 8192, 513)])
+def test_relevance_of_long_text_is_an_fp32_sums(N_v, D, T):
+    """p of random rows against 64 bits: an accumulator is truncated at 16 products of 16
+    elements at most before it is added in fp32, a loss of about half a unit of 2^-23 of a
+    partial sum each, so some five units of 2^-24 of the sums; eight in the 2-norm of p (FFMA
+    sums rounded to nearest over the whole width: 10 at 4096, 17 at 8192)."""
+    g = torch.Generator().manual_seed(D + T)
+    B = 2
+    ev = torch.randn(B, N_v, D, generator=g).to(torch.bfloat16).to(DEV)
+    et = (0.02 * torch.randn(B, T, D, generator=g)).to(torch.bfloat16).to(DEV)
+    mask = (torch.rand(B, T, generator=g) < 0.4).to(torch.uint8).to(DEV)
+    p = P.provip_relevance(ev, et, torch.full((B,), T, dtype=torch.int32, device=DEV), mask).double()
+    V, W = ev.double(), et.double()
+    cos = (W / W.norm(dim=2, keepdim=True)) @ (V / V.norm(dim=2, keepdim=True)).transpose(1, 2)
+    ref = (cos - cos.mean(dim=2, keepdim=True)).masked_fill(mask[:, :, None] == 0, -float("inf")).amax(dim=1)
+    assert (p - ref).norm() <= 8 * 2.0 ** -24 * ref.norm()
+
+
+@pytest.mark.parametrize("N_v,D,T", [(700, 512, 129), (130, 4096, 300), (700, 5120, 300), (97, 8192, 1000), (60, 72, 256)])
+def test_norms_of_the_visual_rows_with_long_text(N_v, D, T):
+    """1/|v_j|, which the merge reads after the relevance (the first part of its workspace),
+    comes from an fp32 sum: slices of 64 products, each to a few roundings that vary from
+    slice to slice, added without loss, then a root and a quotient, rounded once each. Two
+    units of 2^-24 in the root mean square."""
+    g = torch.Generator().manual_seed(D + N_v)
+    B = 2
+    ev = torch.randn(B, N_v, D, generator=g).to(torch.bfloat16).to(DEV)
+    ev[1, 5] = 0
+    et = torch.randn(B, T, D, generator=g).to(torch.bfloat16).to(DEV)
+    tl = torch.tensor([T, 3], dtype=torch.int32, device=DEV)
+    mask = torch.ones(B, T, dtype=torch.uint8, device=DEV)
+    L = P.lib()
+    ws = P.workspace(L.provip_relevance_workspace_size(B, N_v, D, T), torch.device(DEV))
+    p = torch.empty(B, N_v, dtype=torch.float32, device=DEV)
+    rc = L.provip_relevance(P._ptr(ev), B, N_v, D, P._ptr(et), P._i32(tl), T, P._u8(mask), P.BF16, P._ptr(p), P._ptr(ws),
+                            ws.numel(), P._stream(ev.device))
+    assert rc == 0
+    torch.cuda.synchronize()
+    inv = ws[:4 * B * N_v].view(torch.float32).view(B, N_v).double()
+    assert inv[1, 5] == 0
+    norm = ev.double().norm(dim=2)
+    rel = (inv * norm - 1)[norm > 0]
+    assert rel.square().mean().sqrt() <= 2 * 2.0 ** -24
+
+
 @pytest.mark.parametrize("dtype,D,tls", [
     ("bf16", 64, (1, 5, 128)),               # one K slice: a cluster of one CTA
     ("bf16", 264, (17, 0, 33)),              # five slices over four CTAs
