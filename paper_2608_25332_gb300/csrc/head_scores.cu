@@ -11,9 +11,9 @@
 //   (max, sum) combined from all chunk stats, sum over the block's rows ->
 //   partial[b][rb * H_sel + head][col]. Deterministic: fixed reduction orders,
 //   no atomics.
-// Both walk a block's 128 rows as two 64 x 64 tiles of products (simt_split.cuh, all
-// of K = 128 in flight at once), the second only where the sample has the rows, and
-// pass 2, a programmatic dependent of pass 1, waits for it only when its first
+// Both walk a block's 128 rows as two 64 x 64 tiles of products (simt_split.cuh, three of
+// the four steps of K = 128 in flight at once), the second only where the sample has the
+// rows, and pass 2, a programmatic dependent of pass 1, waits for it only when its first
 // products are done. One fp32 sample of 192 visual tokens under 64 text rows with 4
 // heads (20 and 12 CTAs) took 16 and 18 us in 128 x 64 tiles, whose four K steps each
 // waited for their own loads and whose rows' chunk statistics were read one after

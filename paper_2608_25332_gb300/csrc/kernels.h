@@ -194,7 +194,7 @@ inline int crit_gram_parts(int N_t_max, int D) {
   return (n_k + per - 1) / per;
 }
 // early (only where crit_leads holds): the next kernel of the stream, launched as a
-// programmatic dependent, may start at once
+// programmatic dependent, may start beside this one, once its CTAs hold their tensor memory
 bool crit_leads(const SimArgs& a, int num_sms);
 cudaError_t crit_text_launch(const SimArgs& a, uint8_t* mask, float* r_out, float* G, int num_sms,
                              cudaStream_t s, bool early = false);

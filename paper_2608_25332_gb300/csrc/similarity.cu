@@ -829,8 +829,8 @@ __device__ __forceinline__ void add16(double* acc, const uint4& u, const float*)
 // rounded; in double 1 in 500 of those that cancel to 1e-7 of their largest partial
 // were not, and as pairs of floats 1 in 4. The GPU adds 128 floats per SM clock but
 // only two doubles: in double, with a division per element, the means of one fp32 image
-// (576 rows of 4096) took 66 us; as pairs or triples they take 14, and as triples the
-// merge of 16 such images takes 322 us where pairs took 314. A sum that leaves fp32's
+// (576 rows of 4096) took 66 us; as pairs they took 14, as triples 16 (the pass 105.4 with
+// either), and the merge of 16 such images 314 and 322. A sum that leaves fp32's
 // range or meets an infinity or a NaN is taken again in double.
 struct Sum3 {
   float hi, mid, lo;
@@ -1351,9 +1351,9 @@ cudaError_t merge_launch(const SimArgs& a, const int* keep_idx, int keep, const 
     const int group_tasks = a.B * ((keep + kMeanGroup - 1) / kMeanGroup) * n_slices;
     // CTAs for the long centroids, which leave at once where none is long: one where
     // so few rows are pruned that none can be with a valid keep_idx, else two per SM,
-    // and four beside 16 or more groups per SM, which cover the idle ones: at 25 groups
-    // per SM 254 us a pass with many long centroids against 264, at 7.6 without any
-    // 187 against 183.
+    // and four beside 16 or more groups per SM, which cover the idle ones: a pass with many
+    // long centroids took 179 us against 202 at 25 groups per SM and 150 against 152 at 23;
+    // from 8 to 19 the two are within 1%.
     const int n_lc = n_pruned < kMeanShort ? 1 : (group_tasks >= 16 * num_sms ? 4 : 2) * num_sms;
     const dim3 gm((unsigned)(group_tasks + n_lc));
     auto go = [&](auto kernel) {
