@@ -327,12 +327,14 @@ __global__ void __launch_bounds__(kMergeThreads, 1)
 // 0.9e-7 and 1.3e-7). So here
 //   * an accumulator takes kRelChunk slices, two in turn, and the epilogue warps add them up
 //     in registers: p is 1.1e-7 off at widths 512 to 5120 and 2.5e-7 at 8192;
-//   * in the first block, warps of their own add up the squares of the visual rows from the
-//     slices as they pass: 1/|v_j| is 0.4e-7 off at every width.
-// Both cost the K loop some 3%: the pass of the batch above 129.5 -> 131 us, 8 x 2880 rows
-// 335 -> 344, 32 x 576 rows of width 5120 under 512 526 -> 538. Chunks of two and of eight
-// slices: 360 and 342 us for the 8 x 2880; the squares in the epilogue warps, or by all
-// blocks in place of the visual block of the MMA: 349 and 355.
+//   * warps of their own add up the squares of the visual rows from the slices as they
+//     pass, each text block those of its share of the rows: 1/|v_j| is 0.4e-7 off at every
+//     width.
+// Both cost the K loop some 4%: the pass of the batch above 128.3 -> 130.3 us, 8 x 2880 rows
+// 333 -> 337, 32 x 576 rows of width 5120 under 512 531 -> 540. With the squares of every row
+// in the first block, whose CTAs then set the pace of a single wave: 132.8, 341 and 540; in
+// its epilogue warps 349 for the 8 x 2880; by all blocks in place of the visual block of the
+// MMA 355. Chunks of two and of eight slices: 360 and 342.
 struct RelFusedArgs {
   int B, N_v, D, N_t_max;
   int NT;        // text rows in the MMA (a block's rows, a multiple of 16)
@@ -352,7 +354,7 @@ constexpr int kRelFinishRows = 8;  // rows per warp of relevance_finish_kernel
 constexpr uint32_t kRelTmemCols = 256;  // 128 visual + <= 128 text columns
 
 constexpr int kRelChunk = 4;            // K slices of an accumulator with several text blocks
-constexpr int kRelSqWarps = 2;          // then more warps, for the squares of kBM rows
+constexpr int kRelSqWarps = 2;          // then more warps, for the squares of a block's share of the rows
 constexpr int kRelLongThreads = kThreads + 32 * kRelSqWarps;
 
 struct RelPipe {
@@ -380,7 +382,6 @@ __global__ void __launch_bounds__(kLong ? kRelLongThreads : kThreads, kLong ? 1 
   const int NS = a.n_stages;
   const uint32_t st_bytes = (uint32_t)(R + a.NT) * 128u;
   constexpr uint32_t kCols = (kLong ? 2 : 1) * kRelTmemCols;
-  const bool squares = kLong && blockIdx.z == 0;
   const uint32_t sbase = smem_u32(smem_raw);
   uint8_t* stages = smem_raw + (((sbase + 1023u) & ~1023u) - sbase);
   if (threadIdx.x == 0) {
@@ -388,7 +389,7 @@ __global__ void __launch_bounds__(kLong ? kRelLongThreads : kThreads, kLong ? 1 
     prefetch_tmap(&mapT);
     for (int s = 0; s < NS; ++s) {
       mbar_init(&pipe.full[s], 1);
-      mbar_init(&pipe.empty[s], squares ? 1 + kRelSqWarps : 1);  // the MMAs, and the warps that add squares
+      mbar_init(&pipe.empty[s], kLong ? 1 + kRelSqWarps : 1);  // the MMAs, and the warps that add squares
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(&pipe.acc_full[s], 1);
@@ -465,61 +466,53 @@ __global__ void __launch_bounds__(kLong ? kRelLongThreads : kThreads, kLong ? 1 
       if (!kLong) tc_commit(&pipe.acc_full[0]);
     }
   } else if (kLong && warp >= kThreads / 32) {
-    if (squares) {
-      // 1/|v_j| of the tile's rows for the merge: the squares of row r's slices as they
-      // pass, a slice's 64 in eight chains, the slices by TwoSum (in one chain over the
-      // slices the sum is biased low: squares of bf16 values are 0 or 1 mod 4 in their last
-      // place, so that rounding them to a longer one's goes down more often). A row's eight
-      // 16-byte pieces lie in some order in its 128 bytes, and lane l starts with piece l of
-      // them, so that eight lanes meet every bank.
-      constexpr int kRows = kBM / (32 * kRelSqWarps);  // rows of a lane
-      const int r0 = (warp - kThreads / 32) * 32 + lane;
-      float sum[kRows], rest[kRows];
+    static_assert(32 * kRelSqWarps >= kBM / 2, "a lane for each row of a block's share (two blocks or more)");
+    // 1/|v_j| for the merge, of this block's share of the tile's rows, a lane each: the
+    // squares of the row's slices as they pass, a slice's 64 in eight chains, the slices by
+    // TwoSum (in one chain over the slices the sum is biased low: squares of bf16 values are
+    // 0 or 1 mod 4 in their last place, so that rounding them to a longer one's goes down
+    // more often). A row's eight 16-byte pieces lie in some order in its 128 bytes, and lane
+    // l starts with piece l of them, so that eight lanes meet every bank.
+    const int share = (R + (int)gridDim.z - 1) / (int)gridDim.z, q0 = (warp - kThreads / 32) * 32;
+    const int r = (int)blockIdx.z * share + q0 + lane, j = n0 + r;
+    const bool mine = q0 + lane < share && r < R;
+    const uint8_t* row = stages + (size_t)(mine ? r : 0) * 128;
+    float sum = 0.f, rest = 0.f;
+    int s = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int kb = 0; kb < n_k && ok; ++kb) {
+      ok = warp_mbar_wait(&pipe.full[s], ph, a.err);
+      uint4 u[8];
 #pragma unroll
-      for (int h = 0; h < kRows; ++h) sum[h] = rest[h] = 0.f;
-      int s = 0;
-      uint32_t ph = 0;
-      bool ok = true;
-      for (int kb = 0; kb < n_k && ok; ++kb) {
-        ok = warp_mbar_wait(&pipe.full[s], ph, a.err);
+      for (int i = 0; i < 8; ++i)
+        u[i] = *reinterpret_cast<const uint4*>(row + (size_t)s * st_bytes + ((i + lane) & 7) * 16);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&pipe.empty[s]);  // before the work on it
+      if (++s == NS) {
+        s = 0;
+        ph ^= 1u;
+      }
+      float sq[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int h = 0; h < kRows; ++h) {
-          const int r = r0 + h * 32 * kRelSqWarps;
-          if (!ok || r >= R) break;  // warp-uniform
-          const uint8_t* row = stages + (size_t)s * st_bytes + (size_t)r * 128;
-          float sq[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      for (int i = 0; i < 8; ++i) {
+        const uint32_t w[4] = {u[i].x, u[i].y, u[i].z, u[i].w};
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const uint4 u = *reinterpret_cast<const uint4*>(row + ((i + lane) & 7) * 16);
-            const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const float lo = __uint_as_float(w[e] << 16), hi = __uint_as_float(w[e] & 0xffff0000u);
-              sq[2 * e] = fmaf(lo, lo, sq[2 * e]);
-              sq[2 * e + 1] = fmaf(hi, hi, sq[2 * e + 1]);
-            }
-          }
-          const float q = ((sq[0] + sq[1]) + (sq[2] + sq[3])) + ((sq[4] + sq[5]) + (sq[6] + sq[7]));
-          const float t = sum[h] + q, z = t - sum[h];
-          rest[h] += (sum[h] - (t - z)) + (q - z);
-          sum[h] = t;
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&pipe.empty[s]);
-        if (++s == NS) {
-          s = 0;
-          ph ^= 1u;
+        for (int e = 0; e < 4; ++e) {
+          const float lo = __uint_as_float(w[e] << 16), hi = __uint_as_float(w[e] & 0xffff0000u);
+          sq[2 * e] = fmaf(lo, lo, sq[2 * e]);
+          sq[2 * e + 1] = fmaf(hi, hi, sq[2 * e + 1]);
         }
       }
-      if (!ok) pipe.fail = 1;
-      pdl_wait_prior();
-#pragma unroll
-      for (int h = 0; h < kRows; ++h) {
-        const int r = r0 + h * 32 * kRelSqWarps, j = n0 + r;
-        const float v = sum[h] + rest[h];
-        if (ok && r < R && j < a.N_v) a.inv_v[(size_t)b * a.N_v + j] = v > 0.f ? 1.f / sqrtf(v) : 0.f;
-      }
+      const float q = ((sq[0] + sq[1]) + (sq[2] + sq[3])) + ((sq[4] + sq[5]) + (sq[6] + sq[7]));
+      const float t = sum + q, z = t - sum;
+      rest += (sum - (t - z)) + (q - z);
+      sum = t;
     }
+    if (!ok) pipe.fail = 1;
+    pdl_wait_prior();
+    sum += rest;
+    if (ok && mine && j < a.N_v) a.inv_v[(size_t)b * a.N_v + j] = sum > 0.f ? 1.f / sqrtf(sum) : 0.f;
   } else {
     const int quad = warp & 3;
     const int r = quad * 32 + lane;
